@@ -623,8 +623,9 @@ def timed_decode_steps(run, w, inputs, warmup: int, steps: int, world: int = 1, 
             "peak": peak, "peak_kind": peak_kind, "plan": plan, "clocks": clk}
 
 
-PLAN_NAMES = ["stream-K", "warp per segment (wide)", "warp per segment (narrow)", "whole segments, several per warp",
-              "whole segments cut by rows"]
+PLAN_NAMES = ["one unbalanced layer: CTA or cluster per segment, or stream-K", "CTA or cluster per segment, or several per CTA",
+              "warp per segment", "whole segments, several per warp",
+              "unbalanced layers: CTA per segment, or whole segments per warp cut by rows"]
 
 
 def plan_record(plan, launches_per_step: float):
@@ -720,7 +721,7 @@ def run_kvc(args, w):
             "roofline": {"bound": "hbm", "achieved": r["achieved"], "peak": r["peak"], "unit": "GB/s",
                          "frac": r["achieved"] / r["peak"], "frac_of_8tbs": r["achieved"] / 8000.0,
                          "peak_kind": r["peak_kind"],
-                         "kernel": "decode_kernel (single-query attention over the kept rows: whole segments per warp, or split-K with a log-sum-exp combine)",
+                         "kernel": "decode_cta_kernel / decode_kernel (single-query attention over the kept rows: whole segments per CTA, cluster or warp, or split-K, with a log-sum-exp combine)",
                          "traffic": recorded_traffic(w.name, r["bytes"] / n_launch),
                          "bytes_per_launch_mean": r["bytes"] / n_launch,
                          "launch_us_mean": r["dec_total_s"] / n_launch * 1e6},

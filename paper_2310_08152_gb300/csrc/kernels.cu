@@ -11,6 +11,8 @@
 //                         fp32 dot products, warp-shuffle reductions and an online softmax; the
 //                         parts of a split (sequence, head) are merged by a log-sum-exp combine done
 //                         by the last worker to finish (arrival counter).
+//   decode_cta_kernel     the same for launches of few segments: a CTA or a cluster of CTAs per segment,
+//                         merged in (distributed) shared memory
 //
 // No tensor cores: one query per (sequence, head) makes decode a GEMV (1 flop per byte read), far
 // below any tensor-core ridge; the kernels are bound by HBM bandwidth.
@@ -19,6 +21,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <mutex>
@@ -458,17 +461,9 @@ struct Lanes {
   static_assert(D % 16 == 0 && CH % LPR == 0, "unsupported d_head");
 };
 
-// Shapes of the per-warp pipeline (rows per lane per tile x stages).  Whole segments want the
-// largest in-flight window at three resident warps per SM, in as few tiles as possible (each tile
-// costs a fixed share of a warp's issue): 8x2 (128-row tiles, 64 KB per warp) at d=64, 6x2 (96-row
-// tiles, 60 KB) at d=80, 4x3 otherwise; measured on the full-size workloads against 4x3, 4x4 and
-// 6x3.  The narrow 2x3 shape fits the most warps when one warp per segment needs them.  Stream-K
-// runs a full wave of warps: 2x2 fits the most warps per SM.
-template <int D>
-struct WideShape {
-  static constexpr int KPT = D == 64 ? 8 : D == 80 ? 6 : 4;
-  static constexpr int S = (D == 64 || D == 80) ? 2 : 3;
-};
+// Shapes of the per-warp pipeline (rows per lane per tile x stages).  Whole segments, which take this
+// kernel when they are many and short, go to the narrow 2x3 shape (seven or eight warps per SM);
+// stream-K runs a full wave of warps: 2x2 fits the most warps per SM.
 #ifndef KVC_DEC_SEG2_KPT
 #define KVC_DEC_SEG2_KPT 2
 #endif
@@ -975,36 +970,470 @@ __global__ void __launch_bounds__(32, 1) decode_kernel(Geometry g, Static st, De
 }
 
 // ---------------------------------------------------------------------------------------------
-// dispatch
+// Decode with a CTA, or a cluster of CTAs, per segment
 // ---------------------------------------------------------------------------------------------
-// Resident CTAs per SM of one kernel instance, per device (the shared-memory attribute is set on
-// each device the first time the instance runs there).
-template <typename T, int D, int KPT, int S>
-cudaError_t decode_occupancy(int* occ_out) {
-  using C = DecodeCfg<D, KPT, S>;
-  static std::mutex mu;
-  static int occ[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lock(mu);
-  if (occ[dev] == 0) {
-    e = cudaFuncSetAttribute(decode_kernel<T, D, KPT, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    if (e != cudaSuccess) return e;
-    int o = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, decode_kernel<T, D, KPT, S>, C::THREADS, C::SMEM);
-    if (e != cudaSuccess) return e;
-    occ[dev] = o < 1 ? 1 : o;
-  }
-  *occ_out = occ[dev];
-  return cudaSuccess;
+// One layer of a small or ordinary batch has few segments (batch x heads): a warp per segment leaves
+// most of the machine idle, and splitting the rows over every warp pays ~5 us a launch for partial
+// results, fences and counters in global memory.  Here W consumer warps share every tile of a segment
+// and a producer warp streams the tiles (two bulk copies each) through S stages; a segment's rows are
+// cut over the CN CTAs of a cluster when there are too few segments for the SMs.  The warps' results
+// are merged in shared memory and the CTAs' in rank 0's (distributed shared memory), so nothing is
+// written to global memory but the output.  Two CTAs fit on an SM, so the next layer's launch
+// (programmatic dependent launch) fills its stages while this one finishes.
+//
+// What bounds it: HBM, from about 500 segments of 1,000 rows up; below that the fixed chain of a launch
+// (wait for the previous grid, query, first tile, merges, ~3.5 us).  Measured per layer at d_head 64,
+// 992 kept rows, one launch per layer (before, a warp per segment or rows split over all warps -> now;
+// time of the bytes at 7.2 TB/s): 32 segments 13.3 -> 4.8 us (1.1), 128 13.7 -> 7.8 (4.5),
+// 256 14.8 -> 11.7 (9.0), 512 30.1 -> 20.6 (18.1), 768 32.1 -> 30.0 (27.1); 1,536 ragged segments of up
+// to ~4,000 rows 132.7 -> 117.4 (116.7); 112 windows of 1,501 rows at d_head 128 49.2 -> 16.3 (12.0).
+// Several layers in one launch, per layer (before: runs of whole segments per warp, or a launch each):
+// 8 x 2,048 segments of 992 rows 71.9 -> 69.2 (72.3); 12 x 1,536 ragged 117.4 -> 110.0 (116.7),
+// 12 x 512 of up to ~1,000 rows 23.5 -> 13.3 (13.1), 4 x 1,024 of up to ~1,500 42.2 -> 31.5 (30.5).
+//
+// Shapes (consumer warps x rows per lane x stages).  Main: 4 x 2 x 3, two CTAs per SM (2 stages at
+// d_head 80, whose third would leave one CTA).  One row per lane (7 x 1 x 3) was 7 % slower, the fixed
+// work of a tile then weighs twice; 4 x 3 x 2 and 2 x 4 x 3 lost 4-17 %.  Small: 2 x 2 x 3, three or four
+// CTAs per SM, for counts between one wave of the main shape and one of this (512 segments of
+// 140 rows: 6.1 us against 7.6, of 992 rows 20.6 against 20.9).
+template <int D, int W_, int KPT_, int S_>
+struct CtaCfg {
+  using L = Lanes<D>;
+  static constexpr int W = W_, KPT = KPT_, S = S_;
+  static constexpr int WR = KPT * L::RPI;                 // rows per warp per tile
+  static constexpr int TR = W * WR;                       // rows per tile
+  static constexpr int TILE = TR * L::RB;                 // bytes per K (or V) tile
+  static constexpr int THREADS = (W + 1) * 32;
+  static constexpr int PO = D + 4;                        // floats of one partial result: M, L, -, -, O[D]
+  static constexpr int OFF_Z = 2 * S * TILE;              // a row of zeros
+  static constexpr int OFF_Q = OFF_Z + L::RB;             // [W][D] floats
+  static constexpr int OFF_O = OFF_Q + W * D * 4;         // [2][W][PO] floats: the warps' results, by piece parity
+  static constexpr int OFF_C = OFF_O + 2 * W * PO * 4;    // [8][PO] floats: the cluster's results, in rank 0
+  static constexpr int OFF_B = OFF_C + 8 * PO * 4;
+  static constexpr int SMEM = OFF_B + 2 * S * 8;
+  // resident CTAs per SM that the registers are cut for, as the shared memory (1 KB of it reserved
+  // per CTA) allows
+  static constexpr int FIT = 228 * 1024 / (SMEM + 1024);
+  static constexpr int CPS = FIT < 1 ? 1 : FIT > 4 ? 4 : FIT;
+  static_assert(OFF_Q % 16 == 0 && OFF_O % 16 == 0 && OFF_C % 16 == 0 && OFF_B % 8 == 0, "alignment");
+  static_assert(2 * KPT * L::RPI * L::RB >= L::RPI * D * 4, "the warp's rows of a stage hold its row groups' outputs");
+};
+
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void mbar_arrive1(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void st_cluster_f32(const void* p, uint32_t rank, float v) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
 }
 
-template <typename T, int D, int KPT, int S>
-cudaError_t launch_decode_cfg(const Geometry& g, const Static& st, const Buffers& buf, const DecodeArgs& a,
-                              int64_t NW, int seg_per_worker, cudaStream_t stream, int* grid) {
-  using C = DecodeCfg<D, KPT, S>;
+constexpr int kMaxClusterCtas = 8;  // the portable cluster size
+
+// One piece of a CTA's work: rows [r0, r1) of segment (layer, s, h).
+struct Piece {
+  int s, h, layer, r0, r1;
+};
+
+// CTAs [u CN, (u + 1) CN) -- a cluster when CN > 1 -- take segments [u k_segs, (u + 1) k_segs) of the
+// launch's (layer, sequence, head) segments whole; CN > 1 goes with k_segs = 1.
+template <typename T, int D, int W, int KPT, int S>
+__global__ void __launch_bounds__((W + 1) * 32, CtaCfg<D, W, KPT, S>::CPS)
+    decode_cta_kernel(Geometry g, Static st, DecodeDev p, int CN, int k_segs) {
+  using C = CtaCfg<D, W, KPT, S>;
+  using L = Lanes<D>;
+  extern __shared__ __align__(128) unsigned char smem[];
+  pdl_launch_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = CN > 1 ? (int)(blockIdx.x % (unsigned)CN) : 0;  // == the cluster rank (1-D clusters of CN)
+  const int unit = CN > 1 ? (int)(blockIdx.x / (unsigned)CN) : (int)blockIdx.x;
+  const int H = g.H;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::OFF_B);
+  uint64_t* empty = full + S;
+  float* sO = reinterpret_cast<float*>(smem + C::OFF_O);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      mbar_init(&full[i], 1);
+      mbar_init(&empty[i], W);
+    }
+    fence_mbar_init();
+  }
+  if (threadIdx.x >= 32 && threadIdx.x < 32 + L::RB / 16)
+    reinterpret_cast<uint4*>(smem + C::OFF_Z)[threadIdx.x - 32] = make_uint4(0, 0, 0, 0);
+  if (CN > 1) cluster_arrive();
+  __syncthreads();
+  // segments [sg, sg1), each cut over the cluster's CTAs
+  int64_t sg = (int64_t)unit * k_segs;
+  const int64_t sg1 = min(sg + k_segs, (int64_t)p.n_layers * g.b * H);
+  Piece pc;
+  {
+    const int64_t segs_layer = (int64_t)g.b * H;
+    pc.layer = (int)(sg / segs_layer);
+    const int w = (int)(sg - (int64_t)pc.layer * segs_layer);
+    pc.s = w / H;
+    pc.h = w - pc.s * H;
+  }
+  int Lc = 0, ps = -1;
+  auto set_rows = [&]() {  // the CTA's rows of the current segment
+    if (ps != pc.s) {
+      ps = pc.s;
+      Lc = (int)(p.P[ps + 1] - p.P[ps]);
+    }
+    pc.r0 = 0;
+    pc.r1 = Lc;
+    if (CN > 1) {
+      const int step = (Lc + CN - 1) / CN;
+      pc.r0 = min(rank * step, Lc);
+      pc.r1 = min(pc.r0 + step, Lc);
+    }
+  };
+  auto next = [&]() {
+    ++sg;
+    if (++pc.h == H) {
+      pc.h = 0;
+      if (++pc.s == g.b) {
+        pc.s = 0;
+        ++pc.layer;
+      }
+    }
+  };
+  int stage = 0, phase = 0;
+
+  if (warp == W) {
+    if (lane == 0) {
+      int seg_s = -1;
+      int64_t seg_row0 = 0;
+      int seg_begin = 0, seg_wrap = 0, seg_cap = 0;
+      if (!p.kv_before_wait) pdl_wait();
+      int t = 0;
+      bool ok = true;
+      for (; ok && sg < sg1; next()) {
+        set_rows();
+        if (pc.r0 >= pc.r1) continue;
+        if (pc.s != seg_s) {
+          seg_s = pc.s;
+          seg_row0 = st.seq_row0[seg_s];
+          seg_begin = p.ds[seg_s].begin;
+          seg_wrap = p.ds[seg_s].wrap;
+          seg_cap = st.cap[seg_s];
+        }
+        const int64_t base = (int64_t)pc.layer * p.plane + (seg_row0 + (int64_t)pc.h * seg_cap) * D;
+        for (int r = pc.r0; r < pc.r1;) {
+          int n = min(C::TR, pc.r1 - r);
+          if (r < seg_wrap) n = min(n, seg_wrap - r);
+          if (t >= S && !mbar_wait_bounded(&empty[stage], phase ^ 1, p.limit_ns)) {
+            atomicOr(p.status, STATUS_TIMEOUT);
+            ok = false;
+            break;
+          }
+          const int slot = r < seg_wrap ? seg_begin + r : r - seg_wrap;
+          const uint32_t bytes = (uint32_t)n * L::RB;
+          mbar_arrive_expect_tx(&full[stage], 2 * bytes);
+          const int64_t e0 = base + (int64_t)slot * D;
+          unsigned char* dst = smem + stage * 2 * C::TILE;
+          bulk_g2s(dst, p.k + e0, bytes, &full[stage]);
+          bulk_g2s(dst + C::TILE, p.v + e0, bytes, &full[stage]);
+          r += n;
+          ++t;
+          if (++stage == S) {
+            stage = 0;
+            phase ^= 1;
+          }
+        }
+      }
+      if (p.kv_before_wait) pdl_wait();
+      // never leave with copies in flight
+      for (int u = t > S ? t - S : 0; u < t; ++u) (void)mbar_wait_bounded(&full[u % S], (u / S) & 1, p.limit_ns);
+    }
+    return;
+  }
+
+  float* qs = reinterpret_cast<float*>(smem + C::OFF_Q) + warp * D;
+  constexpr int QPL = (D + 31) / 32;
+  uint32_t qraw[QPL];  // element and rotation partner, 16 bits each
+  auto fetch_q = [&]() {
+    const uint16_t* qrow = p.q + (int64_t)pc.layer * p.q_stride + ((int64_t)pc.s * H + pc.h) * D;
+    const int half = g.rot / 2;
+#pragma unroll
+    for (int j = 0; j < QPL; ++j) {
+      const int c = lane + 32 * j;
+      qraw[j] = 0;
+      if (c < D) {
+        qraw[j] = qrow[c];
+        if (c < g.rot) qraw[j] |= (uint32_t)qrow[c < half ? c + half : c - half] << 16;
+      }
+    }
+  };
+  const int grp = lane / L::LPR;
+  const int tl = lane % L::LPR;
+  const int rot = (L::A * grp + L::B * tl) % L::NV;
+  float2 qv[L::EPL / 2], o[L::EPL / 2];
+  int mlo = 0, mhi = 0, wrap = 0;  // hidden rows of the sequence, counted from its first attended row; ring end
+  int32_t qpos = 0;
+  int cur_s = -1;
+  bool dead = false;
+  int piece = 0;
+  const int jw = warp * C::WR;  // the warp's first row of every tile
+  pdl_wait();
+  fetch_q();
+  for (; sg < sg1;) {
+    set_rows();
+    const int s = pc.s, h = pc.h, layer = pc.layer, r1 = pc.r1;
+    if (Lc == 0) {  // a sequence without rows
+      next();
+      if (sg < sg1) fetch_q();
+      continue;
+    }
+    if (s != cur_s) {
+      cur_s = s;
+      const DState d = p.ds[s];
+      mlo = d.mask_lo - d.begin;
+      mhi = d.mask_hi - d.begin;
+      wrap = d.wrap;
+      qpos = d.qpos;
+    }
+    {
+      const int half = g.rot / 2;
+#pragma unroll
+      for (int j = 0; j < QPL; ++j) {
+        const int c = lane + 32 * j;
+        if (c < D) {
+          float x = T::f1((uint16_t)qraw[j]);
+          if (c < g.rot) {
+            const bool lo_half = c < half;
+            float sn, cs;
+            rope_sincos(qpos, st.rope_g[lo_half ? c : c - half], &sn, &cs);
+            const float y = T::f1((uint16_t)(qraw[j] >> 16));
+            x = lo_half ? x * cs - y * sn : x * cs + y * sn;
+          }
+          qs[c] = x * p.qscale;
+        }
+      }
+    }
+    int r = pc.r0;
+    next();
+    if (sg < sg1) fetch_q();  // the next segment's query, a whole piece ahead of its use
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < L::NV; ++i) {
+      const int c = tl * L::NV + (i + rot) % L::NV;
+      const float4 a = reinterpret_cast<const float4*>(qs + c * 8)[0];
+      const float4 b = reinterpret_cast<const float4*>(qs + c * 8)[1];
+      qv[i * 4 + 0] = make_float2(a.x, a.y);
+      qv[i * 4 + 1] = make_float2(a.z, a.w);
+      qv[i * 4 + 2] = make_float2(b.x, b.y);
+      qv[i * 4 + 3] = make_float2(b.z, b.w);
+    }
+#pragma unroll
+    for (int e = 0; e < L::EPL / 2; ++e) o[e] = make_float2(0.f, 0.f);
+    float m = -INFINITY, l = 0.f;
+    unsigned char* scratch = nullptr;  // the last tile's stage
+    int held = -1;
+    while (r < r1) {
+      int n = min(C::TR, r1 - r);
+      if (r < wrap) n = min(n, wrap - r);
+      if (!dead && !mbar_wait_bounded(&full[stage], phase, p.limit_ns)) {
+        dead = true;
+        if (lane == 0) atomicOr(p.status, STATUS_TIMEOUT);
+      }
+      unsigned char* kt = smem + stage * 2 * C::TILE;
+      if (!dead && jw < n) {
+        float z[KPT];
+        bool valid[KPT];
+#pragma unroll
+        for (int k = 0; k < KPT; ++k) {
+          const int j = jw + k * L::RPI + grp;
+          const int row = r + j;
+          valid[k] = j < n && (row < mlo || row >= mhi);
+          const unsigned char* kr = valid[k] ? kt + j * L::RB : smem + C::OFF_Z;
+          float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+#pragma unroll
+          for (int i = 0; i < L::NV; ++i) {
+            const int c = tl * L::NV + (i + rot) % L::NV;
+            const uint4 u = *reinterpret_cast<const uint4*>(kr + c * 16);
+            acc0 = ffma2(qv[i * 4 + 0], T::f2(u.x), acc0);
+            acc1 = ffma2(qv[i * 4 + 1], T::f2(u.y), acc1);
+            acc0 = ffma2(qv[i * 4 + 2], T::f2(u.z), acc0);
+            acc1 = ffma2(qv[i * 4 + 3], T::f2(u.w), acc1);
+          }
+          z[k] = (acc0.x + acc1.x) + (acc0.y + acc1.y);
+        }
+#pragma unroll
+        for (int off = L::LPR / 2; off >= 1; off >>= 1)
+#pragma unroll
+          for (int k = 0; k < KPT; ++k) z[k] += __shfl_xor_sync(kFull, z[k], off);
+        float mn = m;
+#pragma unroll
+        for (int k = 0; k < KPT; ++k) {
+          if (!valid[k]) z[k] = -INFINITY;
+          mn = fmaxf(mn, z[k]);
+        }
+        const float mu = (mn == -INFINITY) ? 0.f : mn;
+        const float alpha = exp2f(m - mu);
+        l *= alpha;
+        const float2 a2 = make_float2(alpha, alpha);
+#pragma unroll
+        for (int e = 0; e < L::EPL / 2; ++e) o[e] = fmul2(o[e], a2);
+#pragma unroll
+        for (int k = 0; k < KPT; ++k) {
+          const int j = jw + k * L::RPI + grp;
+          const float pk = exp2f(z[k] - mu);
+          l += pk;
+          const float2 p2 = make_float2(pk, pk);
+          const unsigned char* vr = valid[k] ? kt + C::TILE + j * L::RB : smem + C::OFF_Z;
+#pragma unroll
+          for (int i = 0; i < L::NV; ++i) {
+            const int c = tl * L::NV + (i + rot) % L::NV;
+            const uint4 u = *reinterpret_cast<const uint4*>(vr + c * 16);
+            o[i * 4 + 0] = ffma2(p2, T::f2(u.x), o[i * 4 + 0]);
+            o[i * 4 + 1] = ffma2(p2, T::f2(u.y), o[i * 4 + 1]);
+            o[i * 4 + 2] = ffma2(p2, T::f2(u.z), o[i * 4 + 2]);
+            o[i * 4 + 3] = ffma2(p2, T::f2(u.w), o[i * 4 + 3]);
+          }
+        }
+        m = mn;
+      }
+      __syncwarp();  // every lane has read the warp's rows of the tile
+      r += n;
+      if (r < r1) {
+        if (lane == 0) mbar_arrive1(&empty[stage]);
+      } else {
+        scratch = kt;  // the piece's last stage: released after the merge
+        held = stage;
+      }
+      if (++stage == S) {
+        stage = 0;
+        phase ^= 1;
+      }
+    }
+    // ------------------------- piece end: merge the row groups, the warps, the cluster ------------
+    float M = m;
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, off));
+    const float Mu = (M == -INFINITY) ? 0.f : M;
+    const float e = exp2f(m - Mu);
+    float* so = sO + ((piece & 1) * W + warp) * C::PO;
+    if (scratch != nullptr) {
+      float Ls = l * e;
+#pragma unroll
+      for (int off = 16; off >= 1; off >>= 1) Ls += __shfl_xor_sync(kFull, Ls, off);
+      Ls *= 1.0f / (float)L::LPR;
+      // the warp's own rows of the stage hold its row groups' outputs
+      auto red = [&](int q) {
+        constexpr int half = KPT > 1 ? L::RPI : L::RPI / 2;  // groups over the K rows; the rest over the V rows
+        return reinterpret_cast<float*>(scratch + (q < half ? 0 : C::TILE) + jw * L::RB) + (q % half) * D;
+      };
+      const float2 e2 = make_float2(e, e);
+      float* mine = red(grp);
+#pragma unroll
+      for (int i = 0; i < L::NV; ++i) {
+        const int c = tl * L::NV + (i + rot) % L::NV;
+        float4* dst = reinterpret_cast<float4*>(mine + c * 8);
+        const float2 x0 = fmul2(o[i * 4 + 0], e2), x1 = fmul2(o[i * 4 + 1], e2);
+        const float2 x2 = fmul2(o[i * 4 + 2], e2), x3 = fmul2(o[i * 4 + 3], e2);
+        dst[0] = make_float4(x0.x, x0.y, x1.x, x1.y);
+        dst[1] = make_float4(x2.x, x2.y, x3.x, x3.y);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < QPL; ++j) {
+        const int col = lane + 32 * j;
+        if (col < D) {
+          float O0 = 0.f, O1 = 0.f;
+#pragma unroll
+          for (int q = 0; q < L::RPI; q += 2) {
+            O0 += red(q)[col];
+            O1 += red(q + 1)[col];
+          }
+          so[4 + col] = O0 + O1;
+        }
+      }
+      if (lane == 0) {
+        so[0] = M;
+        so[1] = Ls;
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive1(&empty[held]);
+    } else {  // no rows of the segment in this CTA
+      for (int col = lane; col < D; col += 32) so[4 + col] = 0.f;
+      if (lane == 0) {
+        so[0] = -INFINITY;
+        so[1] = 0.f;
+      }
+    }
+    bar_sync(1, W * 32);
+    const bool mine_to_merge = warp == piece % W;
+    const int seg = s * H + h;
+    float* orow = p.out + (int64_t)layer * p.out_stride + (int64_t)seg * D;
+    // merges n results of PO floats; lane writes its columns scaled by 1 / L, or to the cluster's rank 0
+    auto merge = [&](const float* sp, int n, bool last) {
+      float Mx = -INFINITY;
+      for (int w = 0; w < n; ++w) Mx = fmaxf(Mx, sp[w * C::PO]);
+      const float Mxu = (Mx == -INFINITY) ? 0.f : Mx;
+      float Lx = 0.f, O[QPL];
+#pragma unroll
+      for (int j = 0; j < QPL; ++j) O[j] = 0.f;
+#pragma unroll 4
+      for (int w = 0; w < n; ++w) {
+        const float ew = exp2f(sp[w * C::PO] - Mxu);
+        Lx += sp[w * C::PO + 1] * ew;
+#pragma unroll
+        for (int j = 0; j < QPL; ++j)
+          if (lane + 32 * j < D) O[j] += sp[w * C::PO + 4 + lane + 32 * j] * ew;
+      }
+      if (last) {
+        const float inv = 1.f / Lx;
+#pragma unroll
+        for (int j = 0; j < QPL; ++j)
+          if (lane + 32 * j < D) orow[lane + 32 * j] = O[j] * inv;
+      } else {
+        float* dst = reinterpret_cast<float*>(smem + C::OFF_C) + rank * C::PO;
+#pragma unroll
+        for (int j = 0; j < QPL; ++j)
+          if (lane + 32 * j < D) st_cluster_f32(dst + 4 + lane + 32 * j, 0, O[j]);
+        if (lane == 0) {
+          st_cluster_f32(dst, 0, Mx);
+          st_cluster_f32(dst + 1, 0, Lx);
+        }
+      }
+    };
+    if (CN > 1) {
+      cluster_wait();  // every CTA of the cluster has started
+      if (mine_to_merge) merge(sO + (piece & 1) * W * C::PO, W, false);
+      cluster_arrive();
+      if (rank == 0) {
+        cluster_wait();
+        if (mine_to_merge && !dead) merge(reinterpret_cast<const float*>(smem + C::OFF_C), CN, true);
+      }
+      return;  // one segment per cluster
+    }
+    if (mine_to_merge && !dead) merge(sO + (piece & 1) * W * C::PO, W, true);
+    ++piece;
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// dispatch
+// ---------------------------------------------------------------------------------------------
+// Resident CTAs per SM of one kernel instance on the current device, whose shared-memory attribute is
+// set here.
+template <typename K>
+cudaError_t kernel_occupancy(K kernel, int threads, int smem, int* occ_out) {
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  int o = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kernel, threads, smem);
+  *occ_out = o < 1 ? 1 : o;
+  return e;
+}
+
+inline DecodeDev decode_dev(const Geometry& g, const Buffers& buf, const DecodeArgs& a, int D, int64_t NW,
+                            int seg_per_worker) {
   DecodeDev p;
   const int64_t plane = (int64_t)g.H * g.C * D;
   p.k = buf.k + (int64_t)a.layer * plane;
@@ -1026,6 +1455,14 @@ cudaError_t launch_decode_cfg(const Geometry& g, const Static& st, const Buffers
   p.limit_ns = a.wait_limit_ns;
   p.kv_before_wait = a.kv_before_wait;
   p.seg_per_worker = seg_per_worker;
+  return p;
+}
+
+template <typename T, int D, int KPT, int S>
+cudaError_t launch_decode_cfg(const Geometry& g, const Static& st, const Buffers& buf, const DecodeArgs& a,
+                              int64_t NW, int seg_per_worker, cudaStream_t stream, int* grid) {
+  using C = DecodeCfg<D, KPT, S>;
+  const DecodeDev p = decode_dev(g, buf, a, D, NW, seg_per_worker);
   const int64_t ctas = (NW + C::WARPS - 1) / C::WARPS;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)ctas);
@@ -1041,16 +1478,30 @@ cudaError_t launch_decode_cfg(const Geometry& g, const Static& st, const Buffers
   return cudaLaunchKernelEx(&cfg, decode_kernel<T, D, KPT, S>, g, st, p);
 }
 
-// k whole segments per worker, k as small as one wave of `occ` warps per SM allows; `busiest` is
-// the segments on the SM with the most resident workers (workers spread evenly over the SMs).
-struct SegSplit {
-  int64_t k, workers, busiest;
-};
-inline SegSplit seg_split(int64_t nseg, int occ, int num_sms) {
-  const int64_t slots = (int64_t)(occ > 0 ? occ : 1) * num_sms;
-  const int64_t k = (nseg + slots - 1) / slots;
-  const int64_t workers = (nseg + k - 1) / k;
-  return {k, workers, (workers + num_sms - 1) / num_sms * k};
+template <typename T, int D, int W, int KPT, int S>
+cudaError_t launch_decode_cta(const Geometry& g, const Static& st, const Buffers& buf, const DecodeArgs& a, int CN,
+                              int64_t k_segs, int mode, cudaStream_t stream, int* grid, DecodePlan* plan) {
+  using C = CtaCfg<D, W, KPT, S>;
+  const DecodeDev p = decode_dev(g, buf, a, D, 0, 0);
+  const int64_t nseg = (int64_t)p.n_layers * g.b * g.H;
+  const int64_t ctas = (nseg + k_segs - 1) / k_segs * CN;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)ctas);
+  cfg.blockDim = dim3(C::THREADS);
+  cfg.dynamicSmemBytes = C::SMEM;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = CN;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = CN > 1 ? 2 : 1;
+  *plan = {mode, (int)(ctas * W), C::TR, S};
+  *grid = (int)ctas;
+  return cudaLaunchKernelEx(&cfg, decode_cta_kernel<T, D, W, KPT, S>, g, st, p, CN, (int)k_segs);
 }
 
 // Segments of the uploaded state are balanced: the longest holds at most 1.3x the mean rows.
@@ -1058,68 +1509,140 @@ inline bool decode_balanced(const DecodeArgs& a) {
   return a.n_segments > 0 && 10 * a.max_segment * a.n_segments <= 13 * a.R;
 }
 
+// Stages of decode_cta_kernel's main shape: three, or as many as leave room for two CTAs per SM.
+template <int D>
+struct CtaMainStages {
+  static constexpr int S = D == 80 ? 2 : 3;
+};
+
+// Whether and how the CTA kernel takes a launch of nseg segments: `cluster` CTAs per segment, or k
+// segments per CTA, of the main or the small shape.  slots_m / slots_s: CTAs of the main / small shape
+// that one wave holds.
+struct CtaPlan {
+  bool use, small;
+  int cluster;
+  int64_t k;
+};
+template <int D>
+CtaPlan decode_cta_plan(const DecodeArgs& a, int64_t nseg, bool balanced, int64_t slots_m, int64_t slots_s) {
+  constexpr CtaPlan kNo = {false, false, 1, 1};
+  const int n_layers = a.n_layers < 1 ? 1 : a.n_layers;
+  const int64_t mean = a.R / (a.n_segments < 1 ? 1 : a.n_segments);  // rows of a segment that has any
+  const int64_t share = n_layers * a.R / slots_m;                    // rows of a CTA in an even split
+  if (nseg <= slots_m) {
+    // unbalanced layers go one by one, each cut over clusters
+    if (!balanced && n_layers > 1) return kNo;
+    // Clusters while a wave holds them and each CTA keeps at least 1.5 tiles of the longest segment:
+    // 32 segments of 992 rows took 6.2 / 5.9 / 4.8 / 5.4 us with 1 / 2 / 4 / 8 CTAs each, of 3,968 rows
+    // 17.1 / 13.7 / 9.5 / 8.4; 128 of 290 rows 5.2 / 5.3; 192 of 992 rows, more than a wave, 10.2 / 13.7.
+    int cn = 1;
+    while (2 * cn <= kMaxClusterCtas && 2 * cn * nseg <= slots_m && a.max_segment >= 2 * cn * 192) cn *= 2;
+    // A few long segments among short ones: past about twice a CTA's even share, and 2,048 rows that
+    // a CTA streams in the ~9 us that splitting the rows over every warp costs, that split is the better
+    // balance (256 ragged segments, the longest 1.8 shares: 30.1 us here, 35.9 there).
+    if (!balanced && a.max_segment > 2 * cn * share + 2048) return kNo;
+    return {true, false, cn, 1};
+  }
+  // More than one wave.  A tile's and a segment's fixed work have to be small beside a segment's rows:
+  // a warp per segment, or several, is as good below these means and up to 40 % better at half of them
+  // (d_head 64, 65,536 segments: 243 rows 19.2 us a layer by warps, 20.3 here; 485 rows 20.6 and 19.0;
+  // 992 rows 71.9 and 69.2.  d_head 128: 170 rows 30.8 and 30.2).
+  constexpr int64_t kMeanRows = Lanes<D>::LPR == 4 ? 160 : 384;
+  if (balanced) {
+    if (nseg <= slots_s) return {true, true, 1, 1};
+    if (mean < kMeanRows) return kNo;
+    // up to eight segments per CTA where that makes one wave: 768 segments of 992 rows 30.0 us against
+    // 33.3 one by one, 2,048 75.2 against 77.1
+    const int64_t k = (nseg + slots_m - 1) / slots_m;
+    return {true, false, 1, k <= 8 ? k : 1};
+  }
+  if (a.max_segment > 6 * mean || a.max_segment > 2 * share + 2048) return kNo;  // as above: split the rows
+  // Unbalanced: the hardware hands the CTAs out as they finish, where a split of the rows over every warp
+  // pays for its partial results (6 layers of 8,192 segments: mean 210 rows 73.1 us a layer, split 109.5;
+  // 80 rows 42.7 and 69.0).  Short segments two to a CTA, of the small shape at d_head 64.
+  if (mean >= kMeanRows) return {true, false, 1, 1};
+  return {true, D == 64, 1, mean < 256 ? 2 : 1};
+}
+
+// Resident CTAs per SM of the decode kernels' instances on the current device: the CTA kernel's main and
+// small shape, the warp kernel's whole-segment and stream-K shape.  Found once per device.
+struct DecodeOcc {
+  int main, small, seg, stream;
+};
+template <typename T, int D>
+cudaError_t decode_occupancies(int dev, DecodeOcc* out) {
+  constexpr int BK = KVC_DEC_SEG2_KPT, BS = KVC_DEC_SEG2_STAGES, TK = KVC_DEC_STREAM_KPT, TS = KVC_DEC_STREAM_STAGES;
+  constexpr int MS = CtaMainStages<D>::S;
+  static std::atomic<uint32_t> found[64];  // eight bits each; 0: not yet
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  uint32_t v = found[dev].load(std::memory_order_acquire);
+  if (v == 0) {
+    int o[4];
+    using M = CtaCfg<D, 4, 2, MS>;
+    using S = CtaCfg<D, 2, 2, 3>;
+    using B = DecodeCfg<D, BK, BS>;
+    using K = DecodeCfg<D, TK, TS>;
+    cudaError_t e = kernel_occupancy(decode_cta_kernel<T, D, 4, 2, MS>, M::THREADS, M::SMEM, &o[0]);
+    if (e == cudaSuccess) e = kernel_occupancy(decode_cta_kernel<T, D, 2, 2, 3>, S::THREADS, S::SMEM, &o[1]);
+    if (e == cudaSuccess) e = kernel_occupancy(decode_kernel<T, D, BK, BS>, B::THREADS, B::SMEM, &o[2]);
+    if (e == cudaSuccess) e = kernel_occupancy(decode_kernel<T, D, TK, TS>, K::THREADS, K::SMEM, &o[3]);
+    if (e != cudaSuccess) return e;
+    v = (uint32_t)o[0] | (uint32_t)o[1] << 8 | (uint32_t)o[2] << 16 | (uint32_t)o[3] << 24;
+    found[dev].store(v, std::memory_order_release);
+  }
+  *out = {(int)(v & 255u), (int)(v >> 8 & 255u), (int)(v >> 16 & 255u), (int)(v >> 24)};
+  return cudaSuccess;
+}
+
 template <typename T, int D>
 cudaError_t launch_decode_t(const Geometry& g, const Static& st, const Buffers& buf, const DecodeArgs& a, int num_sms,
                             cudaStream_t stream, int* grid, DecodePlan* plan) {
-  constexpr int AK = WideShape<D>::KPT, AS = WideShape<D>::S;
   constexpr int BK = KVC_DEC_SEG2_KPT, BS = KVC_DEC_SEG2_STAGES;
   constexpr int TK = KVC_DEC_STREAM_KPT, TS = KVC_DEC_STREAM_STAGES;
-  // Balanced segments (longest within 1.3x of the mean) are never split, so no warp writes split-K
-  // partials or waits on a combine: one warp per (layer, sequence, head) segment when a wave of
-  // resident warps holds them all (the wide pipeline shape first), else k consecutive whole
-  // segments per warp.  Otherwise, over several layers whose segments are short beside a warp's
-  // share of the rows, whole segments cut by rows; else the rows are split evenly over a full wave
-  // (stream-K), one layer per launch.  Whole segments shorter on average than six wide tiles go to
-  // the narrow shape (more warps per SM, less fixed work per tile and per segment): on ragged caches
-  // the wide shape wins from a mean of about 1,000 kept rows, the narrow one below about 500.
+  // A CTA or a cluster per segment, or a few segments per CTA, unless the segments are many and short
+  // or a few of them far longer than the rest (decode_cta_plan).  Those: balanced segments (longest
+  // within 1.3x of the mean) one per warp while a wave of warps holds them all, else k consecutive
+  // whole segments per warp.  Unbalanced ones, over several layers whose segments are short beside a
+  // warp's share of the rows, as whole segments cut by rows; else the rows are split evenly over a full
+  // wave of warps (stream-K), one layer per launch.
   const int n_layers = a.n_layers < 1 ? 1 : a.n_layers;
   const int64_t nseg = (int64_t)n_layers * g.b * g.H;
-  const bool short_segs = a.n_segments > 0 && a.R < 6 * (int64_t)(AK * Lanes<D>::RPI) * a.n_segments;
   const bool balanced = decode_balanced(a);
-  if (balanced || n_layers > 1) {
-    cudaError_t e;
-    int occ_a = 0, occ_b = 0;
-    e = decode_occupancy<T, D, AK, AS>(&occ_a);
-    if (e == cudaSuccess) e = decode_occupancy<T, D, BK, BS>(&occ_b);
-    if (e != cudaSuccess) return e;
-    if (!balanced) {
-      // Unbalanced segments over several layers: a wave of warps takes whole segments cut by rows
-      // when the longest segment is at most 1/16 of a warp's even share (so no warp holds more than
-      // ~6 % above the mean); else the caller launches the layers one by one.
-      const int occ = short_segs ? occ_b : occ_a;
-      int64_t NW = (int64_t)occ * num_sms;
-      if (NW > nseg) NW = nseg;
-      if (NW < 1 || 16 * a.max_segment > (int64_t)n_layers * a.R / NW) return cudaErrorNotSupported;
-      if (short_segs) {
-        *plan = {4, (int)NW, BK * Lanes<D>::RPI, BS};
-        return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, NW, -1, stream, grid);
-      }
-      *plan = {4, (int)NW, AK * Lanes<D>::RPI, AS};
-      return launch_decode_cfg<T, D, AK, AS>(g, st, buf, a, NW, -1, stream, grid);
+  constexpr int MS = CtaMainStages<D>::S;
+  DecodeOcc occ;
+  const cudaError_t e = decode_occupancies<T, D>(a.device, &occ);
+  if (e != cudaSuccess) return e;
+  const CtaPlan c = decode_cta_plan<D>(a, nseg, balanced, (int64_t)occ.main * num_sms, (int64_t)occ.small * num_sms);
+  if (n_layers > 1 && !balanced && nseg > (int64_t)occ.main * num_sms) {
+    // Unbalanced segments over several layers, short ones: a wave of warps takes whole segments cut by
+    // rows when the longest segment is at most 1/16 of a warp's even share (so no warp holds more than
+    // ~6 % above the mean).
+    int64_t NW = (int64_t)occ.seg * num_sms;
+    if (NW > nseg) NW = nseg;
+    const bool long_segs = c.use && !c.small && c.k == 1;
+    if (!long_segs && NW >= 1 && 16 * a.max_segment <= (int64_t)n_layers * a.R / NW) {
+      *plan = {4, (int)NW, BK * Lanes<D>::RPI, BS};
+      return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, NW, -1, stream, grid);
     }
-    if (nseg <= (int64_t)occ_a * num_sms) {
-      *plan = {1, (int)nseg, AK * Lanes<D>::RPI, AS};
-      return launch_decode_cfg<T, D, AK, AS>(g, st, buf, a, nseg, 1, stream, grid);
-    }
-    if (nseg <= (int64_t)occ_b * num_sms) {
+  }
+  if (c.use) {
+    const int mode = balanced ? 1 : n_layers > 1 ? 4 : 0;
+    if (c.small) return launch_decode_cta<T, D, 2, 2, 3>(g, st, buf, a, c.cluster, c.k, mode, stream, grid, plan);
+    return launch_decode_cta<T, D, 4, 2, MS>(g, st, buf, a, c.cluster, c.k, mode, stream, grid, plan);
+  }
+  if (balanced) {
+    if (nseg <= (int64_t)occ.seg * num_sms) {
       *plan = {2, (int)nseg, BK * Lanes<D>::RPI, BS};
       return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, nseg, 1, stream, grid);
     }
-    // several whole segments per warp: the narrow shape for short segments, else the shape and k that
-    // put the fewest segments on the busiest SM
-    const SegSplit sa = seg_split(nseg, occ_a, num_sms), sb = seg_split(nseg, occ_b, num_sms);
-    if (!short_segs && sa.busiest <= sb.busiest) {
-      *plan = {3, (int)sa.workers, AK * Lanes<D>::RPI, AS};
-      return launch_decode_cfg<T, D, AK, AS>(g, st, buf, a, sa.workers, sa.k, stream, grid);
-    }
-    *plan = {3, (int)sb.workers, BK * Lanes<D>::RPI, BS};
-    return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, sb.workers, sb.k, stream, grid);
+    // k whole segments per warp, k as small as one wave of warps allows
+    const int64_t slots = (int64_t)occ.seg * num_sms;
+    const int64_t k = (nseg + slots - 1) / slots, workers = (nseg + k - 1) / k;
+    *plan = {3, (int)workers, BK * Lanes<D>::RPI, BS};
+    return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, workers, k, stream, grid);
   }
-  cudaError_t e;
-  int occ = 0;
-  e = decode_occupancy<T, D, TK, TS>(&occ);
-  if (e != cudaSuccess) return e;
-  int64_t NW = (int64_t)occ * num_sms;
+  if (n_layers > 1) return cudaErrorNotSupported;  // the caller launches the layers one by one
+  int64_t NW = (int64_t)occ.stream * num_sms;
   if (a.R < NW) NW = a.R;
   if (NW > kMaxDecodeWorkers) NW = kMaxDecodeWorkers;
   if (NW < 1) NW = 1;

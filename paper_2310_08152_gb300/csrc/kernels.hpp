@@ -79,6 +79,7 @@ cudaError_t launch_compact(const Geometry& g, const Static& st, const Buffers& b
                            cudaEvent_t between = nullptr);
 
 struct DecodeArgs {
+  int device;            // the current device
   int layer;             // the first layer of the launch
   int n_layers = 1;      // layers layer .. layer + n_layers - 1 in one launch (whole segments only)
   const DState* dstate;  // [b]
@@ -100,18 +101,19 @@ struct DecodeArgs {
   int64_t max_segment;
 };
 
-// How a decode launch split its work: mode 0 = stream-K over all rows, 1 / 2 = one warp per
-// (layer, sequence, head) segment with the wide / narrow pipeline, 3 = several consecutive whole
-// segments per warp, 4 = consecutive whole segments per warp cut by rows (unbalanced segments over
-// several layers); workers = warps; tile rows; stages.
+// How a decode launch split its work: mode 0 = unbalanced segments of one layer, a CTA or cluster per
+// (sequence, head) segment or stream-K over all rows; 1 = balanced segments, a CTA or cluster each or
+// up to eight per CTA; 2 = one warp per segment; 3 = several consecutive whole segments per warp;
+// 4 = unbalanced segments over several layers, one or two per CTA or runs of whole segments per warp
+// cut by rows; workers = warps that attend; tile rows; stages.
 struct DecodePlan {
   int mode, workers, tile_rows, stages;
 };
 
 // Returns the grid used through *grid (0 if nothing launched) and the plan through *plan.  A launch
-// over several layers (a.n_layers > 1) takes whole segments only: when the longest segment is too
-// long beside a warp's share of the rows it launches nothing and returns cudaErrorNotSupported, and
-// the caller goes layer by layer.
+// over several layers (a.n_layers > 1) takes whole segments only: where unbalanced segments are fewer
+// than a wave of CTAs, or the longest too long beside the rest, it launches nothing and returns
+// cudaErrorNotSupported, and the caller goes layer by layer.
 cudaError_t launch_decode(const Geometry& g, const Static& st, const Buffers& buf, const DecodeArgs& a,
                           int num_sms, cudaStream_t stream, int* grid, DecodePlan* plan);
 

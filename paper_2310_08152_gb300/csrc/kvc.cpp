@@ -809,6 +809,7 @@ static kvc_status decode_check(kvc_cache* c, int layer, int n_layers, const void
 
 static kvc::DecodeArgs decode_args(kvc_cache* c, int layer, const void* q, float scale, float* out) {
   kvc::DecodeArgs a;
+  a.device = c->device;
   a.layer = layer;
   a.dstate = reinterpret_cast<const kvc::DState*>(c->wsp(c->ws.dyn));
   a.P = reinterpret_cast<const int64_t*>(c->wsp(c->ws.dyn + c->ws.dyn_P));
@@ -905,6 +906,7 @@ kvc_status kvc_decode_attention_static_scratch(kvc_cache* c, int layer, const vo
   e = cudaMemsetAsync(counters, 0, 4 * segs, stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync (static decode scratch)");
   kvc::DecodeArgs a;
+  a.device = c->device;
   a.layer = layer;
   a.dstate = reinterpret_cast<const kvc::DState*>(c->wsp(c->ws.dyn));
   a.P = reinterpret_cast<const int64_t*>(c->wsp(c->ws.dyn + c->ws.dyn_P));

@@ -1,0 +1,82 @@
+"""Decode with a CTA or a cluster of CTAs per (layer, sequence, head) segment, or several consecutive
+segments per CTA.  Every output against the fp64 oracle at the sizes where the split can
+go wrong: clusters of 8, 4 and 2, rows just below, at and above a tile, CTAs of a cluster without rows,
+rings that wrap, open spans, the small shape, several segments per CTA, and unbalanced segments."""
+import dataclasses
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import harness
+import oracle as orc
+import oracle.workload as ow
+from synth import workloads as wl
+
+from _parity import compare, run_workload
+
+pytestmark = pytest.mark.gpu
+
+
+def _with(w, **kw):
+    d = kw.get("d", w.d)
+    return dataclasses.replace(w, scale=1.0 / math.sqrt(d), name="-".join([w.name] + [f"{k}{v}" for k, v in kw.items()]), **kw)
+
+
+def _lengths(lens, M=1):
+    """Prompts of the given lengths, spans of 32 in every 64 tokens."""
+    w = wl.opt13b(b=len(lens), L=64, M=M)
+    made = [wl.block_kinds(n, 32) for n in lens]
+    return dataclasses.replace(w, prompt_kinds=[k for k, _ in made], prompt_spans=[s for _, s in made], name=f"lens{lens}")
+
+
+# workload, steps, rows per tile and warps (None: not looked at) of the plan after the last step
+CASES = [
+    ("cluster of 8", lambda: wl.opt13b(b=1, L=4000, M=1), 3, 128, 32 * 8 * 4),
+    ("cluster of 4, d 80 rotary", lambda: wl.rope3b(32, b=2, L=2048, M=1), 3, 128, 64 * 4 * 4),
+    ("cluster of 2, bf16, d 128", lambda: _with(wl.opt13b(b=4, L=1000, M=1), dtype="bf16", d=128), 3, 64, 128 * 2 * 4),
+    ("cluster of 4, a short sequence", lambda: _lengths([3000, 40]), 3, 128, 64 * 4 * 4),
+    ("about a tile of rows, two layers", lambda: wl.opt13b_uncompressed(b=2, L=126, M=2), 3, 128, 128 * 4),
+    ("about a tile of rows, d 96", lambda: _with(wl.opt13b_uncompressed(b=2, L=62, M=1), d=96, rotary_dim=32), 3, 64, 64 * 4),
+    ("small shape", lambda: wl.opt13b(b=12, L=200, M=1), 3, 64, 384 * 2),
+    ("small shape, d 80 bf16 rotary", lambda: _with(wl.rope3b(32, b=11, L=180, M=1), dtype="bf16"), 3, 64, 352 * 2),
+    ("several segments per CTA", lambda: wl.opt13b(b=21, L=900, M=1), 3, 128, 224 * 4),
+    ("a segment per CTA, many waves, d 128", lambda: _with(wl.opt13b_uncompressed(b=40, L=170, M=2), d=128), 2, 64, 2560 * 4),
+    ("unbalanced, beyond a wave", lambda: wl.ragged(b=20, lmin=300, lmax=2000, M=1, steps=4), 3, 128, 640 * 4),
+    ("unbalanced, short, two per CTA", lambda: wl.ragged(b=21, lmin=60, lmax=400, M=1, steps=4), 3, 64, 336 * 2),
+    ("unbalanced, short, d 80, two per CTA", lambda: _with(wl.ragged(b=21, lmin=60, lmax=400, M=1, steps=4), d=80), 3, 128, 336 * 4),
+    ("unbalanced layers in one launch", lambda: wl.ragged(b=12, lmin=300, lmax=2000, M=2, steps=4), 3, 128, 768 * 4),
+]
+
+
+@pytest.mark.parametrize("name,make,steps,tile,warps", CASES, ids=[c[0] for c in CASES])
+def test_cta_per_segment(name, make, steps, tile, warps):
+    run, _ = run_workload(make(), steps=steps)
+    plan = run.cache.last_decode_plan
+    assert plan["mode"] in (0, 1, 4), plan
+    assert plan["tile_rows"] == tile and (warps is None or plan["workers"] == warps), plan
+
+
+def test_ring_that_wraps_over_a_cluster():
+    """A Local Attention window cut over a cluster of 4 CTAs, its ring's end inside one CTA's rows."""
+    w = wl.opt13b_local(b=2, L=1700, M=1)
+    run = harness.Runner(w, steps=3)
+    run.load_prompt()
+    out = torch.empty(w.M, w.b, w.H, w.d, dtype=torch.float32, device="cuda")
+    for g in range(3):
+        run.step(run.make_step_inputs(g), out)
+        torch.cuda.synchronize()
+        ref = ow.expected_local_decode(w, g + 1, 0, [0, 1], float(np.float32(0.5)))
+        compare(out[0].cpu().numpy(), ref, f"step {g}")
+    plan = run.cache.last_decode_plan
+    assert plan["workers"] == 64 * 4 * 4, plan
+    assert run.cache.device_status() == 0
+
+
+def test_open_span_hidden_row_in_every_part():
+    """A span opened at the step before: its <CL> row, hidden, lies in the last CTA's rows of a cluster
+    at first and moves into an earlier one as the span grows; both policies."""
+    for policy in (orc.POLICY_PAPER, orc.POLICY_KEEP_CL):
+        w = wl.opt13b(b=2, L=1600, M=1)
+        run_workload(w, steps=4, policy=policy)
