@@ -120,29 +120,37 @@ cudaError_t launch_decode(const Geometry& g, const Static& st, const Buffers& bu
 // ---------------------------------------------------------------------------------------------
 // Masked prefill attention (prefill.cu)
 // ---------------------------------------------------------------------------------------------
-// Per sequence: stored rows [0, len); the queries are stored rows [q0, len), the first of them is
-// token qtok of the q / out arrays; the per-row mask bounds start at meta[moff].
-struct PState {
-  int32_t len, q0, qtok, moff;
+// A prefill query tile as the host lays it out: queries [qr0, qr_end) (stored rows) of sequence s, the
+// first of them token tok0 of the q / out arrays; a work item is one tile of one head.  Its keys
+// are the stored rows some query of the tile may see, in order: the first n_c rows of the sequence's list
+// of rows that no span hides (klist[moff ..]; below vb they are the stored rows of the same number), then
+// stored rows [b0, qr0) -- the interior of a span that begins before the tile and ends in it or after it,
+// if there is one (else b0 = qr0) --, then the tile's own rows; nk tiles of keys.  The per-row mask bounds
+// start at meta[moff]; row0 = seq_row0[s], the K/V plane row of stored row 0 of head 0 in layer 0 (the
+// kernel adds layer * H * C + h * cap).
+struct PfTileRec {
+  int32_t n_c, b0, tok0, moff;
+  int32_t s, cap, qr0, qr_end;
+  int32_t nk, row0, vb, pad;
 };
-// One prefill work item (sequence s, head h, query tile [qr0, qr_end)) as the host lays it out,
-// in the kernel's order; row0 = seq_row0[s] + h * cap[s], the K/V plane row of stored row 0 in
-// layer 0 (the kernel adds layer * H * C).
+static_assert(sizeof(PfTileRec) == 48, "three 16-byte loads");
+// The work items in the kernel's order.
 struct PfItemRec {
-  PState ps;
-  int32_t s, h, qr0, qr_end;
-  int32_t nk, row0_lo, row0_hi, pad;
+  int32_t tile, h;
 };
-static_assert(sizeof(PfItemRec) == 48, "three 16-byte loads");
 
 struct PrefillArgs {
   int layer, H, rot;
   int64_t C;
-  const PfItemRec* items;  // [n_items]: sequences with the most stored rows first, then head, then the query tile with the most keys first
+  const PfItemRec* items;  // [n_items]
+  const PfTileRec* tiles;  // [n_items]: sequences with the most stored rows first, then head, then the query tile with the most keys first
   int64_t n_items;         // (query tile, head) work items
-  unsigned long long* item_counter;  // zero at launch: the CTAs take items [0, n_items) in order from it
+  unsigned long long* item_counter;  // [2], zero at launch and after it: the next item, the CTAs that are through
   int n_ctas;              // persistent grid size
   const int32_t* meta;     // per stored row: (hid << 1) | is_cl
+  const int32_t* klist;    // per sequence, from the same offset as meta: the stored rows no span hides
+  const uint16_t* k;       // the K and V planes of every layer
+  const uint16_t* v;
   const uint16_t* q;       // [sum n_q][H][D]
   float* out;              // [sum n_q][H][D]
   int64_t n_qtok;          // sum n_q
@@ -164,6 +172,10 @@ struct alignas(64) PrefillMaps {
 cudaError_t encode_prefill_maps(const Geometry& g, const Buffers& buf, PrefillMaps* maps);
 // Most CTAs of the persistent prefill grid (sizes its work-range table).
 constexpr int kMaxPrefillCtas = 1024;
+// Keys of one key tile for head dimension D and the cache type, and where a tile's own rows start among
+// its keys when n_before come before them: on a key tile of their own when those divide a query tile.
+int prefill_keys_per_tile(int D, int dtype);
+inline int prefill_own_start(int n_before, int kt) { return 128 % kt == 0 ? (n_before + kt - 1) / kt * kt : n_before; }
 // CTAs of the prefill kernel that fit on one SM for head dimension D (sizes the persistent grid).
 int prefill_ctas_per_sm(int D);
 // A persistent grid of a.n_ctas CTAs walks the a.n_items work items.

@@ -57,13 +57,12 @@ struct WsLayout {
   size_t dyn_payload = 0;  // offset of the payload inside dyn
   size_t dyn_bytes = 0;
   size_t src_map = 0;    // int32 [C]: source row of each destination row of a compaction
-  size_t counters = 0;   // int32 [b*H]
+  size_t counters = 0;   // int32 [b*H], then pre_counter
+  size_t counters_bytes = 0;
   size_t partials = 0;   // float [(kMaxDecodeWorkers + b*H) * (D + 4)]
-  size_t pre_counter = 0;  // uint64: the prefill launch's next work item
-  size_t pre = 0;        // prefill plan: [PfItemRec items][int32 meta C]
-  size_t pre_items = 0;  // offsets inside the plan; PfItemRec [pre_max_items]
-  int64_t pre_max_items = 0;
-  size_t pre_meta = 0;
+  size_t pre_counter = 0;  // uint64 [2]: the prefill launch's next work item, its CTAs that are through
+  size_t pre = 0;        // prefill plan: [PfTileRec tiles][PfItemRec items][int32 meta rows][int32 klist rows]
+  int64_t pre_max_tiles = 0;
   size_t pre_bytes = 0;
   size_t total = 0;
 };
@@ -89,15 +88,14 @@ WsLayout ws_layout(int b, int H, int D, int rot, int64_t C) {
   L.dyn_bytes = L.dyn_payload + std::max(tok, cmp);
   L.dyn = take(L.dyn_bytes);
   L.src_map = take(4 * (size_t)C);
-  L.counters = take(4 * (size_t)b * H);
+  L.pre_counter = align_up(4 * (size_t)b * H, 16);
+  L.counters_bytes = L.pre_counter + 16;
+  L.counters = take(L.counters_bytes);
+  L.pre_counter += L.counters;
   L.partials = take(4 * (size_t)(kvc::kMaxDecodeWorkers + (int64_t)b * H) * (size_t)(D + 4));
-  // work items: H per query tile, and a sequence of capacity cap has at most ceil(cap / 128) query
-  // tiles, so at most H * (C / 128 + b) in all
-  L.pre_items = 0;
-  L.pre_max_items = (int64_t)H * ((C + 127) / 128 + b);
-  L.pre_meta = align_up(L.pre_items + sizeof(kvc::PfItemRec) * (size_t)L.pre_max_items, 16);
-  L.pre_bytes = L.pre_meta + 4 * (size_t)C;
-  L.pre_counter = take(8);
+  // a sequence of capacity cap has at most ceil(cap / 128) query tiles, each with H work items
+  L.pre_max_tiles = (C + 127) / 128 + b;
+  L.pre_bytes = (sizeof(kvc::PfTileRec) + sizeof(kvc::PfItemRec) * (size_t)H) * (size_t)L.pre_max_tiles + 8 * (size_t)C;
   L.pre = take(L.pre_bytes);
   L.total = o;
   return L;
@@ -235,6 +233,7 @@ struct kvc_cache {
   uint64_t pre_version = UINT64_MAX;
   std::vector<int32_t> pre_nq;
   int64_t pre_tiles = 0;
+  size_t pre_items = 0, pre_meta = 0, pre_klist = 0;  // offsets inside the plan
   int pre_ctas = 0;
   kvc::PrefillMaps maps;
   bool amaps_ok = false;  // the append kernel's TMA descriptors are in the workspace
@@ -345,7 +344,7 @@ struct kvc_cache {
       }
     }
     e = cudaMemsetAsync(wsp(ws.hdr), 0, 256, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(wsp(ws.counters), 0, 4 * (size_t)cfg.b * cfg.H, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(wsp(ws.counters), 0, ws.counters_bytes, stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     device = dev;
     cuda_ready = true;
@@ -958,66 +957,90 @@ kvc_status kvc_prefill_attention(kvc_cache* c, int layer, const void* q, const i
   const bool same = c->pre_version == c->version && std::equal(c->pre_nq.begin(), c->pre_nq.end(), n_q) &&
                     (int)c->pre_nq.size() == b;
   if (!same) {
-    // per-sequence state, tile prefix and per-row mask bounds
+    // per-row mask bounds, the rows that no span hides, and the work items
     std::vector<std::vector<int32_t>> metas(b);
     size_t n_meta = 0;
+    int64_t n_tiles = 0;
     for (int s = 0; s < b; ++s) {
       std::string err;
       if (!c->bk.book.prefill_keys(s, n_q[s], metas[s], err)) return fail(KVC_ERR_STATE, "%s", err.c_str());
       n_meta += metas[s].size();
+      n_tiles += (n_q[s] + 127) / 128;
     }
-    const size_t bytes = c->ws.pre_meta + 4 * n_meta;
+    if (n_tiles > c->ws.pre_max_tiles) return fail(KVC_ERR_INVALID_ARG, "prefill query tiles exceed the plan");
+    const int64_t n_items = (int64_t)H * n_tiles;
+    c->pre_version = UINT64_MAX;  // until the new plan is uploaded
+    c->pre_items = sizeof(kvc::PfTileRec) * (size_t)n_tiles;
+    c->pre_meta = c->pre_items + sizeof(kvc::PfItemRec) * (size_t)n_items;
+    c->pre_klist = c->pre_meta + 4 * n_meta;
+    const size_t bytes = c->pre_klist + 4 * n_meta;
     unsigned char* img = c->ring.reserve(bytes, &e);
     if (!img) return e != cudaSuccess ? cuda_fail(e, "staging") : fail(KVC_ERR_INVALID_ARG, "prefill plan exceeds ring");
-    std::vector<kvc::PState> ps(b);
-    std::vector<int32_t> Pq(b + 1);
-    int32_t* meta = reinterpret_cast<int32_t*>(img + c->ws.pre_meta);
-    int64_t qtok = 0, moff = 0;
-    Pq[0] = 0;
-    for (int s = 0; s < b; ++s) {
-      const int64_t len = c->bk.book.stored(s);
-      ps[s].len = (int32_t)len;
-      ps[s].q0 = (int32_t)(len - n_q[s]);
-      ps[s].qtok = (int32_t)qtok;
-      ps[s].moff = (int32_t)moff;
-      std::memcpy(meta + moff, metas[s].data(), 4 * metas[s].size());
-      moff += (int64_t)metas[s].size();
-      qtok += n_q[s];
-      Pq[s + 1] = Pq[s] + (n_q[s] + 127) / 128;
+    kvc::PfTileRec* tiles = reinterpret_cast<kvc::PfTileRec*>(img);
+    kvc::PfItemRec* items = reinterpret_cast<kvc::PfItemRec*>(img + c->pre_items);
+    int32_t* meta = reinterpret_cast<int32_t*>(img + c->pre_meta);
+    int32_t* klist = reinterpret_cast<int32_t*>(img + c->pre_klist);
+    std::vector<int32_t> qtok(b), moff(b);
+    {
+      int64_t t = 0, m = 0;
+      for (int s = 0; s < b; ++s) {
+        qtok[s] = (int32_t)t;
+        moff[s] = (int32_t)m;
+        t += n_q[s];
+        m += (int64_t)metas[s].size();
+      }
     }
-    // Work items (sequence, head, query tile) in the kernel's order: sequence (longest first), head,
-    // the tile with the most keys first.
-    const int64_t n_items = (int64_t)H * Pq[b];
-    if (n_items > c->ws.pre_max_items) return fail(KVC_ERR_INVALID_ARG, "prefill work items exceed the plan");
     // a persistent grid: every SM's CTAs, which take the items in this order from the launch's
     // counter, so the items in flight at any time are neighbours sharing K/V tiles in L2
     const int G = (int)std::min<int64_t>(
         std::min(c->num_sms * kvc::prefill_ctas_per_sm(c->cfg.d_head), kvc::kMaxPrefillCtas), n_items);
     {
-      // sequences with the most stored rows first, so the heaviest items are taken early and the
-      // last ones taken are short
+      // Work items (sequence, head, query tile) in the kernel's order: the sequences with the most
+      // stored rows first, so the heaviest items are taken early and the last ones taken are short, then
+      // head, then the tile with the most keys first.
       std::vector<int> order(b);
       for (int s = 0; s < b; ++s) order[s] = s;
-      std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return ps[x].len > ps[y].len; });
-      kvc::PfItemRec* items = reinterpret_cast<kvc::PfItemRec*>(img + c->ws.pre_items);
-      int64_t item = 0;
+      std::stable_sort(order.begin(), order.end(),
+                       [&](int x, int y) { return c->bk.book.stored(x) > c->bk.book.stored(y); });
+      int32_t tile = 0;
+      const int kt = kvc::prefill_keys_per_tile(c->cfg.d_head, c->cfg.dtype);
+      std::vector<int32_t> before;        // rows that no span hides before each stored row
       for (int s : order) {
-        const int nqt = Pq[s + 1] - Pq[s];
+        const int nqt = (n_q[s] + 127) / 128;
+        if (nqt == 0) continue;
+        const std::vector<int32_t>& mt = metas[s];
+        const int len = (int)mt.size(), q0 = len - n_q[s];
+        std::memcpy(meta + moff[s], mt.data(), 4 * mt.size());
+        before.resize((size_t)len + 1);
+        int32_t n = 0;
+        for (int i = 0; i < len; ++i) {
+          before[i] = n;
+          if ((mt[i] >> 1) == kvc::Book::kPrefillNever) klist[moff[s] + n++] = i;
+        }
+        before[len] = n;
+        int vb = 0;  // list rows before the first hidden row
+        while (vb < n && klist[moff[s] + vb] == vb) ++vb;
+        for (int qt = nqt - 1, t = tile; qt >= 0; --qt, ++t) {
+          kvc::PfTileRec r{};
+          r.qr0 = q0 + 128 * qt;
+          r.qr_end = std::min(r.qr0 + 128, len);
+          // interior rows of a span that begins before the tile and whose <CR> is in or after it
+          int b0 = r.qr0;
+          while (b0 > 0 && (mt[b0 - 1] >> 1) != kvc::Book::kPrefillNever && (mt[b0 - 1] >> 1) >= r.qr0) --b0;
+          r.b0 = b0;
+          r.n_c = before[b0];
+          r.vb = vb;
+          r.tok0 = qtok[s] + 128 * qt;
+          r.moff = moff[s];
+          r.s = s;
+          r.cap = (int32_t)c->cap[s];
+          r.row0 = (int32_t)((int64_t)H * c->off[s]);  // = seq_row0[s]
+          r.nk = (kvc::prefill_own_start(r.n_c + r.qr0 - b0, kt) + r.qr_end - r.qr0 + kt - 1) / kt;
+          tiles[t] = r;
+        }
         for (int h = 0; h < H; ++h)
-          for (int k = 0; k < nqt; ++k, ++item) {
-            kvc::PfItemRec& r = items[item];
-            const int qt = nqt - 1 - k;
-            r.ps = ps[s];
-            r.s = s;
-            r.h = h;
-            r.qr0 = ps[s].q0 + 128 * qt;
-            r.qr_end = std::min(r.qr0 + 128, ps[s].len);
-            r.nk = (r.qr_end + 127) / 128;
-            const int64_t row0 = (int64_t)H * c->off[s] + (int64_t)h * c->cap[s];  // = seq_row0[s] + h * cap[s]
-            r.row0_lo = (int32_t)(uint32_t)(uint64_t)row0;
-            r.row0_hi = (int32_t)((uint64_t)row0 >> 32);
-            r.pad = 0;
-          }
+          for (int t = 0; t < nqt; ++t) *items++ = {tile + t, h};
+        tile += nqt;
       }
     }
     c->pre_ctas = G;
@@ -1025,7 +1048,7 @@ kvc_status kvc_prefill_attention(kvc_cache* c, int layer, const void* q, const i
     if (e != cudaSuccess) return cuda_fail(e, "upload prefill plan");
     c->pre_version = c->version;
     c->pre_nq.assign(n_q, n_q + b);
-    c->pre_tiles = Pq[b];
+    c->pre_tiles = n_tiles;
   }
   if (c->pre_tiles == 0) return ok();
   kvc::PrefillArgs a;
@@ -1033,8 +1056,12 @@ kvc_status kvc_prefill_attention(kvc_cache* c, int layer, const void* q, const i
   a.H = H;
   a.rot = c->cfg.rotary_dim;
   a.C = c->C;
-  a.items = reinterpret_cast<const kvc::PfItemRec*>(c->wsp(c->ws.pre + c->ws.pre_items));
-  a.meta = reinterpret_cast<const int32_t*>(c->wsp(c->ws.pre + c->ws.pre_meta));
+  a.items = reinterpret_cast<const kvc::PfItemRec*>(c->wsp(c->ws.pre + c->pre_items));
+  a.tiles = reinterpret_cast<const kvc::PfTileRec*>(c->wsp(c->ws.pre));
+  a.meta = reinterpret_cast<const int32_t*>(c->wsp(c->ws.pre + c->pre_meta));
+  a.k = static_cast<const uint16_t*>(c->cfg.k_base);
+  a.v = static_cast<const uint16_t*>(c->cfg.v_base);
+  a.klist = reinterpret_cast<const int32_t*>(c->wsp(c->ws.pre + c->pre_klist));
   a.q = static_cast<const uint16_t*>(q);
   a.out = out;
   a.n_qtok = 0;
@@ -1050,8 +1077,6 @@ kvc_status kvc_prefill_attention(kvc_cache* c, int layer, const void* q, const i
   a.n_items = (int64_t)H * c->pre_tiles;
   a.item_counter = reinterpret_cast<unsigned long long*>(c->wsp(c->ws.pre_counter));
   a.n_ctas = c->pre_ctas;
-  e = cudaMemsetAsync(a.item_counter, 0, sizeof(unsigned long long), stream);
-  if (e != cudaSuccess) return cuda_fail(e, "reset the prefill item counter");
   e = kvc::launch_prefill(c->geom(), c->maps, a, stream);
   if (e != cudaSuccess) return cuda_fail(e, "prefill kernel");
   c->launches += 1;

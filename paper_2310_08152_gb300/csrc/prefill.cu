@@ -3,23 +3,37 @@
 //
 // Work items are (sequence, head, 128-query tile); the queries are the last tokens of each
 // sequence's history, the keys the sequence's stored rows of one layer, read straight from the
-// ragged cache.  Persistent CTAs (two per SM for d_head 64 and 80, one otherwise) each walk a
-// contiguous range of items that the host balances.  Per CTA:
+// ragged cache.  Persistent CTAs (two per SM for d_head 64 and 80, one otherwise) take the items one by
+// one in the host's order.  Per CTA:
 //
 //   warps 0..3   softmax, one query row per thread: tcgen05.ld of its S row, the per-key rule on the
 //                tiles that need it, an online softmax in the exp2 domain, P (16-bit) back into TMEM,
 //                the rare rescale of its O row, and the final O / l
-//   warp 4       TMA producer: 2-D tiled copies (cp.async.bulk.tensor, swizzled) of 128-row K and V
-//                tiles into a ring of shared-memory stages, the tile's mask columns and key classes
-//   warp 5       one thread issues tcgen05.mma: S = Q K^T (plus the mask columns) into TMEM, then
-//                O += P V with P read from TMEM; completions are signalled with tcgen05.commit
-//   warps 6, 7   idle (they complete the producer's warpgroup, whose registers go to the softmax)
+//   warp 4       takes the work items and sorts the keys of the tiles that need the per-key rule
+//   warp 5       one thread issues tcgen05.mma: S = Q K^T into TMEM, then O += P V with P read from
+//                TMEM; completions are signalled with tcgen05.commit
+//   warps 6, 7   stream the K tiles and the V tiles, each through a ring of shared-memory stages
 //
 // Mask (Sec. 3.1, the same rows a decode at the query would see): stored row i is visible to the
 // query at stored row iq exactly when i <= iq <= hid(i), except that a <CL> query sees only itself.
 // hid(i) is the stored row of the <CR> that closes a span enclosing row i (its interior stops being
 // visible after the <CR>), i itself for a <CL> row under the paper policy, and "never" otherwise;
 // the host book computes it per stored row.
+//
+// Only keys that some query of a tile may see are fetched: the rows that no span hides, from a list of
+// them, and the rows of the tile itself with the interior of a span it begins in.  A tile of keys whose
+// rows lie side by side is one TMA copy (2-D tiled, swizzled); else its rows are gathered with 16-byte
+// asynchronous copies into the same swizzled layout.
+//
+// What bounds it: the softmax warps' instructions (exp2, max and packing of 128 scores a row), and, since the
+// eight warps of a CTA run five different programs, the instruction cache: every stretch of straight-line code
+// taken out paid more than its instructions' issue slots.  So waits are one short loop, the epilogue and the
+// masking exist once, and nothing but the softmax is unrolled far.  Time of a layer, against a kernel that read
+// every stored row with masks over all of them: OPT-1.3B-shaped prompts (16 x 2048 tokens, 32 heads of 64,
+// interiors of 32) 541 -> 362 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 990 us; the
+// last 512 of 32 x 4096 tokens, compacted before them, bf16 (heads of 80) 664 -> 456 us; the first with 96 and
+// 128 columns 797 -> 580 and 1042 -> 602 us; one prompt of 300 tokens 13.2 -> 12.2 us.  Copying the listed rows side by side first, for TMA tiles alone, took a
+// second kernel and 381, 992 and 454 us on the first three.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -34,15 +48,14 @@
 namespace kvc {
 namespace {
 
-constexpr int kPfRows = 128;  // queries per tile (MMA M) and keys per tile (QK^T N, PV K)
-// Threads: a softmax warpgroup (one thread per query row), then a warpgroup holding the producer
-// warp, the MMA warp and two idle warps (so that registers can be moved between the two).
+constexpr int kPfRows = 128;  // queries per tile (MMA M)
+// Threads: a softmax warpgroup (one thread per query row), then a warpgroup of the four other roles' warps
+// (so that registers can be moved between the two).
 constexpr int kPfThreads = 256;
-// Work items reach the MMA and softmax warps through a ring of this many slots, filled by the
-// producer warp as it takes them from the launch's counter.
-constexpr int kItemRing = 4;
+constexpr int kItemRing = 4;  // a power of two: the item in hand, the ones before and after it
+constexpr int kClsRing = 2;  // sorted key tiles ahead of the softmax
 
-// Shared-memory geometry for head dimension D.  Q, K and V tiles are [128 rows][D] split into
+// Shared-memory geometry for head dimension D.  Q ([128 rows][D]), K and V tiles ([KT rows][D]) are split into
 // column subtiles of SW bytes per row, the widest swizzle (128 / 64 / 32 bytes) that divides a row;
 // each subtile is the canonical K-major (Q, K) or MN-major (V) layout of that swizzle.
 //
@@ -57,58 +70,57 @@ struct PfCfg {
   static constexpr int SW = (2 * D) % 128 == 0 ? 128 : (2 * D) % 64 == 0 ? 64 : 32;
   static constexpr int SUB = SW / 2;  // columns per subtile
   static constexpr int NSUB = D / SUB;
-  static constexpr uint32_t SUBB = kPfRows * SW;  // bytes of one subtile
-  static constexpr uint32_t TILE = kPfRows * D * 2;
   // d_head 64 and 80 run two CTAs per SM (their softmax steps interleave), each with a single S
-  // tile in TMEM and two K/V stages; larger heads run one CTA per SM with a double-buffered S tile.
+  // tile in TMEM; larger heads run one CTA per SM with a double-buffered S tile.
   static constexpr int CPS = (D == 64 || D == 80) ? 2 : 1;  // CTAs per SM
   static constexpr int SBUF = CPS == 2 ? 1 : 2;              // S tiles in TMEM
-  static constexpr bool PSEP = D == 64 && !SPLIT;            // P in TMEM columns of its own
-  static constexpr bool XQT = CPS == 2 && !PSEP;             // Q's mask column in TMEM, not smem
+  static constexpr bool PSEP = CPS == 2;                     // P in TMEM columns of its own
+  // Keys per tile (QK^T N, PV K): with two CTAs per SM as many as leave TMEM columns for a P of its own
+  // (d_head 80, OPT-2.7B-shaped blocks in bf16: 128 keys with P over S 534 us, 64 with P apart 505).
+  static constexpr int KT = !PSEP ? 128 : SPLIT ? 64 : D == 80 ? 112 : 128;
+  static constexpr uint32_t QSUBB = kPfRows * SW;  // bytes of one subtile of Q
+  static constexpr uint32_t SUBB = KT * SW;        // of K or V
+  static constexpr uint32_t QTILE = kPfRows * D * 2;
+  static constexpr uint32_t TILE = KT * D * 2;
   // SPLIT: the low part of the rotated query, the A operand of a second Q.K^T pass, lives in TMEM
   // with two CTAs per SM (whose shared memory is full) and in shared memory with one
   static constexpr bool QLO_TMEM = SPLIT && CPS == 2;
   static constexpr bool QLO_SMEM = SPLIT && CPS == 1;
-  static constexpr int NST = CPS == 2 ? 2 : D <= 96 ? 3 : 2;  // K/V stages
+  // stages of the K and of the V ring
+  static constexpr int KST = CPS == 2 ? (SPLIT ? 3 : 2) : D <= 96 || !SPLIT ? 3 : 2;
+  static constexpr int VST = CPS == 2 ? (SPLIT ? 3 : 2) : D <= 96 ? 3 : 2;
   static constexpr uint32_t Q_OFF = 0;
-  static constexpr uint32_t QLO_OFF = TILE;  // QLO_SMEM only
-  static constexpr uint32_t KV_OFF = TILE * (QLO_SMEM ? 2 : 1);
-  // Mask columns: one 16-column subtile (32-byte swizzle) appended to Q (a constant) and to every K
-  // stage (0 or a large negative number per key), so keys hidden from a whole query tile are masked
-  // by the Q.K^T product itself.
-  static constexpr uint32_t XQ_OFF = KV_OFF + NST * 2 * TILE;
-  static constexpr uint32_t XK_OFF = XQ_OFF + (XQT ? 0 : kPfRows * 32);
-  // d_head 64 has shared memory to spare for O / l: each softmax warp stages 32 rows x 32 columns
-  // (4 KB, 128-byte swizzle) for a TMA tensor store
-  static constexpr bool OSTAGE = D == 64;
-  static constexpr uint32_t OST_OFF = (XK_OFF + NST * kPfRows * 32 + 1023) / 1024 * 1024;
-  static constexpr uint32_t OST_WARP = 32 * 32 * 4;
-  static constexpr uint32_t SMEM = (OSTAGE ? OST_OFF + 4 * OST_WARP : XK_OFF + NST * kPfRows * 32) +
-                                   1024;  // + slack to align the base to 1024
-  // TMEM.  d_head 64 (two CTAs per SM, 256 columns each): S [0,128), P [128,192) (16-bit, two
-  // per column), O [192,256) -- S is released as soon as the softmax has read it, so the next
-  // Q.K^T overlaps the softmax.  d_head 80 (two CTAs per SM): S [0,128) with P written over its
-  // first 64 columns, O [128,208), Q's mask column [208,216) -- the next Q.K^T follows the P.V.
-  // One CTA per SM: S0 [0,128), S1 [128,256), P written over the first 64 columns of its own S
-  // tile, then O0 and O1 (alternating per item).  SPLIT: P's high part over the first 64 columns of
-  // its S tile and its low part over the other 64 (d_head 64 then lays TMEM out as d_head 80 does);
-  // with two CTAs per SM the query's low part follows Q's mask column (D / 2 columns).
-  static constexpr uint32_t P_COL = PSEP ? kPfRows : 0;  // else P lives in its S tile
-  static constexpr uint32_t PLO_COL = kPfRows / 2;       // SPLIT: P's low part, after its high part
+  static constexpr uint32_t QLO_OFF = QTILE;  // QLO_SMEM only
+  static constexpr uint32_t K_OFF = QTILE * (QLO_SMEM ? 2 : 1);
+  static constexpr uint32_t V_OFF = K_OFF + KST * TILE;
+  // With two CTAs per SM there is shared memory left for O / l: each softmax warp has OST_N buffers of 32
+  // rows x 16 columns (2 KB, 64-byte swizzle) for TMA tensor stores.
+  static constexpr bool OSTAGE = CPS == 2;
+  static constexpr int OST_N = D == 64 ? 3 : 2;
+  static constexpr uint32_t OST_OFF = (V_OFF + VST * TILE + 1023) / 1024 * 1024;
+  static constexpr uint32_t OST_BUF = 32 * 16 * 4;
+  static constexpr uint32_t SMEM = OST_OFF + (OSTAGE ? 4 * OST_N * OST_BUF : 0) + 1024;  // + aligning the base
+  // TMEM.  Two CTAs per SM, 256 columns each: S, O, P (16-bit, two per column; SPLIT: its high part, then
+  // its low part) and SPLIT's low part of the query (D / 2 columns) in columns of their own, so S is
+  // released as soon as the softmax has read it and the next Q.K^T overlaps the softmax.  One CTA per SM:
+  // S0, S1, P written over the first half of its own S tile (SPLIT: the low part over the other), then
+  // O0 and O1 (alternating per item).
   static constexpr int OBUF = SBUF == 1 ? 1 : 2;
-  static constexpr uint32_t O_COL = SBUF == 2 ? 2 * kPfRows : PSEP ? kPfRows + kPfRows / 2 : kPfRows;
-  static constexpr uint32_t XQ_COL = O_COL + OBUF * D;  // with XQT: 8 columns, 16 elements per row
-  static constexpr uint32_t QLO_COL = XQ_COL + (XQT ? 8 : 0);
-  static constexpr uint32_t TMEM_END = QLO_COL + (QLO_TMEM ? D / 2 : 0);
+  static constexpr uint32_t O_COL = SBUF == 2 ? 2 * KT : KT;
+  static constexpr uint32_t P_COL = PSEP ? KT + D : 0;  // 0: P lives in its S tile
+  static constexpr uint32_t PLO_COL = KT / 2;           // SPLIT: P's low part, after its high part
+  static constexpr uint32_t QLO_COL = P_COL + KT;       // QLO_TMEM only
+  static constexpr uint32_t TMEM_END = !PSEP ? O_COL + OBUF * D : SPLIT ? QLO_COL + D / 2 : P_COL + KT / 2;
   static constexpr uint32_t TMEM_COLS = TMEM_END <= 256 ? 256 : 512;
   static_assert(TMEM_END <= TMEM_COLS && TMEM_COLS * CPS <= 512, "TMEM budget");
   static_assert(D % 16 == 0 && SW * NSUB == 2 * D, "bad tile geometry");
-  static_assert(SMEM <= 227 * 1024 && (CPS == 1 || SMEM + 4096 <= 113 * 1024), "shared memory budget");
-  // Registers with two CTAs per SM: each thread is launched with REG_LAUNCH, then the producer's
+  static_assert(SMEM <= 227 * 1024 && (CPS == 1 || SMEM + 6 * 1024 <= 113 * 1024), "shared memory budget");
+  // Registers with two CTAs per SM: each thread is launched with REG_LAUNCH, then the other roles'
   // warpgroup gives registers up (setmaxnreg.dec to REG_OTHER) and the softmax warpgroup takes them
   // (setmaxnreg.inc to REG_SOFTMAX); the two shares add up to exactly what the CTA was launched with.
   static constexpr int REG_LAUNCH = 65536 / (CPS * kPfThreads);
-  static constexpr int REG_OTHER = 40;
+  // (the gather spills below that: 64 columns 370 us with 48, 358 with 56; 80 columns 1027 with 48, 984 with 64)
+  static constexpr int REG_OTHER = D == 64 ? 56 : 64;
   static constexpr int REG_SOFTMAX = (REG_LAUNCH * kPfThreads - REG_OTHER * 128) / 128 / 8 * 8;
   static_assert(CPS == 1 || REG_SOFTMAX * 128 + REG_OTHER * 128 <= REG_LAUNCH * kPfThreads,
                 "setmaxnreg shares exceed the launch allocation");
@@ -125,6 +137,13 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
+          "r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
+      : "memory");
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
@@ -140,7 +159,11 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t sr
                : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// At most N of this thread's bulk groups are still reading shared memory.
+template <int N>
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
 __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -276,114 +299,161 @@ constexpr bool kSplit<BF16T> = true;
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+// Arrives on the barrier (within its expected count) once this thread's asynchronous copies so far have
+// completed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+// Waits for every asynchronous copy of this thread, committed or not.
+__device__ __forceinline__ void cp_async_wait_all_groups() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   uint4 v;
   asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
   return v;
 }
 
-// Bits [0, n) of a 32-bit word, n clamped to [0, 32].
-__device__ __forceinline__ uint32_t low_bits(int n) { return n <= 0 ? 0u : n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u; }
+__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 
+// Bits [0, n) of a 32-bit word, n clamped to [0, 32].
+__device__ __forceinline__ uint32_t low_bits(int n) {
+  uint32_t r;
+  asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(r) : "r"(max(n, 0)));
+  return r;
+}
+// The maximum, NaN if one of them is.
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
 
-// Named barrier over the softmax warpgroups that also ANDs a flag across them.
-__device__ __forceinline__ bool bar_and(int id, int n, bool v) {
-  uint32_t r;
+// Bounded wait for the phase with the given parity: false after limit_ns (< 2^32).  A few instructions,
+// because it is inlined at many places of one kernel whose warps run different code at the same time, and
+// the instruction cache holds only so much of that; each role reports a wait that ran out when it ends.
+__device__ __forceinline__ bool pf_wait(uint64_t* bar, uint32_t parity, uint32_t limit_ns) {
+  uint32_t ok;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.and.pred p, %2, %3, q;\n\t"
+      "{\n\t.reg .pred p, q;\n\t.reg .u32 t0, t;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE;\n\t"
+      "mov.u32 t0, %%globaltimer_lo;\n\t"
+      "LOOP:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE;\n\t"
+      "mov.u32 t, %%globaltimer_lo;\n\t"
+      "sub.u32 t, t, t0;\n\t"
+      "setp.lt.u32 q, t, %3;\n\t"
+      "@q bra LOOP;\n\t"
+      "DONE:\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)v), "r"(id), "r"(n)
+      : "=r"(ok)
+      : "r"(smem_addr(bar)), "r"(parity), "r"(limit_ns)
       : "memory");
-  return r != 0;
+  return ok != 0;
 }
 
-// Bounded wait that also gives up as soon as another role of the CTA has given up.
-__device__ __forceinline__ bool pf_wait(uint64_t* bar, uint32_t parity, const PrefillArgs& a,
-                                        volatile int* abort_flag) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 63u) == 0) {
-      if (*abort_flag) return false;
-      if (global_ns() - t0 > a.wait_limit_ns) {
-        *abort_flag = 1;
-        atomicOr(a.status, STATUS_TIMEOUT);
-        return false;
-      }
-    }
-  }
-}
-
-// One work item: query tile [qr0, qr_end) of (sequence s, head h), read from the host's table.
+// One work item (kernels.hpp, PfItemRec and its PfTileRec), read from the host's tables; nk = 0: none left.
 struct PfItem {
-  PState ps;
+  int n_c, b0, tok0, moff;
   int s, h, qr0, qr_end, nk;
-  int64_t row_base;  // K/V plane row of stored row 0 of (layer, s, h)
+  int odd;       // the item's number is odd
+  int row_base;  // K/V plane row of stored row 0 of (layer, s, h)
+  int vb;
+  // keys before the tile's own rows; the first of those (kt keys per tile); one past the last key
+  __device__ __forceinline__ int before() const { return n_c + (qr0 - b0); }
+  __device__ __forceinline__ int own(int kt) const {
+    return kPfRows % kt == 0 ? (before() + kt - 1) / kt * kt : before();
+  }
+  __device__ __forceinline__ int keys(int kt) const { return own(kt) + (qr_end - qr0); }
+  // Key tile of the j-th step: consecutive items run their key tiles in opposite directions, so an item
+  // starts on the tiles its predecessor (same (sequence, head), most often) read last, while they are
+  // still in L2.
+  __device__ __forceinline__ int key_tile(int j) const { return odd ? nk - 1 - j : j; }
 };
 
 __device__ __forceinline__ PfItem pf_item(const PrefillArgs& a, int64_t it) {
-  const int4* r = reinterpret_cast<const int4*>(a.items + it);
+  const int2 t = __ldg(reinterpret_cast<const int2*>(a.items + it));
+  const int4* r = reinterpret_cast<const int4*>(a.tiles + t.x);
   const int4 x = __ldg(r), y = __ldg(r + 1), z = __ldg(r + 2);
   PfItem w;
-  w.ps = PState{x.x, x.y, x.z, x.w};
+  w.n_c = x.x;
+  w.b0 = x.y;
+  w.tok0 = x.z;
+  w.moff = x.w;
   w.s = y.x;
-  w.h = y.y;
+  w.h = t.y;
   w.qr0 = y.z;
   w.qr_end = y.w;
   w.nk = z.x;
-  w.row_base = (int64_t)a.layer * a.H * a.C + (int64_t)(((uint64_t)(uint32_t)z.z << 32) | (uint32_t)z.y);
+  w.odd = (int)(it & 1);
+  w.row_base = (int)((int64_t)a.layer * a.H * a.C) + z.y + t.y * y.y;  // all planes' rows are below 2^31
+  w.vb = z.z;
   return w;
 }
 
-// Key tile of the j-th step of item it: consecutive items run their key tiles in opposite
-// directions, so an item starts on the tiles its predecessor (same (sequence, head), most often)
-// read last, while they are still in L2.
-__device__ __forceinline__ int pf_key_tile(int64_t it, int j, int nk) { return (it & 1) ? nk - 1 - j : j; }
+// Gathers rows p0 .. p0 + 31 of a tile (row: lane's own, -1 none: zeros) below row kt, subtiles U0 .. U0 + NS - 1, with
+// 16-byte asynchronous copies.  Each quarter of the warp, whose 128 bytes are written to shared memory together,
+// covers the chunks of one subtile in as many rows as fill its swizzle pattern, so that they fall into different
+// banks; its quarters lie side by side in the rows, as far as the row goes (96 columns: 621 us with lanes in
+// row order, 577 so).  The steps of a row of the loop wait on shuffles, so they are unrolled where the code has
+// room (128 columns: 657 us by fours, 592 by eights; 64 columns: 358 by fours, 353 by twos, 372 one by one).
+template <int D, int SW, int U0, int NS>
+__device__ __forceinline__ void gather_rows(uint32_t dst, uint32_t subb, const uint16_t* rows, int row, int p0, int kt,
+                                            int lane) {
+  constexpr int CH = SW / 16, RQ = 8 / CH;  // chunks of a subtile's row, rows of a quarter
+  constexpr int RPS = RQ * 4 / NS;          // rows of a step
+  const int q = lane >> 3, cw = lane % CH, u = U0 + q % NS, pr = q / NS * RQ + lane % 8 / CH;
+  const uint16_t* src = rows + u * (SW / 2) + cw * 8;
+  dst += u * subb + p0 * SW;
+  const int n = kt - p0 < 32 ? kt - p0 : 32;  // a multiple of 16
+#pragma unroll (D == 64 ? 2 : 8)
+  for (int i = 0; i < n; i += RPS) {
+    const int p = i + pr, x = __shfl_sync(0xFFFFFFFFu, row, p);
+    const int phys = cw ^ ((p * SW >> 7) & (CH - 1));
+    cp_async16(dst + p * SW + phys * 16, src + (int64_t)max(x, 0) * D, x < 0 ? 0u : 16u);
+  }
+}
 
-// Persistent: the CTAs take items in the table's order from the launch's counter, one at a time (the
-// producer warp takes an item when it starts streaming it and passes it on through the ring); every
+// Persistent: the CTAs take items in the table's order from the launch's counter, one at a time (warp 4
+// takes an item when the K warp is through with the last one and passes it on); every
 // barrier phase counts tiles over all of the CTA's items, so the producer streams the next item's
 // K/V while the current one finishes (with two S tiles, the O accumulator also alternates between
 // two TMEM buffers per item).
 template <typename T, int D>
 __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     prefill_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                   const __grid_constant__ CUtensorMap tm_o, const PrefillArgs a) {
+                   const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_o,
+                   const PrefillArgs a) {
   using Cf = PfCfg<D, kSplit<T>>;
-  constexpr int SW = Cf::SW, SUB = Cf::SUB, NST = Cf::NST, SBUF = Cf::SBUF;
+  constexpr int SW = Cf::SW, SUB = Cf::SUB, KST = Cf::KST, VST = Cf::VST, SBUF = Cf::SBUF, KT = Cf::KT;
   extern __shared__ uint8_t pf_smem_raw[];
-  __shared__ uint64_t full_bar[NST], empty_bar[NST], s_full[SBUF], s_free;
-  __shared__ uint64_t q_full, p_full, pv_done, drain;
-  // the CTA's k-th item in slot k % kItemRing (-1: none left); full: the producer has written it,
-  // empty: the MMA thread and the four softmax warps have read it
-  __shared__ int64_t item_ring[kItemRing];
-  __shared__ uint64_t item_full[kItemRing], item_empty[kItemRing];
-  // Per stage, the tile's keys against its item's query tile [qr0, qr_end): khid has bit c set when
-  // key c's bound holds for every query of the tile (hid >= qr_end - 1).  The keys whose bound falls
-  // inside it (qr0 <= hid < qr_end - 1: a span closing among the queries) come in runs of one bound
-  // -- a span's interior shares its <CR>, a <CL> hidden from every later query is a run of one --
-  // kept as the bound (rhid) and the column range [cb, ce) (rcol = cb | ce << 16), kn runs.
-  __shared__ uint4 khid[NST];
-  __shared__ int32_t rhid[NST][kPfRows];
-  __shared__ uint32_t rcol[NST][kPfRows];
-  __shared__ int32_t kn[NST];
-  __shared__ int32_t kslow[NST];  // the tile needs the per-key rule (else its mask columns decide)
-  __shared__ PfItem next_item;  // the item after the current one, as the softmax warps found it
-  __shared__ int32_t qmeta[kPfRows];  // mask bounds of the query rows of the next item
+  __shared__ uint64_t k_full[KST], k_empty[KST], v_full[VST], v_empty[VST], s_full[SBUF], s_free;
+  // the item's raw query rows are in; rotated (RoPE); its last Q.K^T is complete
+  __shared__ uint64_t q_raw, q_full, q_empty;
+  __shared__ uint64_t p_full, pv_done, drain;
+  // the CTA's k-th item in slot k % kItemRing; full: warp 4 has written it, empty: the MMA thread, the K and V
+  // warps and the four softmax warps are through with it, last: the K warp has issued its last tile
+  __shared__ PfItem item_slot[kItemRing];
+  __shared__ uint64_t item_full[kItemRing], item_empty[kItemRing], item_last;
+  // For the key tiles that hold rows from b0 on, the tile's keys against its item's query tile
+  // [qr0, qr_end): khid has bit c set when key c's bound holds for every query of the tile (hid >=
+  // qr_end - 1).  The keys whose bound falls inside it (qr0 <= hid < qr_end - 1: a span closing among
+  // the queries) come in runs of one bound -- a span's interior shares its <CR>, a <CL> hidden from
+  // every later query is a run of one -- kept as the bound (rhid) and the columns (rbits), kn runs.
+  __shared__ uint4 khid[kClsRing];
+  __shared__ int32_t rhid[kClsRing][KT];
+  __shared__ uint4 rbits[kClsRing][KT];
+  __shared__ int32_t kn[kClsRing];
+  __shared__ int32_t kslow[kClsRing];  // the tile needs the per-key rule (else every key is visible)
+  __shared__ uint64_t cls_full[kClsRing], cls_empty[kClsRing];
   __shared__ uint32_t tmem_slot;
-  __shared__ volatile int abort_flag;
 
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -395,85 +465,102 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (threadIdx.x == 32) {
-    for (int i = 0; i < NST; ++i) {
-      mbar_init(&full_bar[i], 32);
-      mbar_init(&empty_bar[i], 1);
+    for (int i = 0; i < KST; ++i) {
+      mbar_init(&k_full[i], 32);
+      mbar_init(&k_empty[i], 1);
+    }
+    for (int i = 0; i < VST; ++i) {
+      mbar_init(&v_full[i], 32);
+      mbar_init(&v_empty[i], 1);
+    }
+    for (int i = 0; i < kClsRing; ++i) {
+      mbar_init(&cls_full[i], 1);
+      mbar_init(&cls_empty[i], 4);
     }
     for (int i = 0; i < SBUF; ++i) mbar_init(&s_full[i], 1);
     mbar_init(&s_free, 128);  // one S tile: the softmax has read it
+    mbar_init(&q_raw, 1);
     mbar_init(&q_full, 128);
+    mbar_init(&q_empty, 1);
     mbar_init(&p_full, 128);
     mbar_init(&pv_done, 1);
     mbar_init(&drain, 1);
     for (int i = 0; i < kItemRing; ++i) {
       mbar_init(&item_full[i], 1);
-      mbar_init(&item_empty[i], 1 + 4);
+      mbar_init(&item_empty[i], 1 + 2 + 4);
     }
-    abort_flag = 0;
+    mbar_init(&item_last, 1);
     fence_mbar_init();
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_slot;
-  // At the two-CTA register cap, registers go from the producer's warpgroup to the softmax: each
+  const uint32_t limit_ns = (uint32_t)a.wait_limit_ns;
+  bool ok = true;  // false once one of this role's waits has run out
+  // At the two-CTA register cap, registers go from the other roles' warpgroup to the softmax: each
   // role starts with its setmaxnreg (every warp of a warpgroup executes the same one).
   auto regs_other = [] {
     if constexpr (Cf::CPS == 2) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(Cf::REG_OTHER));
   };
 
+  // Waits for the CTA's kk-th item, in item_slot[kk % kItemRing] (false: the wait gave up); done: a whole
+  // warp is through with it.
+  auto item_wait = [&](uint32_t kk) -> bool {
+    return pf_wait(&item_full[kk % kItemRing], (kk / kItemRing) & 1, limit_ns);
+  };
+  auto item_done = [&](uint32_t kk) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&item_empty[kk % kItemRing]);
+  };
+
   if (warp == 4) {
     regs_other();
-    // ---------------- producer ----------------
-    int64_t g = 0;  // tiles issued
-    bool ok = true;
+    // ---------------- items and key classes ----------------
+    uint32_t cg = 0;  // tiles sorted
     for (uint32_t k = 0; ok; ++k) {
-      // take the next item and pass it on
-      const int slot = (int)(k % kItemRing);
-      if (k >= kItemRing && !pf_wait(&item_empty[slot], ((k / kItemRing) - 1) & 1, a, &abort_flag)) {
-        ok = false;
-        break;
-      }
-      int64_t it = -1;
+      // take the next item, once the K warp is through with the last one (no CTA holds an item that
+      // another could start on), and pass it on
+      if (k >= 1) ok = pf_wait(&item_last, (k - 1) & 1, limit_ns);
+      if (ok && k >= kItemRing) ok = pf_wait(&item_empty[k % kItemRing], (k / kItemRing - 1) & 1, limit_ns);
+      ok = __all_sync(0xFFFFFFFFu, ok);
+      if (!ok) break;
       if (lane == 0) {
         const unsigned long long t = atomicAdd(a.item_counter, 1ull);
-        it = t < (unsigned long long)a.n_items ? (int64_t)t : -1;
-        item_ring[slot] = it;
-        mbar_arrive(&item_full[slot]);
+        if (t < (unsigned long long)a.n_items)
+          item_slot[k % kItemRing] = pf_item(a, (int64_t)t);
+        else
+          item_slot[k % kItemRing].nk = 0;
+        mbar_arrive(&item_full[k % kItemRing]);
       }
-      it = __shfl_sync(0xFFFFFFFFu, it, 0);
-      if (it < 0) break;
-      const PfItem w = pf_item(a, it);
-      for (int j = 0; j < w.nk; ++j, ++g) {
-        const int kt = pf_key_tile(it, j, w.nk);
-        const int st = (int)(g % NST);
-        if (g >= NST && !pf_wait(&empty_bar[st], (uint32_t)((g / NST) - 1) & 1, a, &abort_flag)) {
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
-          mbar_expect_tx(&full_bar[st], 2 * Cf::TILE);
-          const int y = (int)(w.row_base + (int64_t)kPfRows * kt);
-          const uint32_t kt = smem_addr(sm + Cf::KV_OFF + st * 2 * Cf::TILE);
-#pragma unroll
-          for (int u = 0; u < Cf::NSUB; ++u) {
-            tma_load_2d(kt + u * Cf::SUBB, &tm_k, u * SUB, y, &full_bar[st]);
-            tma_load_2d(kt + Cf::TILE + u * Cf::SUBB, &tm_v, u * SUB, y, &full_bar[st]);
-          }
-        }
-        // per-key mask bounds of the tile ((hid << 1) | is_cl; rows past the stored ones: invisible)
-        // sorted into the classes above; the causal part (i <= iq) is left to each query
+      __syncwarp();
+      const PfItem w = item_slot[k % kItemRing];
+      if (w.nk == 0) break;
+      const int own = w.own(KT), keys = w.keys(KT), before = w.before();
+      for (int j = 0; j < w.nk; ++j) {
+        const int v0 = KT * w.key_tile(j);
+        if (v0 + KT <= w.n_c) continue;  // rows that no span hides, all before the queries
+        const int cs = (int)(cg % kClsRing);
+        // per-key mask bounds of the tile ((hid << 1) | is_cl) sorted into the classes above; the causal
+        // part (i <= iq) is left to each query
         uint32_t ok_w[4];
-        bool none[4];
         int hp[4];  // the key's bound when it falls among the queries, else -3
 #pragma unroll
         for (int w4 = 0; w4 < 4; ++w4) {
-          const int c = lane + 32 * w4;
-          const int i = kPfRows * kt + c;
-          const int hid = (i < w.ps.len ? a.meta[w.ps.moff + i] : -2) >> 1;
-          none[w4] = i >= w.qr_end || hid < w.qr0;  // visible to no query of the tile
+          const int v = v0 + lane + 32 * w4;
+          int hid = w.qr_end;  // a row that no span hides
+          if (lane + 32 * w4 >= KT || v >= keys || (v >= before && v < own))
+            hid = -2;  // no key
+          else if (v >= own)
+            hid = a.meta[w.moff + w.qr0 + (v - own)] >> 1;
+          else if (v >= w.n_c)
+            hid = a.meta[w.moff + w.b0 + (v - w.n_c)] >> 1;
           ok_w[w4] = __ballot_sync(0xFFFFFFFFu, hid >= w.qr_end - 1);
           hp[w4] = hid >= w.qr0 && hid < w.qr_end - 1 ? hid : -3;
+        }
+        if (cg >= kClsRing && !pf_wait(&cls_empty[cs], ((cg / kClsRing) - 1) & 1, limit_ns)) {
+          ok = false;
+          break;
         }
         // runs: a listed key starts one unless key c - 1 is listed with the same bound, and ends one
         // unless key c + 1 is
@@ -492,78 +579,170 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           const uint32_t sb = __ballot_sync(0xFFFFFFFFu, start);
           const int rid = n_run + __popc(sb & ((2u << lane) - 1u)) - 1;  // runs started at or before c, less one
           if (start) {
-            rhid[st][rid] = hp[w4];
-            reinterpret_cast<uint16_t*>(&rcol[st][rid])[0] = (uint16_t)c;
+            rhid[cs][rid] = hp[w4];
+            rbits[cs][rid].x = (uint32_t)c;  // its columns [x, y), made into bits below
           }
-          if (end) reinterpret_cast<uint16_t*>(&rcol[st][rid])[1] = (uint16_t)(c + 1);
+          if (end) rbits[cs][rid].y = (uint32_t)(c + 1);
           n_run += __popc(sb);
         }
-        if (lane == 0) {
-          khid[st] = make_uint4(ok_w[0], ok_w[1], ok_w[2], ok_w[3]);
-          // per-key masking is needed when a key's visibility differs between the tile's queries
-          // (runs; keys at or past the first query: the causal rule, and a <CL> query sees only
-          // itself), or when the tile holds rows past the stored ones (their K may be anything)
-          kn[st] = n_run;
-          kslow[st] = n_run > 0 || kPfRows * (kt + 1) > w.ps.len || kPfRows * (kt + 1) > w.qr0;
-        }
-        // mask columns of the tile, 0 or a large negative number per key: column 0 for keys no query
-        // of the tile may see, column 1 for keys before the query tile (a <CL> query sees only itself)
-#pragma unroll
-        for (int w4 = 0; w4 < 4; ++w4) {
-          const int c = lane + 32 * w4;
-          const uint32_t neg = (uint32_t)T::r(-32768.f);
-          const uint32_t x01 = (none[w4] ? neg : 0u) | (kPfRows * kt + c < w.qr0 ? neg << 16 : 0u);
-          const uint32_t row = smem_addr(sm + Cf::XK_OFF + st * kPfRows * 32) + c * 32;
-          const uint32_t sw = (c >> 2) & 1;  // 32-byte swizzle: the two 16-byte halves swap every 4 rows
-          st_shared_v4(row + 16 * sw, x01, 0u, 0u, 0u);
-          st_shared_v4(row + 16 * (sw ^ 1), 0u, 0u, 0u, 0u);
-        }
-        fence_proxy_async_smem();
         __syncwarp();
-        mbar_arrive(&full_bar[st]);
+        for (int e = lane; e < n_run; e += 32) {
+          const int cb = (int)rbits[cs][e].x, ce = (int)rbits[cs][e].y;
+          rbits[cs][e] = make_uint4(low_bits(ce) & ~low_bits(cb), low_bits(ce - 32) & ~low_bits(cb - 32),
+                                    low_bits(ce - 64) & ~low_bits(cb - 64), low_bits(ce - 96) & ~low_bits(cb - 96));
+        }
+        __syncwarp();
+        if (lane == 0) {
+          khid[cs] = make_uint4(ok_w[0], ok_w[1], ok_w[2], ok_w[3]);
+          // per-key masking is needed when a key's visibility differs between the tile's queries: runs,
+          // and keys at or past the first query (the causal rule); and for columns without a key
+          kn[cs] = n_run;
+          kslow[cs] = n_run > 0 || v0 + KT > before;
+          mbar_arrive(&cls_full[cs]);
+        }
+        ++cg;
       }
     }
-    if (!ok && lane == 0) {
-      // let the copies already issued land before the CTA exits
-      for (int64_t t = g > NST ? g - NST : 0; t < g; ++t)
-        mbar_wait_bounded(&full_bar[t % NST], (uint32_t)(t / NST) & 1, 100000000ull);
+    // the last CTA to get here leaves the launch's counters at zero for the next launch
+    if (lane == 0) {
+      __threadfence();
+      if (atomicAdd(a.item_counter + 1, 1ull) + 1 == gridDim.x) {
+        a.item_counter[0] = 0;
+        a.item_counter[1] = 0;
+      }
+    }
+  } else if (warp >= 6) {
+    regs_other();
+    // ---------------- K (warp 6) and V (warp 7) tiles ----------------
+    constexpr int NS1 = Cf::NSUB >= 4 ? 4 : Cf::NSUB >= 2 ? 2 : 1;  // subtiles of one step of a gather
+    static_assert(Cf::NSUB - NS1 <= 1, "a gather's second pass takes one subtile");
+    const bool is_v = warp == 7;
+    const int nst = is_v ? VST : KST;
+    uint64_t* full = is_v ? v_full : k_full;
+    uint64_t* empty = is_v ? v_empty : k_empty;
+    const uint32_t ring = smem_addr(sm + (is_v ? Cf::V_OFF : Cf::K_OFF));
+    const CUtensorMap* tm = is_v ? &tm_v : &tm_k;
+    const uint16_t* plane = is_v ? a.v : a.k;
+    int st = 0;
+    uint32_t ph = 1, issued = 0;  // parity of the stage's previous release; tiles issued
+    uint32_t q_items = 0;         // items whose query rows were requested (warp 7)
+    for (uint32_t k = 0; ok; ++k) {
+      if (!(ok = item_wait(k))) break;
+      const PfItem w = item_slot[k % kItemRing];
+      item_done(k);
+      if (w.nk == 0) break;
+      if (is_v) {
+        // the item's query rows (past its last query another sequence's, or zeros past the last token: those
+        // rows' results go nowhere), once the Q.K^T of the item before are complete
+        if (k >= 1 && !(ok = pf_wait(&q_empty, (k - 1) & 1, limit_ns))) break;
+        if (lane == 0) {
+          mbar_arrive_expect_tx(&q_raw, Cf::QTILE);
+#pragma unroll
+          for (int u = 0; u < Cf::NSUB; ++u)
+            tma_load_3d(smem_addr(sm + Cf::Q_OFF) + u * Cf::QSUBB, &tm_q, u * SUB, w.h, w.tok0, &q_raw);
+        }
+        q_items = k + 1;
+      }
+      const int own = w.own(KT), keys = w.keys(KT), before = w.before();
+      const uint16_t* rows = plane + (int64_t)w.row_base * D;
+      for (int j = 0; j < w.nk; ++j) {
+        const int v0 = KT * w.key_tile(j), v1 = v0 + KT;
+        // rows side by side go in one copy: a tile of the list before its first gap, of the tile's own rows,
+        // or of all rows up to its last one
+        const bool in_list = v1 <= w.n_c && v1 <= w.vb, in_own = v0 >= own && v1 <= keys;
+        const bool tiled = in_list || in_own || (w.n_c == w.b0 && own == before && v1 <= keys);
+        int r0 = -1, r1 = -1, r2 = -1, r3 = -1;  // stored rows of keys v0 + 32 q + lane (-1: no key)
+        if (!tiled) {
+          auto key_row = [&](int v) -> int {
+            if (v < w.n_c) return v < w.vb ? v : __ldg(a.klist + w.moff + v);
+            if (v < before) return w.b0 + (v - w.n_c);
+            return v >= own && v < keys ? w.qr0 + (v - own) : -1;
+          };
+          r0 = key_row(v0 + lane);
+          r1 = key_row(v0 + 32 + lane);
+          if (KT > 64) r2 = key_row(v0 + 64 + lane);
+          if (KT > 96) r3 = key_row(v0 + 96 + lane);
+        }
+        if (issued >= (uint32_t)nst && !pf_wait(&empty[st], ph, limit_ns)) {
+          ok = false;
+          break;
+        }
+        const uint32_t dst = ring + st * Cf::TILE;
+        if (tiled) {
+          if (lane == 0) {
+            mbar_expect_tx(&full[st], Cf::TILE);
+            const int y = in_own ? w.row_base + w.qr0 + (v0 - own) : w.row_base + v0;
+#pragma unroll
+            for (int u = 0; u < Cf::NSUB; ++u) tma_load_2d(dst + u * Cf::SUBB, tm, u * SUB, y, &full[st]);
+          }
+          mbar_arrive(&full[st]);
+        } else {
+          // scattered rows
+#pragma unroll 1
+          for (int p0 = 0; p0 < KT; p0 += 32) {
+            gather_rows<D, SW, 0, NS1>(dst, Cf::SUBB, rows, r0, p0, KT, lane);
+            if constexpr (NS1 < Cf::NSUB) gather_rows<D, SW, NS1, 1>(dst, Cf::SUBB, rows, r0, p0, KT, lane);
+            r0 = r1;
+            r1 = r2;
+            r2 = r3;
+          }
+          cp_async_arrive(&full[st]);
+        }
+        ++issued;
+        if (++st == nst) {
+          st = 0;
+          ph ^= 1;
+        }
+      }
+      if (ok && !is_v && lane == 0) mbar_arrive(&item_last);
+    }
+    cp_async_wait_all_groups();
+    if (lane == 0) {
+      // no copy is in flight when the CTA exits
+      for (int n = issued < (uint32_t)nst ? (int)issued : nst; n > 0; --n) {
+        if (st == 0) {
+          st = nst;
+          ph ^= 1;
+        }
+        --st;
+        pf_wait(&full[st], ph ^ 1, limit_ns);
+      }
+      if (q_items > 0) pf_wait(&q_raw, (q_items - 1) & 1, limit_ns);
     }
   } else if (warp == 5) {
     regs_other();
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
-      constexpr uint32_t idS = mma_idesc(Pack16<T>::kType, 0, kPfRows, kPfRows);
+      constexpr uint32_t idS = mma_idesc(Pack16<T>::kType, 0, kPfRows, KT);
       constexpr uint32_t idO = mma_idesc(Pack16<T>::kType, 1, kPfRows, D);
       const uint32_t q_s = smem_addr(sm + Cf::Q_OFF);
       [[maybe_unused]] const uint32_t qlo_s = smem_addr(sm + Cf::QLO_OFF);
-      const uint32_t xq_s = smem_addr(sm + Cf::XQ_OFF), xk_s = smem_addr(sm + Cf::XK_OFF);
       int64_t g = 0;
-      bool ok = true;
       for (uint32_t k = 0; ok; ++k) {
-        const int slot = (int)(k % kItemRing);
-        if (!(ok = pf_wait(&item_full[slot], (k / kItemRing) & 1, a, &abort_flag))) break;
-        const int64_t it = item_ring[slot];
-        mbar_arrive(&item_empty[slot]);
-        if (it < 0) break;
-        const int nk = pf_item(a, it).nk;
-        ok = pf_wait(&q_full, k & 1, a, &abort_flag);
+        if (!(ok = item_wait(k))) break;
+        const int nk = item_slot[k % kItemRing].nk;
+        mbar_arrive(&item_empty[k % kItemRing]);
+        if (nk == 0) break;
+        ok = pf_wait(a.rot > 0 ? &q_full : &q_raw, k & 1, limit_ns);
         if (!ok) break;
         tc_fence_after();
         const uint32_t o_t = tmem + Cf::O_COL + (Cf::OBUF == 2 ? (k & 1) * D : 0);
         // S = Q K^T of tile gj into its S tile.  One S tile: once the softmax has read S of tile
         // gj - 1.  Two: the tile last held P of tile gj - 2, whose P.V was issued before (tcgen05.mma
         // from one thread run in issue order).
-        auto issue_qk = [&](int64_t gj) -> bool {
-          const int st = (int)(gj % NST), sb = (int)(gj % SBUF);
-          if (!pf_wait(&full_bar[st], (uint32_t)(gj / NST) & 1, a, &abort_flag)) return false;
-          if (Cf::PSEP && gj >= 1 && !pf_wait(&s_free, (uint32_t)(gj - 1) & 1, a, &abort_flag)) return false;
+        auto issue_qk = [&](int64_t gj, bool last) -> bool {
+          const int st = (int)(gj % KST), sb = (int)(gj % SBUF);
+          if (!pf_wait(&k_full[st], (uint32_t)(gj / KST) & 1, limit_ns)) return false;
+          if (Cf::PSEP && gj >= 1 && !pf_wait(&s_free, (uint32_t)(gj - 1) & 1, limit_ns)) return false;
+          fence_proxy_async_smem();  // gathered rows were written through the generic proxy
           tc_fence_after();
-          const uint32_t k_s = smem_addr(sm + Cf::KV_OFF + st * 2 * Cf::TILE);
+          const uint32_t k_s = smem_addr(sm + Cf::K_OFF + st * Cf::TILE);
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
             const uint32_t off = (kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2;
-            tc_mma(tmem + sb * kPfRows, smem_desc(q_s + off, 16, 8 * SW, SW), smem_desc(k_s + off, 16, 8 * SW, SW),
-                   idS, kk > 0);
+            const uint32_t qoff = (kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2;
+            tc_mma(tmem + sb * KT, smem_desc(q_s + qoff, 16, 8 * SW, SW), smem_desc(k_s + off, 16, 8 * SW, SW), idS,
+                   kk > 0);
           }
           // SPLIT with RoPE: + Q_lo K^T (without RoPE the query is exact in the cache type)
           if constexpr (Cf::SPLIT) {
@@ -571,41 +750,39 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
 #pragma unroll
               for (int kk = 0; kk < D / 16; ++kk) {
                 const uint32_t off = (kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2;
+                [[maybe_unused]] const uint32_t qoff = (kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2;
                 if constexpr (Cf::QLO_TMEM)
-                  tc_mma_ts(tmem + sb * kPfRows, tmem + Cf::QLO_COL + 8 * kk, smem_desc(k_s + off, 16, 8 * SW, SW),
-                            idS, 1);
+                  tc_mma_ts(tmem + sb * KT, tmem + Cf::QLO_COL + 8 * kk, smem_desc(k_s + off, 16, 8 * SW, SW), idS, 1);
                 else
-                  tc_mma(tmem + sb * kPfRows, smem_desc(qlo_s + off, 16, 8 * SW, SW),
-                         smem_desc(k_s + off, 16, 8 * SW, SW), idS, 1);
+                  tc_mma(tmem + sb * KT, smem_desc(qlo_s + qoff, 16, 8 * SW, SW), smem_desc(k_s + off, 16, 8 * SW, SW),
+                         idS, 1);
               }
             }
           }
-          // + the mask column: 256 x (0 or -32768) per key
-          if constexpr (Cf::XQT)
-            tc_mma_ts(tmem + sb * kPfRows, tmem + Cf::XQ_COL, smem_desc(xk_s + st * kPfRows * 32, 16, 8 * 32, 32), idS, 1);
-          else
-            tc_mma(tmem + sb * kPfRows, smem_desc(xq_s, 16, 8 * 32, 32),
-                   smem_desc(xk_s + st * kPfRows * 32, 16, 8 * 32, 32), idS, 1);
           tc_commit(&s_full[sb]);
+          tc_commit(&k_empty[st]);
+          if (last) tc_commit(&q_empty);
           return true;
         };
         // O += P V of tile gp (8 TMEM columns of P per 16 keys); the first of an item: O = P V
         auto issue_pv = [&](int64_t gp, bool first) -> bool {
-          const int st = (int)(gp % NST);
-          if (!pf_wait(&p_full, (uint32_t)gp & 1, a, &abort_flag)) return false;
+          const int st = (int)(gp % VST);
+          if (!pf_wait(&v_full[st], (uint32_t)(gp / VST) & 1, limit_ns)) return false;
+          if (!pf_wait(&p_full, (uint32_t)gp & 1, limit_ns)) return false;
+          fence_proxy_async_smem();
           tc_fence_after();
-          const uint32_t v_s = smem_addr(sm + Cf::KV_OFF + st * 2 * Cf::TILE + Cf::TILE);
-          const uint32_t p_t = tmem + (Cf::PSEP ? Cf::P_COL : (uint32_t)(gp % SBUF) * kPfRows);
+          const uint32_t v_s = smem_addr(sm + Cf::V_OFF + st * Cf::TILE);
+          const uint32_t p_t = tmem + (Cf::PSEP ? Cf::P_COL : (uint32_t)(gp % SBUF) * KT);
 #pragma unroll
-          for (int kk = 0; kk < kPfRows / 16; ++kk)
+          for (int kk = 0; kk < KT / 16; ++kk)
             tc_mma_ts(o_t, p_t + 8 * kk, smem_desc(v_s + kk * 16 * SW, Cf::SUBB, 8 * SW, SW), idO, (!first || kk > 0));
           if constexpr (Cf::SPLIT) {  // + P_lo V
 #pragma unroll
-            for (int kk = 0; kk < kPfRows / 16; ++kk)
+            for (int kk = 0; kk < KT / 16; ++kk)
               tc_mma_ts(o_t, p_t + Cf::PLO_COL + 8 * kk, smem_desc(v_s + kk * 16 * SW, Cf::SUBB, 8 * SW, SW), idO, 1);
           }
           tc_commit(&pv_done);
-          tc_commit(&empty_bar[st]);
+          tc_commit(&v_empty[st]);
           return true;
         };
         // Q K^T of the next tile goes in ahead of P.V of the current one: it runs while the softmax
@@ -613,9 +790,9 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         for (int j = 0; ok && j <= nk; ++j) {
           if (SBUF == 1 && !Cf::PSEP) {  // P sits in the one S tile: its P.V before the next Q K^T
             if (j >= 1) ok = issue_pv(g + j - 1, j == 1);
-            if (ok && j < nk) ok = issue_qk(g + j);
+            if (ok && j < nk) ok = issue_qk(g + j, j == nk - 1);
           } else {
-            if (j < nk) ok = issue_qk(g + j);
+            if (j < nk) ok = issue_qk(g + j, j == nk - 1);
             if (ok && j >= 1) ok = issue_pv(g + j - 1, j == 1);
           }
         }
@@ -623,37 +800,22 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       }
       // every MMA issued above has completed once this phase does
       tc_commit(&drain);
-      mbar_wait_bounded(&drain, 0, a.wait_limit_ns);
+      pf_wait(&drain, 0, limit_ns);
     }
   } else if (warp < 4) {
     if constexpr (Cf::CPS == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Cf::REG_SOFTMAX));
     // ---------------- softmax: one thread per query row ----------------
-    constexpr int CW = kPfRows;  // S columns of one thread
-    constexpr int NSM = 128;     // softmax threads (named barrier 1)
+    constexpr int CW = KT;           // S columns of one thread
     const int r = warp * 32 + lane;  // tile row == TMEM lane
     const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
     const float c2 = a.c2;
-    // The query rows of item w into the K-major Q tile (row r per thread), in two halves: q_issue
-    // starts 16-byte asynchronous copies of the raw row into its swizzled slots (no registers, so
-    // they can be issued early, while the previous item's last tile is still in the softmax);
-    // q_finish waits for them, rotates the row in place for RoPE (pairs (e, e + rot/2), at the
-    // query's position, rounded to the cache type), writes the row's mask columns (256 in column 0;
-    // 256 in column 1 for a <CL> query, which the keys before the query tile then mask) and
-    // releases the tile to the MMA thread.
+    // RoPE: row r of the K-major Q tile, rotated in place (pairs (e, e + rot/2), at the query's position,
+    // rounded to the cache type) once item kk's raw rows are in, and released to the MMA thread.
     auto q_chunk = [&](int c8) -> uint32_t {  // shared address of 8-column chunk c8 of row r
       const int e0 = c8 * 8;
       const int u = e0 / SUB, cw = (e0 % SUB) / 8;
       const int phys = cw ^ ((r * SW >> 7) & (SW / 16 - 1));
-      return smem_addr(sm + Cf::Q_OFF) + u * Cf::SUBB + r * SW + phys * 16;
-    };
-    auto q_issue = [&](const PfItem& w) {
-      const int iq = w.qr0 + r;
-      const bool valid = iq < w.qr_end;
-      const int64_t row = valid ? ((int64_t)(w.ps.qtok + (iq - w.ps.q0)) * a.H + w.h) * D : 0;
-#pragma unroll
-      for (int c8 = 0; c8 < D / 8; ++c8) cp_async16(q_chunk(c8), a.q + row + 8 * c8, valid ? 16u : 0u);
-      cp_async4(smem_addr(&qmeta[r]), a.meta + (valid ? w.ps.moff + iq : 0), valid ? 4u : 0u);
-      cp_async_commit();
+      return smem_addr(sm + Cf::Q_OFF) + u * Cf::QSUBB + r * SW + phys * 16;
     };
     // SPLIT: the address of chunk c8 of row r in the query's low-part tile (QLO_SMEM)
     [[maybe_unused]] auto qlo_chunk = [&](int c8) -> uint32_t {
@@ -665,8 +827,8 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       else
         st_shared_v4(qlo_chunk(c8), w0, w1, w2, w3);
     };
-    auto q_finish = [&](const PfItem& w) {
-      cp_async_wait_all();
+    auto q_rotate = [&](const PfItem& w, uint32_t kk) -> bool {
+      if (!__all_sync(0xFFFFFFFFu, pf_wait(&q_raw, kk & 1, limit_ns))) return false;
       const int half = a.rot / 2;
       const int iq = w.qr0 + r;
       if constexpr (Cf::SPLIT) {
@@ -674,7 +836,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         if (half > 0) {
           const int32_t qpos = iq < w.qr_end ? a.pos[a.off[w.s] + iq] : 0;
           const int hc = half / 8;  // chunks per rotated half
-#pragma unroll
+#pragma unroll 1
           for (int c8 = 0; c8 < D / 16; ++c8) {
             if (c8 < hc) {
               const uint32_t a1 = q_chunk(c8), a2 = q_chunk(c8 + hc);
@@ -697,177 +859,254 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
             }
           }
           // the dimensions past the rotary ones are exact: their low part is zero
-#pragma unroll
+#pragma unroll 1
           for (int c8 = 0; c8 < D / 8; ++c8)
             if (c8 >= 2 * hc) qlo_store(c8, 0u, 0u, 0u, 0u);
         }
       } else if (half > 0 && iq < w.qr_end) {
         const int32_t qpos = a.pos[a.off[w.s] + iq];
+#pragma unroll 1
         for (int c8 = 0; c8 < half / 8; ++c8) {
           const uint32_t a1 = q_chunk(c8), a2 = q_chunk(c8 + half / 8);
-          const uint4 u1 = ld_shared_v4(a1), u2 = ld_shared_v4(a2);
-          const uint32_t w1[4] = {u1.x, u1.y, u1.z, u1.w}, w2[4] = {u2.x, u2.y, u2.z, u2.w};
-          uint32_t o1[4], o2[4];
-#pragma unroll
+#pragma unroll 2
           for (int e = 0; e < 4; ++e) {
-            const float2 x1 = T::f2(w1[e]), x2 = T::f2(w2[e]);
+            const float2 x1 = T::f2(ld_shared_u32(a1 + 4 * e)), x2 = T::f2(ld_shared_u32(a2 + 4 * e));
             float sn0, cs0, sn1, cs1;
             rope_sincos(qpos, a.rope_g[8 * c8 + 2 * e], &sn0, &cs0);
             rope_sincos(qpos, a.rope_g[8 * c8 + 2 * e + 1], &sn1, &cs1);
-            o1[e] = Pack16<T>::two(x1.x * cs0 - x2.x * sn0, x1.y * cs1 - x2.y * sn1);
-            o2[e] = Pack16<T>::two(x2.x * cs0 + x1.x * sn0, x2.y * cs1 + x1.y * sn1);
+            st_shared_u32(a1 + 4 * e, Pack16<T>::two(x1.x * cs0 - x2.x * sn0, x1.y * cs1 - x2.y * sn1));
+            st_shared_u32(a2 + 4 * e, Pack16<T>::two(x2.x * cs0 + x1.x * sn0, x2.y * cs1 + x1.y * sn1));
           }
-          st_shared_v4(a1, o1[0], o1[1], o1[2], o1[3]);
-          st_shared_v4(a2, o2[0], o2[1], o2[2], o2[3]);
         }
       }
-      const uint32_t x01 = (uint32_t)T::r(256.f) | (qmeta[r] & 1 ? (uint32_t)T::r(256.f) << 16 : 0u);
-      if constexpr (Cf::XQT) {
-        const uint32_t wd[8] = {x01, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        tmem_st8u(tl + Cf::XQ_COL, wd);
-        tmem_wait_st();  // also the query's low part (QLO_TMEM)
+      if constexpr (Cf::QLO_TMEM) {
+        tmem_wait_st();  // the query's low part
         tc_fence_before();
-      } else {
-        const uint32_t row = smem_addr(sm + Cf::XQ_OFF) + r * 32;
-        const uint32_t sw = (r >> 2) & 1;  // 32-byte swizzle: the two 16-byte halves swap every 4 rows
-        st_shared_v4(row + 16 * sw, x01, 0u, 0u, 0u);
-        st_shared_v4(row + 16 * (sw ^ 1), 0u, 0u, 0u, 0u);
       }
       fence_proxy_async_smem();
       mbar_arrive(&q_full);
+      return true;
+    };
+    // the item's row r is a <CL> query
+    auto is_cl = [&](const PfItem& w) -> bool {
+      return w.qr0 + r < w.qr_end && (__ldg(a.meta + w.moff + w.qr0 + r) & 1);
     };
 
-    // the CTA's kk-th item from the ring (-1: none left, -2: the wait gave up); each softmax warp
-    // reads it once and releases the slot
-    auto take = [&](uint32_t kk) -> int64_t {
-      const int slot = (int)(kk % kItemRing);
-      if (!pf_wait(&item_full[slot], (kk / kItemRing) & 1, a, &abort_flag)) return -2;
-      const int64_t v = item_ring[slot];
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&item_empty[slot]);
-      return v;
+    int64_t g = 0;    // tiles consumed
+    uint32_t k = 0;   // items done
+    uint32_t cg = 0;  // sorted key tiles consumed
+    // waits of a whole warp
+    auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+      return __all_sync(0xFFFFFFFFu, pf_wait(bar, parity, limit_ns));
     };
-    bool ok = true;
-    int64_t g = 0;  // tiles consumed
-    uint32_t k = 0;  // items done
-    int64_t it = take(0);
-    PfItem w{};
-    if (it >= 0) {
-      w = pf_item(a, it);
-      q_issue(w);
-      q_finish(w);
+    // Epilogue of item kk (row sum l_): O / l, 16 columns at a time.  A full tile goes out through each
+    // warp's swizzled buffers in turn as TMA tensor stores of box (16 columns, head h, 32 tokens); else
+    // each thread stores its query's row.
+    auto epilogue = [&](uint32_t kk, float l_) {
+      const PfItem& w = item_slot[kk % kItemRing];
+      const uint32_t o_t = tl + Cf::O_COL + (Cf::OBUF == 2 ? (kk & 1) * D : 0);
+      const bool staged = Cf::OSTAGE && w.qr_end - w.qr0 == kPfRows;
+      const bool valid = w.qr0 + r < w.qr_end;
+      const float inv = 1.f / l_;
+      uint32_t buf = smem_addr(sm + Cf::OST_OFF + warp * Cf::OST_N * Cf::OST_BUF);
+      const uint32_t buf_end = buf + Cf::OST_N * Cf::OST_BUF;
+      float* orow = a.out + ((int64_t)(w.tok0 + r) * a.H + w.h) * D;
+#pragma unroll 1
+      for (int u = 0; u < D / 16; ++u) {
+        float o[16];
+        tmem_ld16(o_t + 16 * u, o);
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) o[e] *= inv;
+        if (staged) {
+          if (lane == 0) {  // the buffer's last store has read it
+            if (u == 0)
+              bulk_wait_read<0>();
+            else
+              bulk_wait_read<Cf::OST_N - 1>();
+          }
+          __syncwarp();
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            st_shared_v4(buf + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), __float_as_uint(o[4 * c]),
+                         __float_as_uint(o[4 * c + 1]), __float_as_uint(o[4 * c + 2]), __float_as_uint(o[4 * c + 3]));
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            tma_store_3d(&tm_o, buf, 16 * u, w.h, w.tok0 + 32 * warp);
+            bulk_commit();
+          }
+          buf += Cf::OST_BUF;
+          if (buf == buf_end) buf -= Cf::OST_N * Cf::OST_BUF;
+        } else if (valid) {
+#pragma unroll
+          for (int e = 0; e < 16; e += 4)
+            *reinterpret_cast<float4*>(orow + 16 * u + e) = make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
+        }
+      }
+      tc_fence_before();
+      item_done(kk);
+    };
+    ok = __all_sync(0xFFFFFFFFu, item_wait(0));
+    bool more = ok && item_slot[0].nk > 0;
+    bool cl_next = false;  // is_cl of the next item
+    float l_prev = 0.f;    // the item before's row sum: its epilogue comes once its last P.V is complete
+    if (more) {
+      cl_next = is_cl(item_slot[0]);
+      if (a.rot > 0) ok = q_rotate(item_slot[0], 0);
     }
-    while (it >= 0) {
-      int64_t it_next = -1;  // the next item, taken at this item's last tile
-      const int iq = w.qr0 + r;  // stored row of this query
-      const bool valid = iq < w.qr_end;
-      const bool cl_q = valid && (qmeta[r] & 1);
+    // after the last item (!more) once more, for its epilogue alone
+    while (ok && (more || k >= 1)) {
+      const PfItem& w = item_slot[k % kItemRing];
+      const int nk = more ? w.nk : 1, n_c = w.n_c;
+      const int iq = w.qr0 + r;      // stored row of this query
+      const int vq = w.own(KT) + r;  // its own key
+      const bool cl_q = cl_next;
+      bool next_ok = false;  // there is another item
       const uint32_t o_t = tl + Cf::O_COL + (Cf::OBUF == 2 ? (k & 1) * D : 0);
       float m = -INFINITY, l = 0.f;
-      for (int j = 0; j < w.nk; ++j) {
+      for (int j = 0; j < nk; ++j) {
         const int64_t gj = g + j;
-        const int sb = (int)(gj % SBUF), st = (int)(gj % NST);
-        // the S tile, and (acquired from the producer directly) the stage's mask bounds; the stage's
-        // barrier cannot move to its next phase before this thread releases P of this tile
-        ok = ok && pf_wait(&s_full[sb], (uint32_t)(gj / SBUF) & 1, a, &abort_flag) &&
-             pf_wait(&full_bar[st], (uint32_t)(gj / NST) & 1, a, &abort_flag);
-        const bool wok = __all_sync(0xFFFFFFFFu, ok);  // tcgen05.ld / st are warp-collective
-        float sv[CW];
-        if (wok) {
+        const int sb = (int)(gj % SBUF);
+        const uint32_t p_tl = tl + (Cf::PSEP ? Cf::P_COL : sb * KT);
+        float sv[CW], alpha = 1.f, ref = 0.f, m_new = 0.f;
+        float2 rs4[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        uint32_t pk[2][16];
+        [[maybe_unused]] uint32_t pl[2][16];
+        // P = 2^(s c2 - ref) of columns [32 q, 32 q + 32) (or their first 16) as 16-bit pairs; the row sum
+        auto make_p = [&](int q) {
+          const float2 c2v = make_float2(c2, c2), nref = make_float2(-ref, -ref);
+#pragma unroll
+          for (int c = 0; c < 32; c += 2) {
+            if (32 * q + c >= CW) continue;
+            const float2 x = __ffma2_rn(make_float2(sv[32 * q + c], sv[32 * q + c + 1]), c2v, nref);
+            const float2 p = make_float2(ex2(x.x), ex2(x.y));
+            rs4[(c >> 1) & 3] = __fadd2_rn(rs4[(c >> 1) & 3], p);
+            if constexpr (Cf::SPLIT)
+              pl[q & 1][c / 2] = bf16_split2(p, &pk[q & 1][c / 2]);
+            else
+              pk[q & 1][c / 2] = Pack16<T>::two(p.x, p.y);
+          }
+        };
+        auto store_p = [&](int q) {  // into row r's lane
+          if (CW - 32 * q >= 32)
+            tmem_st16u(p_tl + 16 * q, pk[q & 1]);
+          else
+            tmem_st8u(p_tl + 16 * q, pk[q & 1]);
+          if constexpr (Cf::SPLIT) tmem_st16u(p_tl + Cf::PLO_COL + 16 * q, pl[q & 1]);
+        };
+        // pv_done phases are consumed one by one, each while it is the only one that can be pending
+        // (the next P.V waits for this tile's P): phase gj - 1 during tile gj, before O is rescaled and
+        // before this tile's P is written where P.V of the tile before reads its P from.  The wait comes as
+        // late as that allows: with P in columns of its own after the first 64 columns of P are made, with
+        // two S tiles (P goes into its own) at the end.  An item's first tile then runs the epilogue of
+        // the item before, whose last P.V that was.
+        bool pv_wait = gj >= 1;
+        if (more) {
+          const int v0 = KT * w.key_tile(j);    // the tile's first key
+          const bool sorted = v0 + KT > n_c;    // warp 4 has sorted its keys
+          const int cs = (int)(cg % kClsRing);
+          ok = warp_wait(&s_full[sb], (uint32_t)(gj / SBUF) & 1) &&
+               (!sorted || warp_wait(&cls_full[cs], (cg / kClsRing) & 1));
+          // warp 4 takes the next item as soon as this item's last K tile is on its way
+          if (ok && j == nk - 1) ok = __all_sync(0xFFFFFFFFu, item_wait(k + 1));
+          // nothing is exchanged between the softmax warps: each stops by itself
+          if (!ok) break;
           tc_fence_after();
 #pragma unroll
-          for (int c = 0; c < CW; c += 32) tmem_ld32(tl + sb * kPfRows + c, sv + c);
-          tmem_wait_ld();
-          tc_fence_before();
-        } else {
-#pragma unroll
-          for (int c = 0; c < CW; ++c) sv[c] = 0.f;
-        }
-        if (Cf::PSEP) mbar_arrive(&s_free);  // the next Q K^T may overwrite S
-        // S of the item's last tile is in: every Q K^T of the item is complete, the next item's
-        // queries may go into the Q tile (the producer has taken that item by now: it takes the
-        // next one as soon as it has issued this item's last tile)
-        if (j == w.nk - 1) {
-          it_next = take(k + 1);
-          if (it_next == -2) ok = false;
-          if (it_next >= 0) {
-            const PfItem nx = pf_item(a, it_next);
-            q_issue(nx);
-            if (lane == 0) next_item = nx;  // every warp writes the same item
-          }
-        }
-        const int kb = kPfRows * pf_key_tile(it, j, w.nk);
-        if (kslow[st]) {
-          // visibility of the tile's keys to this query as four 32-bit words: the causal prefix (key
-          // row <= iq) with the tile-wide bound words plus the runs whose bound admits iq.  Other
-          // tiles are masked by their mask columns alone.
-          const int t = iq - kb;  // last visible column
-          const uint4 hw = khid[st];
-          uint32_t v0 = hw.x, v1 = hw.y, v2 = hw.z, v3 = hw.w;
-          const int nr = kn[st];
-          for (int e = 0; e < nr; ++e) {
-            if (rhid[st][e] >= iq) {
-              const uint32_t cc = rcol[st][e];
-              const int cb = (int)(cc & 0xFFFFu), ce = (int)(cc >> 16);
-              v0 |= low_bits(ce) & ~low_bits(cb);
-              v1 |= low_bits(ce - 32) & ~low_bits(cb - 32);
-              v2 |= low_bits(ce - 64) & ~low_bits(cb - 64);
-              v3 |= low_bits(ce - 96) & ~low_bits(cb - 96);
+          for (int c = 0; c + 32 <= CW; c += 32) tmem_ld32(tl + sb * KT + c, sv + c);
+          if constexpr (CW % 32 == 16) tmem_ld16(tl + sb * KT + CW - 16, sv + CW - 16);
+          const bool slow = sorted && kslow[cs] != 0;
+          uint32_t vw[4];
+          if (slow) {
+            // visibility of the tile's keys to this query as 32-bit words: the causal prefix (keys up to the
+            // query's own) with the tile-wide bound words plus the runs whose bound admits iq.  Every key of
+            // the other tiles is visible (to all but a <CL> query).
+            const int t = vq - v0;  // the query's own column, the last visible one
+            const uint4 hw = khid[cs];
+            vw[0] = hw.x;
+            vw[1] = hw.y;
+            vw[2] = hw.z;
+            vw[3] = hw.w;
+            const int nr = kn[cs];
+#pragma unroll 1
+            for (int e = 0; e < nr; ++e) {
+              const uint4 rb = rbits[cs][e];
+              const uint32_t on = rhid[cs][e] >= iq ? 0xFFFFFFFFu : 0u;
+              vw[0] |= rb.x & on;
+              vw[1] |= rb.y & on;
+              vw[2] |= rb.z & on;
+              vw[3] |= rb.w & on;
             }
+            // the causal prefix; a <CL> query sees its own key alone
+#pragma unroll
+            for (int u = 0; u < 4; ++u) vw[u] &= low_bits(t + 1 - 32 * u) & ~low_bits(cl_q ? t - 32 * u : 0);
           }
-          // the causal prefix; a <CL> query sees its own key alone
-          const int t1 = t + 1, t0 = cl_q ? t : 0;
-          v0 &= low_bits(t1) & ~low_bits(t0);
-          v1 &= low_bits(t1 - 32) & ~low_bits(t0 - 32);
-          v2 &= low_bits(t1 - 64) & ~low_bits(t0 - 64);
-          v3 &= low_bits(t1 - 96) & ~low_bits(t0 - 96);
-          const uint32_t vw[4] = {v0, v1, v2, v3};
+          if (j == nk - 1) {
+            next_ok = item_slot[(k + 1) % kItemRing].nk > 0;
+            cl_next = next_ok && is_cl(item_slot[(k + 1) % kItemRing]);
+          }
+          tmem_wait_ld();
 #pragma unroll
-          for (int c = 0; c < CW; ++c) sv[c] = (vw[c >> 5] >> (c & 31)) & 1u ? sv[c] : -INFINITY;
-        }
-        // row max: a tree (eight partial maxima: columns 0-7, then pairs of 8-column blocks, then the
-        // last block when one is left over)
-        static_assert(CW % 8 == 0, "slice width");
-        constexpr int kPairEnd = 8 + (CW - 8) / 16 * 16;  // columns [8, kPairEnd) go in pairs of blocks
-        float mx8[8];
+          for (int c = 0; c < CW; ++c) asm volatile("" : "+f"(sv[c]));  // no use of S moves above the wait
+          tc_fence_before();
+          if (Cf::PSEP) mbar_arrive(&s_free);  // the next Q K^T may overwrite S
+          if (sorted) {
+            __syncwarp();  // every lane has read the tile's classes
+            if (lane == 0) mbar_arrive(&cls_empty[cs]);
+            ++cg;
+          }
+          // A <CL> query sees none of the keys of a tile without the per-key rule: an infinite reference makes
+          // its P there 0.  Only if one of those scores is not below infinity the row is masked as well, in a
+          // second round.
+          const bool unseen = cl_q && !slow;
+          bool masked = slow;
+          float mx;
+          // row max: a tree (eight partial maxima: columns 0-7, then pairs of 8-column blocks, then the
+          // last block when one is left over)
+          static_assert(CW % 8 == 0, "slice width");
+          constexpr int kPairEnd = 8 + (CW - 8) / 16 * 16;  // columns [8, kPairEnd) go in pairs of blocks
+          for (;;) {
+            if (masked) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) mx8[u] = sv[u];
+              for (int u = 0; u < (CW + 31) / 32; ++u) {
+                if (!__any_sync(0xFFFFFFFFu, vw[u] != 0xFFFFFFFFu)) continue;  // visible to the whole warp
 #pragma unroll
-        for (int c = 8; c < kPairEnd; c += 16)
+                for (int c = 32 * u; c < 32 * u + 32; ++c)
+                  if (c < CW) sv[c] = vw[u] & (1u << (c & 31)) ? sv[c] : -INFINITY;
+              }
+            }
+            float mx8[8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) mx8[u] = max3(mx8[u], sv[c + u], sv[c + 8 + u]);
-        if constexpr (kPairEnd < CW) {
+            for (int u = 0; u < 8; ++u) mx8[u] = sv[u];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) mx8[u] = fmaxf(mx8[u], sv[kPairEnd + u]);
-        }
-        const float mx = max3(max3(mx8[0], mx8[1], mx8[2]), max3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
-        if (!__all_sync(0xFFFFFFFFu, ok)) {
-          // no exchange between the warps, so no barrier inside the tile loop -- a warp that stops
-          // here meets the others at the barrier after the loop (their bounded waits give up at once
-          // once any role has given up)
-          ok = false;
-          break;
-        }
-        // Reference maximum: moved only when the row maximum grows by more than 2^8 (log2 units), so
-        // O is rescaled rarely; P stays below 2^8 and its scale cancels exactly in O / l.
-        const float cand = mx * c2;
-        const bool move = cand > m + 8.f;
-        const float m_new = move ? cand : m;
-        const float ref = m_new == -INFINITY ? 0.f : m_new;
-        const float alpha = !move ? 1.f : (m == -INFINITY ? 0.f : ex2(m - ref));
-        // pv_done phases are consumed one by one, each while it is the only one that can be pending
-        // (the next P.V waits for this tile's P): phase gj - 1 during tile j >= 1, before this
-        // tile's P is written (P.V of the previous tile has read its P) and before O is rescaled;
-        // an item's last phase in its epilogue.
-        // (With two S tiles, P goes into its own S tile, so the wait can come last unless O needs
-        // the rescale.)
-        bool pv_early = j >= 1;
-        if constexpr (SBUF == 2) pv_early = j >= 1 && __any_sync(0xFFFFFFFFu, alpha != 1.f);
-        if (pv_early) {
-          ok = pf_wait(&pv_done, (uint32_t)(gj - 1) & 1, a, &abort_flag) && ok;
-          if (__all_sync(0xFFFFFFFFu, ok) && __any_sync(0xFFFFFFFFu, alpha != 1.f)) {
+            for (int c = 8; c < kPairEnd; c += 16)
+#pragma unroll
+              for (int u = 0; u < 8; ++u) mx8[u] = max3(mx8[u], sv[c + u], sv[c + 8 + u]);
+            if constexpr (kPairEnd < CW) {
+#pragma unroll
+              for (int u = 0; u < 8; ++u) mx8[u] = max3(mx8[u], sv[kPairEnd + u], sv[kPairEnd + u]);
+            }
+            mx = max3(max3(mx8[0], mx8[1], mx8[2]), max3(mx8[3], mx8[4], mx8[5]), max3(mx8[6], mx8[7], mx8[7]));
+            masked = __any_sync(0xFFFFFFFFu, unseen && !(mx < INFINITY));
+            if (!masked) break;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) vw[u] = unseen ? 0u : 0xFFFFFFFFu;
+          }
+          // Reference maximum: moved only when the row maximum grows by more than 2^8 (log2 units), so
+          // O is rescaled rarely; P stays below 2^8 and its scale cancels exactly in O / l.
+          const float cand = unseen ? -INFINITY : mx * c2;
+          const bool move = cand > m + 8.f;
+          m_new = move ? cand : m;
+          ref = unseen ? INFINITY : m_new == -INFINITY ? 0.f : m_new;
+          // a row that has seen no key so far has O = 0 and l = 0: nothing to rescale
+          alpha = !move || m == -INFINITY ? 1.f : ex2(m - ref);
+          if (pv_wait && __any_sync(0xFFFFFFFFu, alpha != 1.f)) {
+            pv_wait = false;
+            ok = warp_wait(&pv_done, (uint32_t)(gj - 1) & 1);
+            if (!ok) break;
             tc_fence_after();
-#pragma unroll
+#pragma unroll 1
             for (int u = 0; u < D / 16; ++u) {
               float o[16];
               tmem_ld16(o_t + 16 * u, o);
@@ -877,152 +1116,53 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
               tmem_st16(o_t + 16 * u, o);
             }
           }
-        }
-        // P = 2^(s c2 - ref) as 16-bit pairs (row r in lane r), stored 32 columns at a time as they
-        // are made; the row sum
-        const uint32_t p_tl = tl + (Cf::PSEP ? Cf::P_COL : sb * kPfRows);
-        float2 rs4[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-        const float2 c2v = make_float2(c2, c2), nref = make_float2(-ref, -ref);
-        const bool sok = __all_sync(0xFFFFFFFFu, ok);
-        if (sok) tc_fence_after();
+          make_p(0);
+          if (!Cf::PSEP) store_p(0);
+          make_p(1);
+          if (!Cf::PSEP) {
+            store_p(1);
 #pragma unroll
-        for (int q = 0; q < CW / 32; ++q) {
-          uint32_t pk[16];
-          [[maybe_unused]] uint32_t pl[16];
-#pragma unroll
-          for (int c = 0; c < 32; c += 2) {
-            const float2 x = __ffma2_rn(make_float2(sv[32 * q + c], sv[32 * q + c + 1]), c2v, nref);
-            const float2 p = make_float2(ex2(x.x), ex2(x.y));
-            rs4[(c >> 1) & 3] = __fadd2_rn(rs4[(c >> 1) & 3], p);
-            if constexpr (Cf::SPLIT)
-              pl[c / 2] = bf16_split2(p, &pk[c / 2]);
-            else
-              pk[c / 2] = Pack16<T>::two(p.x, p.y);
-          }
-          if (sok) tmem_st16u(p_tl + 16 * q, pk);
-          if constexpr (Cf::SPLIT) {
-            if (sok) tmem_st16u(p_tl + Cf::PLO_COL + 16 * q, pl);
+            for (int q = 2; q < (CW + 31) / 32; ++q) {
+              make_p(q);
+              store_p(q);
+            }
           }
         }
-        const float rs = ((rs4[0].x + rs4[0].y) + (rs4[1].x + rs4[1].y)) + ((rs4[2].x + rs4[2].y) + (rs4[3].x + rs4[3].y));
+        if (pv_wait) {
+          ok = warp_wait(&pv_done, (uint32_t)(gj - 1) & 1);
+          if (!ok) break;
+        }
+        tc_fence_after();
+        if (j == 0 && k >= 1) epilogue(k - 1, l_prev);
+        if (!more) break;
+        if (Cf::PSEP) {
+          store_p(0);
+          store_p(1);
+#pragma unroll
+          for (int q = 2; q < (CW + 31) / 32; ++q) {
+            make_p(q);
+            store_p(q);
+          }
+        }
+        const float rs =
+            ((rs4[0].x + rs4[0].y) + (rs4[1].x + rs4[1].y)) + ((rs4[2].x + rs4[2].y) + (rs4[3].x + rs4[3].y));
         l = l * alpha + rs;
         tmem_wait_st();
-        if (kb + kPfRows > w.ps.len && kb + r >= w.ps.len) {
-          // a V row past the stored rows (stale or another stream's): zero it so 0 * V stays 0
-          const uint32_t v_row = smem_addr(sm + Cf::KV_OFF + st * 2 * Cf::TILE + Cf::TILE) + r * SW;
-#pragma unroll
-          for (int u = 0; u < Cf::NSUB; ++u)
-#pragma unroll
-            for (int b16 = 0; b16 < SW / 16; ++b16) st_shared_v4(v_row + u * Cf::SUBB + b16 * 16, 0, 0, 0, 0);
-          fence_proxy_async_smem();
-        }
-        if constexpr (SBUF == 2) {
-          if (j >= 1 && !pv_early) ok = pf_wait(&pv_done, (uint32_t)(gj - 1) & 1, a, &abort_flag) && ok;
-        }
         tc_fence_before();
         mbar_arrive(&p_full);
         m = m_new;
       }
-      // a wait that ran out after the tile loop's last barrier: decided by every thread together
-      if (!bar_and(1, NSM, ok)) {
-        ok = false;
-        break;
-      }
-      g += w.nk;
-      // the next item's queries go in as soon as this item's last S tile is read (every Q K^T of
-      // this item is complete), so its first tiles overlap this item's epilogue
-      const bool has_next = it_next >= 0;
-      __syncwarp();
-      const PfItem wn = has_next ? next_item : w;
-      if (has_next) q_finish(wn);
-      // epilogue: O / l
-      ok = pf_wait(&pv_done, (uint32_t)(g - 1) & 1, a, &abort_flag);
-      if (!bar_and(1, NSM, ok)) {
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      const float inv = 1.f / l;
-      if (Cf::OSTAGE && w.qr_end - w.qr0 == kPfRows) {
-        // a full tile: 32 columns at a time, each warp's 32 rows through its swizzled staging buffer
-        // into one TMA tensor store of box (32 columns, head h, 32 tokens)
-        const uint32_t stage_buf = smem_addr(sm + Cf::OST_OFF + warp * Cf::OST_WARP);
-        const int tok = w.ps.qtok + (w.qr0 - w.ps.q0) + 32 * warp;  // token of the warp's first row
-#pragma unroll
-        for (int hc = 0; hc < D / 32; ++hc) {
-          float o[32];
-          tmem_ld16(o_t + 32 * hc, o);
-          tmem_ld16(o_t + 32 * hc + 16, o + 16);
-          tmem_wait_ld();
-          if (lane == 0) bulk_wait_read0();  // the warp's previous store has read the buffer
-          __syncwarp();
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            st_shared_v4(stage_buf + lane * 128 + ((k ^ (lane & 7)) << 4), __float_as_uint(o[4 * k] * inv),
-                         __float_as_uint(o[4 * k + 1] * inv), __float_as_uint(o[4 * k + 2] * inv),
-                         __float_as_uint(o[4 * k + 3] * inv));
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            tma_store_3d(&tm_o, stage_buf, 32 * hc, w.h, tok);
-            bulk_commit();
-          }
-        }
-      } else {
-        const int64_t out_row = valid ? ((int64_t)(w.ps.qtok + (iq - w.ps.q0)) * a.H + w.h) * D : -1;
-        // O / l to global memory.  Each group of four lanes (four consecutive query rows) swaps float4s
-        // so that lane i of the group writes the i-th 16 bytes of each of the four rows in turn: a
-        // store instruction covers 64 contiguous bytes of eight rows, not 16 bytes of 32 rows.
-        const int gi = lane & 3;
-        int64_t orow[4];
-  #pragma unroll
-        for (int q = 0; q < 4; ++q) orow[q] = __shfl_sync(0xFFFFFFFFu, out_row, (lane & ~3) | q);
-  #pragma unroll
-        for (int u = 0; u < D / 16; ++u) {
-          float o[16];
-          tmem_ld16(o_t + 16 * u, o);
-          tmem_wait_ld();
-          float4 f[4];
-  #pragma unroll
-          for (int e = 0; e < 4; ++e) f[e] = make_float4(o[4 * e] * inv, o[4 * e + 1] * inv, o[4 * e + 2] * inv, o[4 * e + 3] * inv);
-          // 4 x 4 transpose of float4s across the group: exchange with lane gi ^ m the float4s whose
-          // index differs from gi in bit m, for m = 2 then 1
-  #pragma unroll
-          for (int m = 2; m >= 1; m >>= 1) {
-            const bool hi = (gi & m) != 0;
-  #pragma unroll
-            for (int j0 = 0; j0 < 4; ++j0) {
-              if (j0 & m) continue;
-              const int j1 = j0 | m;
-              const float4 snd = hi ? f[j0] : f[j1];
-              float4 rcv;
-              rcv.x = __shfl_xor_sync(0xFFFFFFFFu, snd.x, m);
-              rcv.y = __shfl_xor_sync(0xFFFFFFFFu, snd.y, m);
-              rcv.z = __shfl_xor_sync(0xFFFFFFFFu, snd.z, m);
-              rcv.w = __shfl_xor_sync(0xFFFFFFFFu, snd.w, m);
-              if (hi)
-                f[j0] = rcv;
-              else
-                f[j1] = rcv;
-            }
-          }
-  #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (orow[q] >= 0) reinterpret_cast<float4*>(a.out + orow[q] + 16 * u)[gi] = f[q];
-        }
-      }
-      tc_fence_before();
-      // every warp has read the next item (above) before any of them can overwrite it at the next
-      // item's last tile
-      bar_and(1, NSM, true);
-      it = it_next;
-      w = wn;
+      if (!ok || !more) break;
+      g += nk;
+      l_prev = l;
+      // the next item's queries came in after this item's last Q.K^T
+      if (next_ok && a.rot > 0) ok = q_rotate(item_slot[(k + 1) % kItemRing], k + 1);
+      more = next_ok;
       ++k;
     }
     if (Cf::OSTAGE && lane == 0) bulk_wait0();  // this warp's tensor stores are complete
-  } else {
-    regs_other();  // the two idle warps of the producer's warpgroup
   }
+  if (!ok) atomicOr(a.status, STATUS_TIMEOUT);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
@@ -1039,7 +1179,7 @@ cudaError_t encode_plane(const Geometry& g, void* base, unsigned char* out) {
   const int sw = (2 * g.D) % 128 == 0 ? 128 : (2 * g.D) % 64 == 0 ? 64 : 32;
   cuuint64_t dims[2] = {(cuuint64_t)g.D, (cuuint64_t)((int64_t)g.M * g.H * g.C)};
   cuuint64_t strides[1] = {(cuuint64_t)g.D * 2};
-  cuuint32_t box[2] = {(cuuint32_t)(sw / 2), (cuuint32_t)kPfRows};
+  cuuint32_t box[2] = {(cuuint32_t)(sw / 2), (cuuint32_t)prefill_keys_per_tile(g.D, g.dtype)};
   cuuint32_t elem[2] = {1, 1};
   const CUtensorMapSwizzle swz =
       sw == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : sw == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
@@ -1078,23 +1218,36 @@ cudaError_t launch_prefill_t(const PrefillMaps& maps, const PrefillArgs& a, int6
     }
     attr_set[dev] = true;
   }
-  CUtensorMap mk, mv, mo;
+  CUtensorMap mk, mv, mq, mo;
   std::memcpy(&mk, maps.k, sizeof mk);
   std::memcpy(&mv, maps.v, sizeof mv);
   std::memset(&mo, 0, sizeof mo);
+  cuuint32_t elem[3] = {1, 1, 1};
+  {
+    // q as [token][head][D], in boxes of one column subtile x one head x 128 tokens
+    cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)a.H, (cuuint64_t)a.n_qtok};
+    cuuint64_t strides[2] = {(cuuint64_t)D * 2, (cuuint64_t)a.H * D * 2};
+    cuuint32_t box[3] = {(cuuint32_t)Cf::SUB, 1, (cuuint32_t)kPfRows};
+    const CUresult r = g_encode(&mq, CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, const_cast<uint16_t*>(a.q), dims, strides, box, elem,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE,
+                                Cf::SW == 128   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                : Cf::SW == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                               : CU_TENSOR_MAP_SWIZZLE_32B,
+                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  }
   if (Cf::OSTAGE && a.n_qtok >= kPfRows) {
-    // out as [token][head][D] fp32, stored in boxes of 32 columns x one head x 32 tokens from the
+    // out as [token][head][D] fp32, stored in boxes of 16 columns x one head x 32 tokens from the
     // softmax warps' swizzled staging buffers (only full query tiles take this path)
     cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)a.H, (cuuint64_t)a.n_qtok};
     cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)a.H * D * 4};
-    cuuint32_t box[3] = {32, 1, 32};
-    cuuint32_t elem[3] = {1, 1, 1};
+    cuuint32_t box[3] = {16, 1, 32};
     const CUresult r = g_encode(&mo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a.out, dims, strides, box, elem,
-                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
   }
-  prefill_kernel<T, D><<<(unsigned)grid, kPfThreads, Cf::SMEM, stream>>>(mk, mv, mo, a);
+  prefill_kernel<T, D><<<(unsigned)grid, kPfThreads, Cf::SMEM, stream>>>(mk, mv, mq, mo, a);
   return cudaGetLastError();
 }
 
@@ -1144,6 +1297,15 @@ cudaError_t encode_prefill_maps(const Geometry& g, const Buffers& buf, PrefillMa
   return e;
 }
 
+int prefill_keys_per_tile(int D, int dtype) {
+  switch (D) {
+    case 64: return dtype ? PfCfg<64, true>::KT : PfCfg<64, false>::KT;
+    case 80: return dtype ? PfCfg<80, true>::KT : PfCfg<80, false>::KT;
+    case 96: return PfCfg<96>::KT;
+    default: return PfCfg<128>::KT;
+  }
+}
+
 int prefill_ctas_per_sm(int D) {
   switch (D) {
     case 64: return PfCfg<64>::CPS;
@@ -1156,7 +1318,7 @@ int prefill_ctas_per_sm(int D) {
 
 cudaError_t launch_prefill(const Geometry& g, const PrefillMaps& maps, const PrefillArgs& a, cudaStream_t stream) {
   if (a.n_items <= 0 || a.n_ctas <= 0) return cudaSuccess;
-  const int64_t grid = a.n_ctas;  // persistent: at most one CTA per SM
+  const int64_t grid = a.n_ctas;  // persistent
   const bool bf = g.dtype == 1;
   switch (g.D) {
     case 64:

@@ -195,3 +195,48 @@ def test_prefill_rope_partial_rotary_dim():
     # only the first 32 of 80 dimensions rotated (pairs (e, e + 16)); blocks of 200 tokens
     w = dataclasses.replace(wl.rope3b(32, b=2, L=384, M=1), rotary_dim=32, name="rope-partial")
     run_prefill(w, 200, layers=[0], heads=[5, 30])
+
+
+def _edge_history(rng, L, what):
+    """A history of L tokens: no span; many spans of 0 to 2 tokens (most tiles hold a run of keys per span);
+    spans longer than a query tile (their interiors begin in one tile and close in a later one, or never)."""
+    kinds, spans = np.zeros(L, np.uint8), []
+    if what == "none":
+        return kinds, spans
+    lo, hi, gap = (0, 3, 4) if what == "short" else (100, 260, 60)
+    t = int(rng.integers(0, 3))
+    while t < L:
+        cr = t + 1 + int(rng.integers(lo, hi))
+        kinds[t] = 1
+        if cr >= L:
+            break
+        kinds[cr] = 2
+        spans.append((t, cr))
+        t = cr + 1 + int(rng.integers(0, gap))
+    return kinds, spans
+
+
+@pytest.mark.parametrize("d,dtype,rot,block,policy", [
+    (64, "f16", 0, 0, orc.POLICY_PAPER),
+    (64, "f16", 64, 130, orc.POLICY_KEEP_CL),
+    (64, "bf16", 0, 130, orc.POLICY_PAPER),
+    (80, "f16", 80, 0, orc.POLICY_PAPER),
+    (80, "f16", 0, 130, orc.POLICY_KEEP_CL),
+    (80, "bf16", 32, 0, orc.POLICY_KEEP_CL),
+    (96, "f16", 0, 130, orc.POLICY_PAPER),
+    (128, "bf16", 64, 0, orc.POLICY_PAPER),
+])
+def test_prefill_key_lists_at_tile_edges(d, dtype, rot, block, policy):
+    """Each query tile reads the rows that no span hides from a list, then the interior of a span it begins in,
+    then its own rows, in tiles of 64, 112 or 128 keys that are copied whole where their rows lie side by side
+    and gathered where they do not: lengths at the edges of both tiles (items of a single key tile among
+    them), histories without spans, with many short ones, and with spans longer than a query tile."""
+    import dataclasses
+
+    rng = np.random.default_rng(d + rot + block)
+    lens = [1, 2, 63, 64, 65, 111, 112, 113, 127, 128, 129, 225, 256, 257, 511, 640]
+    hist = [_edge_history(rng, L, what) for what in ("none", "short", "long") for L in lens]
+    w = dataclasses.replace(wl.opt13b(b=len(hist), L=64, M=1), name="edges", d=d, dtype=dtype,
+                            prompt_kinds=[k for k, _ in hist], prompt_spans=[sp for _, sp in hist],
+                            scale=1.0 / np.sqrt(d), rotary_dim=rot)
+    run_prefill(w, block, layers=[0], heads=[0, 31], policy=policy)
