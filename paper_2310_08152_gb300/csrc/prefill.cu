@@ -32,8 +32,8 @@
 // every stored row with masks over all of them: OPT-1.3B-shaped prompts (16 x 2048 tokens, 32 heads of 64,
 // interiors of 32) 541 -> 362 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 990 us; the
 // last 512 of 32 x 4096 tokens, compacted before them, bf16 (heads of 80) 664 -> 456 us; the first with 96 and
-// 128 columns 797 -> 580 and 1042 -> 602 us; one prompt of 300 tokens 13.2 -> 12.2 us.  Copying the listed rows side by side first, for TMA tiles alone, took a
-// second kernel and 381, 992 and 454 us on the first three.
+// 128 columns 797 -> 580 and 1042 -> 602 us; one prompt of 300 tokens 13.2 -> 12.2 us.  Copying the listed rows
+// side by side first, for TMA tiles alone, took a second kernel and 381, 992 and 454 us on the first three.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
