@@ -245,11 +245,13 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
 }
 
 // Shared-memory matrix descriptor: start address, leading / stride byte offsets, version 1, and
-// the swizzle (layout type 2 = 128 B, 4 = 64 B, 6 = 32 B).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo, int sw) {
-  const uint64_t layout = sw == 128 ? 2 : sw == 64 ? 4 : 6;
-  return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | (1ull << 46) | (layout << 61);
+// the swizzle (layout type 2 = 128 B, 4 = 64 B, 6 = 32 B).  Its low word holds the address and the leading
+// offset, so a tile's descriptors are one word plus constants (addresses stay below 256 KB): built in full for each
+// one, about 100 cycles of the issuing thread per tcgen05.mma.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return addr >> 4 | (lbo >> 4) << 16; }
+__device__ __forceinline__ uint64_t desc(uint32_t lo, uint32_t sbo, int sw) {
+  const uint32_t hi = (sbo >> 4) | 1u << 14 | (sw == 128 ? 2u : sw == 64 ? 4u : 6u) << 29;
+  return (uint64_t)hi << 32 | lo;
 }
 // Instruction descriptor of kind::f16 with an fp32 accumulator: A and B of one 16-bit type
 // (0 = f16, 1 = bf16), A K-major, B K-major (0) or MN-major (1), N >> 3, M >> 4.
@@ -715,88 +717,102 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     if (lane == 0) {
       constexpr uint32_t idS = mma_idesc(Pack16<T>::kType, 0, kPfRows, KT);
       constexpr uint32_t idO = mma_idesc(Pack16<T>::kType, 1, kPfRows, D);
-      const uint32_t q_s = smem_addr(sm + Cf::Q_OFF);
-      [[maybe_unused]] const uint32_t qlo_s = smem_addr(sm + Cf::QLO_OFF);
-      int64_t g = 0;
-      for (uint32_t k = 0; ok; ++k) {
-        if (!(ok = item_wait(k))) break;
-        const int nk = item_slot[k % kItemRing].nk;
-        mbar_arrive(&item_empty[k % kItemRing]);
-        if (nk == 0) break;
-        ok = pf_wait(a.rot > 0 ? &q_full : &q_raw, k & 1, limit_ns);
-        if (!ok) break;
+      constexpr uint32_t SBO = 8 * SW;
+      const uint32_t q_d = desc_lo(smem_addr(sm + Cf::Q_OFF), 16);
+      [[maybe_unused]] const uint32_t qlo_d = desc_lo(smem_addr(sm + Cf::QLO_OFF), 16);
+      // S = Q K^T of tile gj into its S tile.  One S tile: once the softmax has read S of tile
+      // gj - 1.  Two: the tile last held P of tile gj - 2, whose P.V was issued before (tcgen05.mma
+      // from one thread run in issue order).
+      auto issue_qk = [&](uint32_t gj, bool last) -> bool {
+        const int st = (int)(gj % KST), sb = (int)(gj % SBUF);
+        if (!pf_wait(&k_full[st], (gj / KST) & 1, limit_ns)) return false;
+        if (Cf::PSEP && gj >= 1 && !pf_wait(&s_free, (gj - 1) & 1, limit_ns)) return false;
+        fence_proxy_async_smem();  // gathered rows were written through the generic proxy
         tc_fence_after();
-        const uint32_t o_t = tmem + Cf::O_COL + (Cf::OBUF == 2 ? (k & 1) * D : 0);
-        // S = Q K^T of tile gj into its S tile.  One S tile: once the softmax has read S of tile
-        // gj - 1.  Two: the tile last held P of tile gj - 2, whose P.V was issued before (tcgen05.mma
-        // from one thread run in issue order).
-        auto issue_qk = [&](int64_t gj, bool last) -> bool {
-          const int st = (int)(gj % KST), sb = (int)(gj % SBUF);
-          if (!pf_wait(&k_full[st], (uint32_t)(gj / KST) & 1, limit_ns)) return false;
-          if (Cf::PSEP && gj >= 1 && !pf_wait(&s_free, (uint32_t)(gj - 1) & 1, limit_ns)) return false;
-          fence_proxy_async_smem();  // gathered rows were written through the generic proxy
-          tc_fence_after();
-          const uint32_t k_s = smem_addr(sm + Cf::K_OFF + st * Cf::TILE);
+        const uint32_t k_d = desc_lo(smem_addr(sm + Cf::K_OFF + st * Cf::TILE), 16);
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t off = (kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2;
-            const uint32_t qoff = (kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2;
-            tc_mma(tmem + sb * KT, smem_desc(q_s + qoff, 16, 8 * SW, SW), smem_desc(k_s + off, 16, 8 * SW, SW), idS,
-                   kk > 0);
-          }
-          // SPLIT with RoPE: + Q_lo K^T (without RoPE the query is exact in the cache type)
-          if constexpr (Cf::SPLIT) {
-            if (a.rot > 0) {
+        for (int kk = 0; kk < D / 16; ++kk) {
+          const uint32_t off = ((kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2) >> 4;
+          const uint32_t qoff = ((kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2) >> 4;
+          tc_mma(tmem + sb * KT, desc(q_d + qoff, SBO, SW), desc(k_d + off, SBO, SW), idS, kk > 0);
+        }
+        // SPLIT with RoPE: + Q_lo K^T (without RoPE the query is exact in the cache type)
+        if constexpr (Cf::SPLIT) {
+          if (a.rot > 0) {
 #pragma unroll
-              for (int kk = 0; kk < D / 16; ++kk) {
-                const uint32_t off = (kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2;
-                [[maybe_unused]] const uint32_t qoff = (kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2;
-                if constexpr (Cf::QLO_TMEM)
-                  tc_mma_ts(tmem + sb * KT, tmem + Cf::QLO_COL + 8 * kk, smem_desc(k_s + off, 16, 8 * SW, SW), idS, 1);
-                else
-                  tc_mma(tmem + sb * KT, smem_desc(qlo_s + qoff, 16, 8 * SW, SW), smem_desc(k_s + off, 16, 8 * SW, SW),
-                         idS, 1);
-              }
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const uint32_t off = ((kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2) >> 4;
+              [[maybe_unused]] const uint32_t qoff = ((kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2) >> 4;
+              if constexpr (Cf::QLO_TMEM)
+                tc_mma_ts(tmem + sb * KT, tmem + Cf::QLO_COL + 8 * kk, desc(k_d + off, SBO, SW), idS, 1);
+              else
+                tc_mma(tmem + sb * KT, desc(qlo_d + qoff, SBO, SW), desc(k_d + off, SBO, SW), idS, 1);
             }
           }
-          tc_commit(&s_full[sb]);
-          tc_commit(&k_empty[st]);
-          if (last) tc_commit(&q_empty);
-          return true;
-        };
-        // O += P V of tile gp (8 TMEM columns of P per 16 keys); the first of an item: O = P V
-        auto issue_pv = [&](int64_t gp, bool first) -> bool {
-          const int st = (int)(gp % VST);
-          if (!pf_wait(&v_full[st], (uint32_t)(gp / VST) & 1, limit_ns)) return false;
-          if (!pf_wait(&p_full, (uint32_t)gp & 1, limit_ns)) return false;
-          fence_proxy_async_smem();
-          tc_fence_after();
-          const uint32_t v_s = smem_addr(sm + Cf::V_OFF + st * Cf::TILE);
-          const uint32_t p_t = tmem + (Cf::PSEP ? Cf::P_COL : (uint32_t)(gp % SBUF) * KT);
+        }
+        tc_commit(&s_full[sb]);
+        tc_commit(&k_empty[st]);
+        if (last) tc_commit(&q_empty);
+        return true;
+      };
+      // O += P V of tile gp (8 TMEM columns of P per 16 keys) into o_t; the first of an item: O = P V
+      auto issue_pv = [&](uint32_t gp, uint32_t o_t, bool first) -> bool {
+        const int st = (int)(gp % VST);
+        if (!pf_wait(&v_full[st], (gp / VST) & 1, limit_ns)) return false;
+        if (!pf_wait(&p_full, gp & 1, limit_ns)) return false;
+        fence_proxy_async_smem();
+        tc_fence_after();
+        const uint32_t v_d = desc_lo(smem_addr(sm + Cf::V_OFF + st * Cf::TILE), Cf::SUBB);
+        const uint32_t p_t = tmem + (Cf::PSEP ? Cf::P_COL : gp % SBUF * KT);
+#pragma unroll
+        for (int kk = 0; kk < KT / 16; ++kk)
+          tc_mma_ts(o_t, p_t + 8 * kk, desc(v_d + kk * SW, SBO, SW), idO, (!first || kk > 0));
+        if constexpr (Cf::SPLIT) {  // + P_lo V
 #pragma unroll
           for (int kk = 0; kk < KT / 16; ++kk)
-            tc_mma_ts(o_t, p_t + 8 * kk, smem_desc(v_s + kk * 16 * SW, Cf::SUBB, 8 * SW, SW), idO, (!first || kk > 0));
-          if constexpr (Cf::SPLIT) {  // + P_lo V
-#pragma unroll
-            for (int kk = 0; kk < KT / 16; ++kk)
-              tc_mma_ts(o_t, p_t + Cf::PLO_COL + 8 * kk, smem_desc(v_s + kk * 16 * SW, Cf::SUBB, 8 * SW, SW), idO, 1);
+            tc_mma_ts(o_t, p_t + Cf::PLO_COL + 8 * kk, desc(v_d + kk * SW, SBO, SW), idO, 1);
+        }
+        tc_commit(&pv_done);
+        tc_commit(&v_empty[st]);
+        return true;
+      };
+      // Q K^T of a tile goes in ahead of P.V of the tile before, also when that is the last of its item: it
+      // runs while the softmax works on that tile (an item's first scores were 1900 to 2900 cycles late with its
+      // Q K^T after that P.V: OPT-1.3B-shaped prompts 362 us a layer, 348 so, with the cheaper descriptors).  The
+      // rotated queries of an item come from the softmax warps after their last tile, whose P.V does not wait
+      // for them.
+      const bool rot = a.rot > 0;
+      uint32_t gq = 0, gp = 0;  // Q K^T, P.V issued
+      uint32_t kq = 0, kp = 0;  // their items
+      int jq = 0, jp = 0, nkq = 0;
+      bool items = true;  // there may be another one
+      while (ok) {
+        if (items && !(rot && jq == 0 && gq != gp)) {
+          if (jq == 0) {
+            if (!(ok = item_wait(kq))) break;
+            nkq = item_slot[kq % kItemRing].nk;
+            items = nkq > 0;
+            if (items && !(ok = pf_wait(rot ? &q_full : &q_raw, kq & 1, limit_ns))) break;
+            tc_fence_after();
           }
-          tc_commit(&pv_done);
-          tc_commit(&v_empty[st]);
-          return true;
-        };
-        // Q K^T of the next tile goes in ahead of P.V of the current one: it runs while the softmax
-        // works on the current tile
-        for (int j = 0; ok && j <= nk; ++j) {
-          if (SBUF == 1 && !Cf::PSEP) {  // P sits in the one S tile: its P.V before the next Q K^T
-            if (j >= 1) ok = issue_pv(g + j - 1, j == 1);
-            if (ok && j < nk) ok = issue_qk(g + j, j == nk - 1);
-          } else {
-            if (j < nk) ok = issue_qk(g + j, j == nk - 1);
-            if (ok && j >= 1) ok = issue_pv(g + j - 1, j == 1);
+          if (items) {
+            if (!(ok = issue_qk(gq, jq == nkq - 1))) break;
+            ++gq;
+            if (++jq == nkq) {
+              jq = 0;
+              ++kq;
+            }
+            if (gq - gp == 1 && !(rot && jq == 0)) continue;
           }
         }
-        g += nk;
+        if (gq == gp) break;
+        if (!(ok = issue_pv(gp, tmem + Cf::O_COL + (Cf::OBUF == 2 ? (kp & 1) * D : 0), jp == 0))) break;
+        ++gp;
+        if (++jp == item_slot[kp % kItemRing].nk) {
+          mbar_arrive(&item_empty[kp % kItemRing]);
+          jp = 0;
+          ++kp;
+        }
       }
       // every MMA issued above has completed once this phase does
       tc_commit(&drain);
