@@ -93,13 +93,7 @@ struct PfCfg {
   static constexpr uint32_t QLO_OFF = QTILE;  // QLO_SMEM only
   static constexpr uint32_t K_OFF = QTILE * (QLO_SMEM ? 2 : 1);
   static constexpr uint32_t V_OFF = K_OFF + KST * TILE;
-  // With two CTAs per SM there is shared memory left for O / l: each softmax warp has OST_N buffers of 32
-  // rows x 16 columns (2 KB, 64-byte swizzle) for TMA tensor stores.
-  static constexpr bool OSTAGE = CPS == 2;
-  static constexpr int OST_N = D == 64 ? 3 : 2;
-  static constexpr uint32_t OST_OFF = (V_OFF + VST * TILE + 1023) / 1024 * 1024;
-  static constexpr uint32_t OST_BUF = 32 * 16 * 4;
-  static constexpr uint32_t SMEM = OST_OFF + (OSTAGE ? 4 * OST_N * OST_BUF : 0) + 1024;  // + aligning the base
+  static constexpr uint32_t SMEM = V_OFF + VST * TILE + 1024;  // + aligning the base
   // TMEM.  Two CTAs per SM, 256 columns each: S, O, P (16-bit, two per column; SPLIT: its high part, then
   // its low part) and SPLIT's low part of the query (D / 2 columns) in columns of their own, so S is
   // released as soon as the softmax has read it and the next Q.K^T overlaps the softmax.  One CTA per SM:
@@ -151,20 +145,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
       : "memory");
 }
-// Tensor store from shared memory (bulk group of the issuing thread) and its waits.
-__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
-  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(x), "r"(y), "r"(z), "r"(src)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// At most N of this thread's bulk groups are still reading shared memory.
-template <int N>
-__device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-__device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
@@ -206,6 +186,48 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+}
+// 16 TMEM lanes of 8 n columns: lane l gets of columns 8 c + 2 (l % 4) and the next those of rows l / 4 (v[4 c],
+// v[4 c + 1]) and l / 4 + 8 (v[4 c + 2], v[4 c + 3]).
+__device__ __forceinline__ void tmem_ld_16x256b_x2(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {"
+      "%0,%1,%2,%3,%4,%5,%6,%7"
+      "}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {"
+      "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15"
+      "}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, float* v) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 {"
+      "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,"
+      "%25,%26,%27,%28,%29,%30,%31"
+      "}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+template <int D>
+__device__ __forceinline__ void tmem_ld_16x256b(uint32_t taddr, float* v) {
+  tmem_ld_16x256b_x8(taddr, v);
+  if constexpr (D == 80) tmem_ld_16x256b_x2(taddr + 64, v + 32);
+  if constexpr (D == 96) tmem_ld_16x256b_x4(taddr + 64, v + 32);
+  if constexpr (D == 128) tmem_ld_16x256b_x8(taddr + 64, v + 32);
+  static_assert(D == 64 || D == 80 || D == 96 || D == 128, "head dimension");
 }
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
   const uint32_t* r = reinterpret_cast<const uint32_t*>(v);
@@ -431,8 +453,7 @@ __device__ __forceinline__ void gather_rows(uint32_t dst, uint32_t subb, const u
 template <typename T, int D>
 __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     prefill_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                   const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_o,
-                   const PrefillArgs a) {
+                   const __grid_constant__ CUtensorMap tm_q, const PrefillArgs a) {
   using Cf = PfCfg<D, kSplit<T>>;
   constexpr int SW = Cf::SW, SUB = Cf::SUB, KST = Cf::KST, VST = Cf::VST, SBUF = Cf::SBUF, KT = Cf::KT;
   extern __shared__ uint8_t pf_smem_raw[];
@@ -915,50 +936,45 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
       return __all_sync(0xFFFFFFFFu, pf_wait(bar, parity, limit_ns));
     };
-    // Epilogue of item kk (row sum l_): O / l, 16 columns at a time.  A full tile goes out through each
-    // warp's swizzled buffers in turn as TMA tensor stores of box (16 columns, head h, 32 tokens); else
-    // each thread stores its query's row.
+    // Epilogue of item kk (row sum l_): O / l, 16 rows at a time.  The 16-lane form of tcgen05.ld gives four
+    // neighbouring lanes 8 columns of a row, so each store fills 32-byte sectors of eight queries' rows (3000
+    // cycles an item when each warp staged 16 columns at a time in shared memory for tensor stores).  A few
+    // columns at a time: the next tile's scores are in registers meanwhile (64 columns: 348 us staged, 399 with
+    // 64 columns at a time, 333 with 32).
     auto epilogue = [&](uint32_t kk, float l_) {
       const PfItem& w = item_slot[kk % kItemRing];
       const uint32_t o_t = tl + Cf::O_COL + (Cf::OBUF == 2 ? (kk & 1) * D : 0);
-      const bool staged = Cf::OSTAGE && w.qr_end - w.qr0 == kPfRows;
-      const bool valid = w.qr0 + r < w.qr_end;
       const float inv = 1.f / l_;
-      uint32_t buf = smem_addr(sm + Cf::OST_OFF + warp * Cf::OST_N * Cf::OST_BUF);
-      const uint32_t buf_end = buf + Cf::OST_N * Cf::OST_BUF;
-      float* orow = a.out + ((int64_t)(w.tok0 + r) * a.H + w.h) * D;
+      const int64_t row8 = (int64_t)8 * a.H * D;
+      float* o_row = a.out + ((int64_t)(w.tok0 + warp * 32 + (lane >> 2)) * a.H + w.h) * D + 2 * (lane & 3);
+      constexpr int CO = D % 32 == 0 ? 32 : 16;  // columns at a time
 #pragma unroll 1
-      for (int u = 0; u < D / 16; ++u) {
-        float o[16];
-        tmem_ld16(o_t + 16 * u, o);
-        tmem_wait_ld();
+      for (int i = 0; i < 32; i += 16) {
+        const float inv0 = __shfl_sync(0xFFFFFFFFu, inv, i + (lane >> 2));
+        const float inv1 = __shfl_sync(0xFFFFFFFFu, inv, i + 8 + (lane >> 2));
+        const int left = w.qr_end - w.qr0 - (warp * 32 + i + (lane >> 2));  // queries from this lane's row on
+#pragma unroll 1
+        for (int u = 0; u < D; u += CO) {
+          float o[CO / 2];
+          if constexpr (CO == 32)
+            tmem_ld_16x256b_x4(o_t + (i << 16) + u, o);
+          else
+            tmem_ld_16x256b_x2(o_t + (i << 16) + u, o);
+          tmem_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 16; ++e) o[e] *= inv;
-        if (staged) {
-          if (lane == 0) {  // the buffer's last store has read it
-            if (u == 0)
-              bulk_wait_read<0>();
-            else
-              bulk_wait_read<Cf::OST_N - 1>();
+          for (int e = 0; e < CO / 2; ++e) asm volatile("" : "+f"(o[e]));  // no use of O moves above the wait
+          if (left > 0) {
+#pragma unroll
+            for (int c = 0; c < CO / 8; ++c)
+              *reinterpret_cast<float2*>(o_row + u + 8 * c) = make_float2(o[4 * c] * inv0, o[4 * c + 1] * inv0);
           }
-          __syncwarp();
+          if (left > 8) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c)
-            st_shared_v4(buf + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), __float_as_uint(o[4 * c]),
-                         __float_as_uint(o[4 * c + 1]), __float_as_uint(o[4 * c + 2]), __float_as_uint(o[4 * c + 3]));
-          fence_proxy_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-            tma_store_3d(&tm_o, buf, 16 * u, w.h, w.tok0 + 32 * warp);
-            bulk_commit();
+            for (int c = 0; c < CO / 8; ++c)
+              *reinterpret_cast<float2*>(o_row + row8 + u + 8 * c) = make_float2(o[4 * c + 2] * inv1, o[4 * c + 3] * inv1);
           }
-          buf += Cf::OST_BUF;
-          if (buf == buf_end) buf -= Cf::OST_N * Cf::OST_BUF;
-        } else if (valid) {
-#pragma unroll
-          for (int e = 0; e < 16; e += 4)
-            *reinterpret_cast<float4*>(orow + 16 * u + e) = make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
         }
+        o_row += 2 * row8;
       }
       tc_fence_before();
       item_done(kk);
@@ -1149,11 +1165,13 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           if (!ok) break;
         }
         tc_fence_after();
+        if (Cf::PSEP && more) {
+          store_p(0);
+          store_p(1);
+        }
         if (j == 0 && k >= 1) epilogue(k - 1, l_prev);
         if (!more) break;
         if (Cf::PSEP) {
-          store_p(0);
-          store_p(1);
 #pragma unroll
           for (int q = 2; q < (CW + 31) / 32; ++q) {
             make_p(q);
@@ -1176,7 +1194,6 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       more = next_ok;
       ++k;
     }
-    if (Cf::OSTAGE && lane == 0) bulk_wait0();  // this warp's tensor stores are complete
   }
   if (!ok) atomicOr(a.status, STATUS_TIMEOUT);
   tc_fence_before();
@@ -1234,10 +1251,9 @@ cudaError_t launch_prefill_t(const PrefillMaps& maps, const PrefillArgs& a, int6
     }
     attr_set[dev] = true;
   }
-  CUtensorMap mk, mv, mq, mo;
+  CUtensorMap mk, mv, mq;
   std::memcpy(&mk, maps.k, sizeof mk);
   std::memcpy(&mv, maps.v, sizeof mv);
-  std::memset(&mo, 0, sizeof mo);
   cuuint32_t elem[3] = {1, 1, 1};
   {
     // q as [token][head][D], in boxes of one column subtile x one head x 128 tokens
@@ -1252,18 +1268,7 @@ cudaError_t launch_prefill_t(const PrefillMaps& maps, const PrefillArgs& a, int6
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
   }
-  if (Cf::OSTAGE && a.n_qtok >= kPfRows) {
-    // out as [token][head][D] fp32, stored in boxes of 16 columns x one head x 32 tokens from the
-    // softmax warps' swizzled staging buffers (only full query tiles take this path)
-    cuuint64_t dims[3] = {(cuuint64_t)D, (cuuint64_t)a.H, (cuuint64_t)a.n_qtok};
-    cuuint64_t strides[2] = {(cuuint64_t)D * 4, (cuuint64_t)a.H * D * 4};
-    cuuint32_t box[3] = {16, 1, 32};
-    const CUresult r = g_encode(&mo, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a.out, dims, strides, box, elem,
-                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
-                                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-  }
-  prefill_kernel<T, D><<<(unsigned)grid, kPfThreads, Cf::SMEM, stream>>>(mk, mv, mq, mo, a);
+  prefill_kernel<T, D><<<(unsigned)grid, kPfThreads, Cf::SMEM, stream>>>(mk, mv, mq, a);
   return cudaGetLastError();
 }
 
