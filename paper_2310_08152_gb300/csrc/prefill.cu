@@ -208,27 +208,6 @@ __device__ __forceinline__ void tmem_ld_16x256b_x4(uint32_t taddr, float* v) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, float* v) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x8.b32 {"
-      "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,"
-      "%25,%26,%27,%28,%29,%30,%31"
-      "}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-}
-template <int D>
-__device__ __forceinline__ void tmem_ld_16x256b(uint32_t taddr, float* v) {
-  tmem_ld_16x256b_x8(taddr, v);
-  if constexpr (D == 80) tmem_ld_16x256b_x2(taddr + 64, v + 32);
-  if constexpr (D == 96) tmem_ld_16x256b_x4(taddr + 64, v + 32);
-  if constexpr (D == 128) tmem_ld_16x256b_x8(taddr + 64, v + 32);
-  static_assert(D == 64 || D == 80 || D == 96 || D == 128, "head dimension");
-}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float* v) {
   const uint32_t* r = reinterpret_cast<const uint32_t*>(v);
   asm volatile(
@@ -468,12 +447,12 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
   // For the key tiles that hold rows from b0 on, the tile's keys against its item's query tile
   // [qr0, qr_end): khid has bit c set when key c's bound holds for every query of the tile (hid >=
   // qr_end - 1).  The keys whose bound falls inside it (qr0 <= hid < qr_end - 1: a span closing among
-  // the queries) come in runs of one bound -- a span's interior shares its <CR>, a <CL> hidden from
-  // every later query is a run of one -- kept as the bound (rhid) and the columns (rbits), kn runs.
-  __shared__ uint4 khid[kClsRing];
-  __shared__ int32_t rhid[kClsRing][KT];
-  __shared__ uint4 rbits[kClsRing][KT];
-  __shared__ int32_t kn[kClsRing];
+  // the queries; a <CL> hidden from every later query) go by their bound: kend has bit hid - qr0 set for
+  // each such bound, and kafter[i] are the keys whose bound is the i-th of those or a later one, so a
+  // query finds all of them that it may see with one lookup (a loop over the spans in each softmax thread
+  // before: OPT-1.3B-shaped prompts 333 us, 327 so).
+  __shared__ uint4 khid[kClsRing], kend[kClsRing];
+  __shared__ uint4 kafter[kClsRing][KT + 1];
   __shared__ int32_t kslow[kClsRing];  // the tile needs the per-key rule (else every key is visible)
   __shared__ uint64_t cls_full[kClsRing], cls_empty[kClsRing];
   __shared__ uint32_t tmem_slot;
@@ -566,10 +545,11 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         const int cs = (int)(cg % kClsRing);
         // per-key mask bounds of the tile ((hid << 1) | is_cl) sorted into the classes above; the causal
         // part (i <= iq) is left to each query
-        uint32_t ok_w[4];
-        int hp[4];  // the key's bound when it falls among the queries, else -3
+        constexpr int NW = (KT + 31) / 32;
+        uint32_t ok_w[4] = {0u, 0u, 0u, 0u}, end_w[4] = {0u, 0u, 0u, 0u};
+        int hp[NW];  // the key's bound from the first query on when it falls among the queries, else -1
 #pragma unroll
-        for (int w4 = 0; w4 < 4; ++w4) {
+        for (int w4 = 0; w4 < NW; ++w4) {
           const int v = v0 + lane + 32 * w4;
           int hid = w.qr_end;  // a row that no span hides
           if (lane + 32 * w4 >= KT || v >= keys || (v >= before && v < own))
@@ -579,48 +559,35 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           else if (v >= w.n_c)
             hid = a.meta[w.moff + w.b0 + (v - w.n_c)] >> 1;
           ok_w[w4] = __ballot_sync(0xFFFFFFFFu, hid >= w.qr_end - 1);
-          hp[w4] = hid >= w.qr0 && hid < w.qr_end - 1 ? hid : -3;
+          hp[w4] = hid >= w.qr0 && hid < w.qr_end - 1 ? hid - w.qr0 : -1;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) end_w[u] |= hp[w4] >> 5 == u ? 1u << (hp[w4] & 31) : 0u;
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) end_w[u] = __reduce_or_sync(0xFFFFFFFFu, end_w[u]);
         if (cg >= kClsRing && !pf_wait(&cls_empty[cs], ((cg / kClsRing) - 1) & 1, limit_ns)) {
           ok = false;
           break;
         }
-        // runs: a listed key starts one unless key c - 1 is listed with the same bound, and ends one
-        // unless key c + 1 is
-        int n_run = 0;
+        int n_end = 0;
+#pragma unroll 1
+        for (int u = 0; u < 4; ++u) {
+          uint32_t left = u == 0 ? end_w[0] : u == 1 ? end_w[1] : u == 2 ? end_w[2] : end_w[3];
+          for (; left != 0u; left &= left - 1u, ++n_end) {
+            const int h = 32 * u + __ffs(left) - 1;
+            uint32_t m[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-        for (int w4 = 0; w4 < 4; ++w4) {
-          const int c = lane + 32 * w4;
-          int prev = __shfl_up_sync(0xFFFFFFFFu, hp[w4], 1);
-          int next = __shfl_down_sync(0xFFFFFFFFu, hp[w4], 1);
-          const int prev_w = w4 > 0 ? __shfl_sync(0xFFFFFFFFu, hp[w4 > 0 ? w4 - 1 : 0], 31) : -3;
-          const int next_w = w4 < 3 ? __shfl_sync(0xFFFFFFFFu, hp[w4 < 3 ? w4 + 1 : 3], 0) : -3;
-          if (lane == 0) prev = prev_w;
-          if (lane == 31) next = next_w;
-          const bool start = hp[w4] >= 0 && prev != hp[w4];
-          const bool end = hp[w4] >= 0 && next != hp[w4];
-          const uint32_t sb = __ballot_sync(0xFFFFFFFFu, start);
-          const int rid = n_run + __popc(sb & ((2u << lane) - 1u)) - 1;  // runs started at or before c, less one
-          if (start) {
-            rhid[cs][rid] = hp[w4];
-            rbits[cs][rid].x = (uint32_t)c;  // its columns [x, y), made into bits below
+            for (int w4 = 0; w4 < NW; ++w4) m[w4] = __ballot_sync(0xFFFFFFFFu, hp[w4] >= h);
+            if (lane == 0) kafter[cs][n_end] = make_uint4(m[0], m[1], m[2], m[3]);
           }
-          if (end) rbits[cs][rid].y = (uint32_t)(c + 1);
-          n_run += __popc(sb);
         }
-        __syncwarp();
-        for (int e = lane; e < n_run; e += 32) {
-          const int cb = (int)rbits[cs][e].x, ce = (int)rbits[cs][e].y;
-          rbits[cs][e] = make_uint4(low_bits(ce) & ~low_bits(cb), low_bits(ce - 32) & ~low_bits(cb - 32),
-                                    low_bits(ce - 64) & ~low_bits(cb - 64), low_bits(ce - 96) & ~low_bits(cb - 96));
-        }
-        __syncwarp();
         if (lane == 0) {
+          kafter[cs][n_end] = make_uint4(0u, 0u, 0u, 0u);
           khid[cs] = make_uint4(ok_w[0], ok_w[1], ok_w[2], ok_w[3]);
-          // per-key masking is needed when a key's visibility differs between the tile's queries: runs,
-          // and keys at or past the first query (the causal rule); and for columns without a key
-          kn[cs] = n_run;
-          kslow[cs] = n_run > 0 || v0 + KT > before;
+          kend[cs] = make_uint4(end_w[0], end_w[1], end_w[2], end_w[3]);
+          // per-key masking is needed when a key's visibility differs between the tile's queries: bounds
+          // among them, and keys at or past the first query (the causal rule); and for columns without a key
+          kslow[cs] = n_end > 0 || v0 + KT > before;
           mbar_arrive(&cls_full[cs]);
         }
         ++cg;
@@ -991,7 +958,6 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     while (ok && (more || k >= 1)) {
       const PfItem& w = item_slot[k % kItemRing];
       const int nk = more ? w.nk : 1, n_c = w.n_c;
-      const int iq = w.qr0 + r;      // stored row of this query
       const int vq = w.own(KT) + r;  // its own key
       const bool cl_q = cl_next;
       bool next_ok = false;  // there is another item
@@ -1052,24 +1018,16 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           uint32_t vw[4];
           if (slow) {
             // visibility of the tile's keys to this query as 32-bit words: the causal prefix (keys up to the
-            // query's own) with the tile-wide bound words plus the runs whose bound admits iq.  Every key of
-            // the other tiles is visible (to all but a <CL> query).
+            // query's own) with the tile-wide bound words plus the keys whose bound, among the
+            // queries, is this one or a later one.  Every key of the other tiles is visible (to all but a <CL> query).
             const int t = vq - v0;  // the query's own column, the last visible one
-            const uint4 hw = khid[cs];
-            vw[0] = hw.x;
-            vw[1] = hw.y;
-            vw[2] = hw.z;
-            vw[3] = hw.w;
-            const int nr = kn[cs];
-#pragma unroll 1
-            for (int e = 0; e < nr; ++e) {
-              const uint4 rb = rbits[cs][e];
-              const uint32_t on = rhid[cs][e] >= iq ? 0xFFFFFFFFu : 0u;
-              vw[0] |= rb.x & on;
-              vw[1] |= rb.y & on;
-              vw[2] |= rb.z & on;
-              vw[3] |= rb.w & on;
-            }
+            const uint4 hw = khid[cs], he = kend[cs];
+            const uint4 af = kafter[cs][__popc(he.x & low_bits(r)) + __popc(he.y & low_bits(r - 32)) +
+                                        __popc(he.z & low_bits(r - 64)) + __popc(he.w & low_bits(r - 96))];
+            vw[0] = hw.x | af.x;
+            vw[1] = hw.y | af.y;
+            vw[2] = hw.z | af.z;
+            vw[3] = hw.w | af.w;
             // the causal prefix; a <CL> query sees its own key alone
 #pragma unroll
             for (int u = 0; u < 4; ++u) vw[u] &= low_bits(t + 1 - 32 * u) & ~low_bits(cl_q ? t - 32 * u : 0);
