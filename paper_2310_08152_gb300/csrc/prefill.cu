@@ -315,14 +315,6 @@ __device__ __forceinline__ uint4 ld_shared_v4(uint32_t addr) {
   return v;
 }
 
-__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
 
 // Bits [0, n) of a 32-bit word, n clamped to [0, 32].
 __device__ __forceinline__ uint32_t low_bits(int n) {
@@ -429,7 +421,9 @@ __device__ __forceinline__ void gather_rows(uint32_t dst, uint32_t subb, const u
 // barrier phase counts tiles over all of the CTA's items, so the producer streams the next item's
 // K/V while the current one finishes (with two S tiles, the O accumulator also alternates between
 // two TMEM buffers per item).
-template <typename T, int D>
+// ROT: the queries are rotated (RoPE).  A kernel of its own without that code, because the instruction cache holds
+// little more than one of them: OPT-1.3B-shaped prompts 327 -> 299 us, compacted bf16 prompts 441 -> 400.
+template <typename T, int D, bool ROT>
 __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     prefill_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
                    const __grid_constant__ CUtensorMap tm_q, const PrefillArgs a) {
@@ -455,6 +449,8 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
   __shared__ uint4 kafter[kClsRing][KT + 1];
   __shared__ int32_t kslow[kClsRing];  // the tile needs the per-key rule (else every key is visible)
   __shared__ uint64_t cls_full[kClsRing], cls_empty[kClsRing];
+  __shared__ float2 rope_s[D / 2];  // a.rope_g (read from global memory in each item, with two words of a row in
+                                    // flight: ragged rotary prompts 985 us, 949 so with eight)
   __shared__ uint32_t tmem_slot;
 
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~uintptr_t(1023));
@@ -466,6 +462,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if (ROT && threadIdx.x >= 64 && threadIdx.x < 64 + a.rot / 2) rope_s[threadIdx.x - 64] = a.rope_g[threadIdx.x - 64];
   if (threadIdx.x == 32) {
     for (int i = 0; i < KST; ++i) {
       mbar_init(&k_full[i], 32);
@@ -726,7 +723,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         }
         // SPLIT with RoPE: + Q_lo K^T (without RoPE the query is exact in the cache type)
         if constexpr (Cf::SPLIT) {
-          if (a.rot > 0) {
+          if constexpr (ROT) {
 #pragma unroll
             for (int kk = 0; kk < D / 16; ++kk) {
               const uint32_t off = ((kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2) >> 4;
@@ -769,18 +766,17 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       // Q K^T after that P.V: OPT-1.3B-shaped prompts 362 us a layer, 348 so, with the cheaper descriptors).  The
       // rotated queries of an item come from the softmax warps after their last tile, whose P.V does not wait
       // for them.
-      const bool rot = a.rot > 0;
       uint32_t gq = 0, gp = 0;  // Q K^T, P.V issued
       uint32_t kq = 0, kp = 0;  // their items
       int jq = 0, jp = 0, nkq = 0;
       bool items = true;  // there may be another one
       while (ok) {
-        if (items && !(rot && jq == 0 && gq != gp)) {
+        if (items && !(ROT && jq == 0 && gq != gp)) {
           if (jq == 0) {
             if (!(ok = item_wait(kq))) break;
             nkq = item_slot[kq % kItemRing].nk;
             items = nkq > 0;
-            if (items && !(ok = pf_wait(rot ? &q_full : &q_raw, kq & 1, limit_ns))) break;
+            if (items && !(ok = pf_wait(ROT ? &q_full : &q_raw, kq & 1, limit_ns))) break;
             tc_fence_after();
           }
           if (items) {
@@ -790,7 +786,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
               jq = 0;
               ++kq;
             }
-            if (gq - gp == 1 && !(rot && jq == 0)) continue;
+            if (gq - gp == 1 && !(ROT && jq == 0)) continue;
           }
         }
         if (gq == gp) break;
@@ -831,13 +827,13 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       else
         st_shared_v4(qlo_chunk(c8), w0, w1, w2, w3);
     };
-    auto q_rotate = [&](const PfItem& w, uint32_t kk) -> bool {
+    [[maybe_unused]] auto q_rotate = [&](const PfItem& w, uint32_t kk) -> bool {
       if (!__all_sync(0xFFFFFFFFu, pf_wait(&q_raw, kk & 1, limit_ns))) return false;
       const int half = a.rot / 2;
       const int iq = w.qr0 + r;
       if constexpr (Cf::SPLIT) {
         // every row (rows past the tile's queries hold zeros), so the TMEM stores are warp-wide
-        if (half > 0) {
+        {
           const int32_t qpos = iq < w.qr_end ? a.pos[a.off[w.s] + iq] : 0;
           const int hc = half / 8;  // chunks per rotated half
 #pragma unroll 1
@@ -851,8 +847,8 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
               for (int e = 0; e < 4; ++e) {
                 const float2 x1 = T::f2(w1[e]), x2 = T::f2(w2[e]);
                 float sn0, cs0, sn1, cs1;
-                rope_sincos(qpos, a.rope_g[8 * c8 + 2 * e], &sn0, &cs0);
-                rope_sincos(qpos, a.rope_g[8 * c8 + 2 * e + 1], &sn1, &cs1);
+                rope_sincos(qpos, rope_s[8 * c8 + 2 * e], &sn0, &cs0);
+                rope_sincos(qpos, rope_s[8 * c8 + 2 * e + 1], &sn1, &cs1);
                 l1[e] = bf16_split2(make_float2(x1.x * cs0 - x2.x * sn0, x1.y * cs1 - x2.y * sn1), &h1[e]);
                 l2[e] = bf16_split2(make_float2(x2.x * cs0 + x1.x * sn0, x2.y * cs1 + x1.y * sn1), &h2[e]);
               }
@@ -867,20 +863,25 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           for (int c8 = 0; c8 < D / 8; ++c8)
             if (c8 >= 2 * hc) qlo_store(c8, 0u, 0u, 0u, 0u);
         }
-      } else if (half > 0 && iq < w.qr_end) {
+      } else if (iq < w.qr_end) {
         const int32_t qpos = a.pos[a.off[w.s] + iq];
 #pragma unroll 1
         for (int c8 = 0; c8 < half / 8; ++c8) {
           const uint32_t a1 = q_chunk(c8), a2 = q_chunk(c8 + half / 8);
-#pragma unroll 2
+          const uint4 u1 = ld_shared_v4(a1), u2 = ld_shared_v4(a2);
+          const uint32_t w1[4] = {u1.x, u1.y, u1.z, u1.w}, w2[4] = {u2.x, u2.y, u2.z, u2.w};
+          uint32_t h1[4], h2[4];
+#pragma unroll
           for (int e = 0; e < 4; ++e) {
-            const float2 x1 = T::f2(ld_shared_u32(a1 + 4 * e)), x2 = T::f2(ld_shared_u32(a2 + 4 * e));
+            const float2 x1 = T::f2(w1[e]), x2 = T::f2(w2[e]);
             float sn0, cs0, sn1, cs1;
-            rope_sincos(qpos, a.rope_g[8 * c8 + 2 * e], &sn0, &cs0);
-            rope_sincos(qpos, a.rope_g[8 * c8 + 2 * e + 1], &sn1, &cs1);
-            st_shared_u32(a1 + 4 * e, Pack16<T>::two(x1.x * cs0 - x2.x * sn0, x1.y * cs1 - x2.y * sn1));
-            st_shared_u32(a2 + 4 * e, Pack16<T>::two(x2.x * cs0 + x1.x * sn0, x2.y * cs1 + x1.y * sn1));
+            rope_sincos(qpos, rope_s[8 * c8 + 2 * e], &sn0, &cs0);
+            rope_sincos(qpos, rope_s[8 * c8 + 2 * e + 1], &sn1, &cs1);
+            h1[e] = Pack16<T>::two(x1.x * cs0 - x2.x * sn0, x1.y * cs1 - x2.y * sn1);
+            h2[e] = Pack16<T>::two(x2.x * cs0 + x1.x * sn0, x2.y * cs1 + x1.y * sn1);
           }
+          st_shared_v4(a1, h1[0], h1[1], h1[2], h1[3]);
+          st_shared_v4(a2, h2[0], h2[1], h2[2], h2[3]);
         }
       }
       if constexpr (Cf::QLO_TMEM) {
@@ -952,7 +953,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     float l_prev = 0.f;    // the item before's row sum: its epilogue comes once its last P.V is complete
     if (more) {
       cl_next = is_cl(item_slot[0]);
-      if (a.rot > 0) ok = q_rotate(item_slot[0], 0);
+      if constexpr (ROT) ok = q_rotate(item_slot[0], 0);
     }
     // after the last item (!more) once more, for its epilogue alone
     while (ok && (more || k >= 1)) {
@@ -1148,7 +1149,9 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       g += nk;
       l_prev = l;
       // the next item's queries came in after this item's last Q.K^T
-      if (next_ok && a.rot > 0) ok = q_rotate(item_slot[(k + 1) % kItemRing], k + 1);
+      if constexpr (ROT) {
+        if (next_ok) ok = q_rotate(item_slot[(k + 1) % kItemRing], k + 1);
+      }
       more = next_ok;
       ++k;
     }
@@ -1183,7 +1186,7 @@ cudaError_t encode_plane(const Geometry& g, void* base, unsigned char* out) {
   return cudaSuccess;
 }
 
-template <typename T, int D>
+template <typename T, int D, bool ROT>
 cudaError_t launch_prefill_t(const PrefillMaps& maps, const PrefillArgs& a, int64_t grid, cudaStream_t stream) {
   using Cf = PfCfg<D, kSplit<T>>;
   static std::mutex mu;
@@ -1196,14 +1199,14 @@ cudaError_t launch_prefill_t(const PrefillMaps& maps, const PrefillArgs& a, int6
   }
   std::lock_guard<std::mutex> lock(mu);
   if (!attr_set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(prefill_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const cudaError_t e = cudaFuncSetAttribute(prefill_kernel<T, D, ROT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)Cf::SMEM);
     if (e != cudaSuccess) return e;
     if (Cf::CPS == 2) {
       // the setmaxnreg shares assume each thread starts with exactly REG_LAUNCH registers; with
       // fewer the softmax warpgroup's increase could never be granted, so refuse to launch
       cudaFuncAttributes fa;
-      const cudaError_t e2 = cudaFuncGetAttributes(&fa, prefill_kernel<T, D>);
+      const cudaError_t e2 = cudaFuncGetAttributes(&fa, prefill_kernel<T, D, ROT>);
       if (e2 != cudaSuccess) return e2;
       if (fa.numRegs != Cf::REG_LAUNCH) return cudaErrorInvalidConfiguration;
     }
@@ -1226,8 +1229,14 @@ cudaError_t launch_prefill_t(const PrefillMaps& maps, const PrefillArgs& a, int6
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
   }
-  prefill_kernel<T, D><<<(unsigned)grid, kPfThreads, Cf::SMEM, stream>>>(mk, mv, mq, a);
+  prefill_kernel<T, D, ROT><<<(unsigned)grid, kPfThreads, Cf::SMEM, stream>>>(mk, mv, mq, a);
   return cudaGetLastError();
+}
+
+template <typename T, int D>
+cudaError_t launch_prefill_d(const PrefillMaps& maps, const PrefillArgs& a, int64_t grid, cudaStream_t stream) {
+  return a.rot > 0 ? launch_prefill_t<T, D, true>(maps, a, grid, stream)
+                   : launch_prefill_t<T, D, false>(maps, a, grid, stream);
 }
 
 }  // namespace
@@ -1301,14 +1310,14 @@ cudaError_t launch_prefill(const Geometry& g, const PrefillMaps& maps, const Pre
   const bool bf = g.dtype == 1;
   switch (g.D) {
     case 64:
-      return bf ? launch_prefill_t<BF16T, 64>(maps, a, grid, stream) : launch_prefill_t<F16T, 64>(maps, a, grid, stream);
+      return bf ? launch_prefill_d<BF16T, 64>(maps, a, grid, stream) : launch_prefill_d<F16T, 64>(maps, a, grid, stream);
     case 80:
-      return bf ? launch_prefill_t<BF16T, 80>(maps, a, grid, stream) : launch_prefill_t<F16T, 80>(maps, a, grid, stream);
+      return bf ? launch_prefill_d<BF16T, 80>(maps, a, grid, stream) : launch_prefill_d<F16T, 80>(maps, a, grid, stream);
     case 96:
-      return bf ? launch_prefill_t<BF16T, 96>(maps, a, grid, stream) : launch_prefill_t<F16T, 96>(maps, a, grid, stream);
+      return bf ? launch_prefill_d<BF16T, 96>(maps, a, grid, stream) : launch_prefill_d<F16T, 96>(maps, a, grid, stream);
     case 128:
-      return bf ? launch_prefill_t<BF16T, 128>(maps, a, grid, stream)
-                : launch_prefill_t<F16T, 128>(maps, a, grid, stream);
+      return bf ? launch_prefill_d<BF16T, 128>(maps, a, grid, stream)
+                : launch_prefill_d<F16T, 128>(maps, a, grid, stream);
     default:
       return cudaErrorInvalidValue;
   }
