@@ -447,6 +447,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
   // before: OPT-1.3B-shaped prompts 333 us, 327 so).
   __shared__ uint4 khid[kClsRing], kend[kClsRing];
   __shared__ uint4 kafter[kClsRing][KT + 1];
+  __shared__ int8_t bound[128];  // of the tile being sorted
   __shared__ int32_t kslow[kClsRing];  // the tile needs the per-key rule (else every key is visible)
   __shared__ uint64_t cls_full[kClsRing], cls_empty[kClsRing];
   __shared__ float2 rope_s[D / 2];  // a.rope_g (read from global memory in each item, with two words of a row in
@@ -542,46 +543,51 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         const int cs = (int)(cg % kClsRing);
         // per-key mask bounds of the tile ((hid << 1) | is_cl) sorted into the classes above; the causal
         // part (i <= iq) is left to each query
-        constexpr int NW = (KT + 31) / 32;
-        uint32_t ok_w[4] = {0u, 0u, 0u, 0u}, end_w[4] = {0u, 0u, 0u, 0u};
-        int hp[NW];  // the key's bound from the first query on when it falls among the queries, else -1
-#pragma unroll
-        for (int w4 = 0; w4 < NW; ++w4) {
-          const int v = v0 + lane + 32 * w4;
-          int hid = w.qr_end;  // a row that no span hides
-          if (lane + 32 * w4 >= KT || v >= keys || (v >= before && v < own))
-            hid = -2;  // no key
-          else if (v >= own)
-            hid = a.meta[w.moff + w.qr0 + (v - own)] >> 1;
-          else if (v >= w.n_c)
-            hid = a.meta[w.moff + w.b0 + (v - w.n_c)] >> 1;
-          ok_w[w4] = __ballot_sync(0xFFFFFFFFu, hid >= w.qr_end - 1);
-          hp[w4] = hid >= w.qr0 && hid < w.qr_end - 1 ? hid - w.qr0 : -1;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) end_w[u] |= hp[w4] >> 5 == u ? 1u << (hp[w4] & 31) : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) end_w[u] = __reduce_or_sync(0xFFFFFFFFu, end_w[u]);
         if (cg >= kClsRing && !pf_wait(&cls_empty[cs], ((cg / kClsRing) - 1) & 1, limit_ns)) {
           ok = false;
           break;
         }
+        uint32_t* hid_w = reinterpret_cast<uint32_t*>(&khid[cs]);
+        uint32_t* end_w = reinterpret_cast<uint32_t*>(&kend[cs]);
+        uint32_t my_end = 0u;  // word `lane` of kend
+        constexpr int NW = (KT + 31) / 32;
+        // (a rolled loop: this warp has some time, the instruction cache no room -- unrolled OPT-1.3B-shaped prompts
+        // take 302 us, 293 so; with the loops below rolled too, 299, and one prompt of 300 tokens 12.0 for 11.0)
+#pragma unroll 1
+        for (int w4 = 0; w4 < NW; ++w4) {
+          const int c = lane + 32 * w4, v = v0 + c;
+          int hid = w.qr_end;  // a row that no span hides
+          if (c >= KT || v >= keys || (v >= before && v < own))
+            hid = -2;  // no key
+          else if (v >= w.n_c)
+            hid = a.meta[w.moff + (v >= own ? w.qr0 + (v - own) : w.b0 + (v - w.n_c))] >> 1;
+          const uint32_t all = __ballot_sync(0xFFFFFFFFu, hid >= w.qr_end - 1);
+          // the key's bound from the first query on when it falls among the queries, else -1
+          const int h = hid >= w.qr0 && hid < w.qr_end - 1 ? hid - w.qr0 : -1;
+          bound[c] = (int8_t)h;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const uint32_t e = __reduce_or_sync(0xFFFFFFFFu, h >> 5 == u ? 1u << (h & 31) : 0u);
+            if (lane == u) my_end |= e;
+          }
+          if (lane == 0) hid_w[w4] = all;
+        }
+        if (lane < 4) end_w[lane] = my_end;
+        __syncwarp();
         int n_end = 0;
 #pragma unroll 1
         for (int u = 0; u < 4; ++u) {
-          uint32_t left = u == 0 ? end_w[0] : u == 1 ? end_w[1] : u == 2 ? end_w[2] : end_w[3];
-          for (; left != 0u; left &= left - 1u, ++n_end) {
+          for (uint32_t left = __shfl_sync(0xFFFFFFFFu, my_end, u); left != 0u; left &= left - 1u, ++n_end) {
             const int h = 32 * u + __ffs(left) - 1;
             uint32_t m[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-            for (int w4 = 0; w4 < NW; ++w4) m[w4] = __ballot_sync(0xFFFFFFFFu, hp[w4] >= h);
+            for (int w4 = 0; w4 < NW; ++w4) m[w4] = __ballot_sync(0xFFFFFFFFu, bound[lane + 32 * w4] >= h);
             if (lane == 0) kafter[cs][n_end] = make_uint4(m[0], m[1], m[2], m[3]);
           }
         }
+        __syncwarp();
         if (lane == 0) {
           kafter[cs][n_end] = make_uint4(0u, 0u, 0u, 0u);
-          khid[cs] = make_uint4(ok_w[0], ok_w[1], ok_w[2], ok_w[3]);
-          kend[cs] = make_uint4(end_w[0], end_w[1], end_w[2], end_w[3]);
           // per-key masking is needed when a key's visibility differs between the tile's queries: bounds
           // among them, and keys at or past the first query (the causal rule); and for columns without a key
           kslow[cs] = n_end > 0 || v0 + KT > before;
@@ -912,7 +918,9 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     auto epilogue = [&](uint32_t kk, float l_) {
       const PfItem& w = item_slot[kk % kItemRing];
       const uint32_t o_t = tl + Cf::O_COL + (Cf::OBUF == 2 ? (kk & 1) * D : 0);
-      const float inv = 1.f / l_;
+      float inv;  // 1 / l_: the approximation and a Newton step
+      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(l_));
+      inv = __fmaf_rn(inv, __fmaf_rn(-l_, inv, 1.f), inv);
       const int64_t row8 = (int64_t)8 * a.H * D;
       float* o_row = a.out + ((int64_t)(w.tok0 + warp * 32 + (lane >> 2)) * a.H + w.h) * D + 2 * (lane & 3);
       constexpr int CO = D % 32 == 0 ? 32 : 16;  // columns at a time
