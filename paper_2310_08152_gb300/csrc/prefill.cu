@@ -906,9 +906,8 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     int64_t g = 0;    // tiles consumed
     uint32_t k = 0;   // items done
     uint32_t cg = 0;  // sorted key tiles consumed
-    // waits of a whole warp
-    // -- with 64 keys a tile the warp's lanes agree on them once a tile, as a share of its work a vote at each is
-    // dear (compacted bf16 prompts 399 -> 387 us, bf16 heads of 64 396 -> 383; with more keys nothing or a loss)
+    // waits of a whole warp -- with 64 keys a tile the lanes agree on them once a tile: as a share of its work a vote at
+    // each is dear (compacted bf16 prompts 399 -> 387 us, bf16 heads of 64 396 -> 383; with more keys it is no gain)
     [[maybe_unused]] bool got_all = true;
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
       const bool got = pf_wait(bar, parity, limit_ns);
