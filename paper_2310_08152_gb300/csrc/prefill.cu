@@ -903,7 +903,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       return w.qr0 + r < w.qr_end && (__ldg(a.meta + w.moff + w.qr0 + r) & 1);
     };
 
-    int64_t g = 0;    // tiles consumed
+    uint32_t g = 0;   // tiles consumed
     uint32_t k = 0;   // items done
     uint32_t cg = 0;  // sorted key tiles consumed
     // waits of a whole warp -- with 64 keys a tile the lanes agree on them once a tile: as a share of its work a vote at
@@ -972,14 +972,15 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     // after the last item (!more) once more, for its epilogue alone
     while (ok && (more || k >= 1)) {
       const PfItem& w = item_slot[k % kItemRing];
-      const int nk = more ? w.nk : 1, n_c = w.n_c;
+      const int nk = more ? w.nk : 1, n_c = w.n_c, step = w.odd ? -KT : KT;
+      int v0 = KT * w.key_tile(0);  // the tile's first key
       const int vq = w.own(KT) + r;  // its own key
       const bool cl_q = cl_next;
       bool next_ok = false;  // there is another item
       const uint32_t o_t = tl + Cf::O_COL + (Cf::OBUF == 2 ? (k & 1) * D : 0);
       float m = -INFINITY, l = 0.f;
-      for (int j = 0; j < nk; ++j) {
-        const int64_t gj = g + j;
+      for (int j = 0; j < nk; ++j, v0 += step) {
+        const uint32_t gj = g + j;
         const int sb = (int)(gj % SBUF);
         const uint32_t p_tl = tl + (Cf::PSEP ? Cf::P_COL : sb * KT);
         float sv[CW], alpha = 1.f, ref = 0.f, m_new = 0.f;
@@ -1016,10 +1017,9 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         // the item before, whose last P.V that was.
         bool pv_wait = gj >= 1;
         if (more) {
-          const int v0 = KT * w.key_tile(j);    // the tile's first key
           const bool sorted = v0 + KT > n_c;    // warp 4 has sorted its keys
           const int cs = (int)(cg % kClsRing);
-          ok = warp_wait(&s_full[sb], (uint32_t)(gj / SBUF) & 1) &&
+          ok = warp_wait(&s_full[sb], (gj / SBUF) & 1) &&
                (!sorted || warp_wait(&cls_full[cs], (cg / kClsRing) & 1));
           // warp 4 takes the next item as soon as this item's last K tile is on its way
           if (ok && j == nk - 1) ok = __all_sync(0xFFFFFFFFu, item_wait(k + 1));
@@ -1108,7 +1108,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           alpha = !move || m == -INFINITY ? 1.f : ex2(m - ref);
           if (pv_wait && __any_sync(0xFFFFFFFFu, alpha != 1.f)) {
             pv_wait = false;
-            ok = warp_wait(&pv_done, (uint32_t)(gj - 1) & 1);
+            ok = warp_wait(&pv_done, (gj - 1) & 1);
             if (!ok) break;
             tc_fence_after();
 #pragma unroll 1
@@ -1134,7 +1134,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           }
         }
         if (pv_wait) {
-          ok = warp_wait(&pv_done, (uint32_t)(gj - 1) & 1);
+          ok = warp_wait(&pv_done, (gj - 1) & 1);
           if (!ok) break;
         }
         tc_fence_after();
