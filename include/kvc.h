@@ -181,6 +181,12 @@ kvc_status kvc_required_bytes(const kvc_config* cfg, size_t* k_bytes, size_t* v_
 kvc_status kvc_create(const kvc_config* cfg, kvc_cache** out);
 void kvc_destroy(kvc_cache* cache);
 
+/* Uploads go through a ring in pinned host memory, which the cache allocates at its first append unless the
+ * caller hands it at least kvc_staging_bytes(cache) bytes of its own before that (KVC_ERR_STATE after it).
+ * The caller's memory is 16-byte aligned, pinned, and the cache's until kvc_destroy returns. */
+size_t kvc_staging_bytes(const kvc_cache* cache);
+kvc_status kvc_set_staging(kvc_cache* cache, void* pinned, size_t bytes);
+
 /* The cache's span book (read-only view: positions, pending spans, lengths, layout). */
 const kvc_book* kvc_get_book(const kvc_cache* cache);
 
@@ -203,6 +209,12 @@ kvc_status kvc_append(kvc_cache* cache, int layer, const void* k, const void* v,
  * with kvc_compress_spans).  Capacity counts only stored rows.  Same arguments as kvc_append. */
 kvc_status kvc_append_free_closed(kvc_cache* cache, int layer, const void* k, const void* v, const int32_t* n_new,
                                   const int32_t* pos, const uint8_t* kinds, void* stream);
+
+/* kvc_append (free_closed == 0) or kvc_append_free_closed (else) of tokens at their tied positions
+ * (kvc_book_next_positions), for layer -1 or 0: pos_out[N] (host) receives the positions.  On an
+ * error nothing is appended and pos_out is undefined. */
+kvc_status kvc_append_tied(kvc_cache* cache, int layer, const void* k, const void* v, const int32_t* n_new,
+                           const uint8_t* kinds, int32_t* pos_out, int free_closed, void* stream);
 
 /* Free closed spans (Sec. 3.1): for each listed (seq, cl, cr) -- history indices of a closed,
  * not yet freed span -- drop its rows (<CL> and the enclosed tokens under the paper policy, only

@@ -59,7 +59,8 @@ def _stream_handle(stream) -> Optional[int]:
     if stream is None:
         import torch
 
-        return torch.cuda.current_stream().cuda_stream
+        # the handle alone: torch.cuda.current_stream() builds a Stream object (3.8 us a call, 0.4 so)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -123,12 +124,14 @@ def kvc_book_compress(book: int, seq, cl, cr):
 
 
 def kvc_book_pending_spans(book: int, seq: int):
-    n = ctypes.c_int64()
-    _check(lib().kvc_book_pending_spans(book, seq, None, None, 0, ctypes.byref(n)))
-    cl = np.empty(max(n.value, 1), np.int64)
-    cr = np.empty(max(n.value, 1), np.int64)
-    _check(lib().kvc_book_pending_spans(book, seq, cl.ctypes.data, cr.ctypes.data, n.value, ctypes.byref(n)))
-    return [(int(cl[i]), int(cr[i])) for i in range(n.value)]
+    n = ctypes.c_int64(64)  # room for most; more take a second call
+    spans = None
+    while spans is None or n.value > spans.shape[1]:
+        spans = np.empty((2, n.value), np.int64)
+        at = spans.ctypes.data
+        _check(lib().kvc_book_pending_spans(book, seq, at, at + 8 * spans.shape[1], spans.shape[1], ctypes.byref(n)))
+    cl, cr = spans[:, :n.value].tolist()
+    return list(zip(cl, cr))
 
 
 def kvc_book_lengths(book: int, b: int):
@@ -275,6 +278,20 @@ def kvc_append_free_closed(cache: int, layer: int, k, v, n_new, pos, kinds, stre
                                         _stream_handle(stream)))
 
 
+def kvc_append_tied(cache: int, layer: int, k, v, n_new, kinds, pos_out, free_closed: bool, stream=None):
+    """kvc_append (or kvc_append_free_closed) at the tied positions, which go into pos_out."""
+    _check(lib().kvc_append_tied(cache, layer, k.data_ptr(), v.data_ptr(), n_new.ctypes.data, kinds.ctypes.data,
+                                 pos_out.ctypes.data, 1 if free_closed else 0, _stream_handle(stream)))
+
+
+def kvc_staging_bytes(cache: int) -> int:
+    return lib().kvc_staging_bytes(cache)
+
+
+def kvc_set_staging(cache: int, pinned):
+    _check(lib().kvc_set_staging(cache, pinned.data_ptr(), pinned.numel() * pinned.element_size()))
+
+
 def kvc_compress_spans(cache: int, seq, cl, cr, stream=None):
     seq, cl, cr = _np(seq, np.int32), _np(cl, np.int64), _np(cr, np.int64)
     _check(lib().kvc_compress_spans(cache, seq.ctypes.data, cl.ctypes.data, cr.ctypes.data, seq.size,
@@ -380,6 +397,10 @@ class KVCache:
         cfg.workspace, cfg.workspace_bytes = self.workspace.data_ptr(), sizes["workspace"]
         self._cfg = cfg
         self.handle = kvc_create(cfg)
+        # the upload ring, from torch's pool of pinned memory (allocating and freeing it with each cache takes
+        # about 300 us); kvc_destroy waits for the device before the pool gets it back
+        self.staging = torch.empty(kvc_staging_bytes(self.handle), dtype=torch.uint8, pin_memory=True)
+        kvc_set_staging(self.handle, self.staging)
         self.book = Book(self.b, cap, policy, _handle=lib().kvc_get_book(self.handle))
 
     # views of the device layout (rows of d_head elements)
@@ -399,12 +420,20 @@ class KVCache:
         free_closed: free spans opened and closed among these tokens as they are written."""
         n_new = _np(n_new, np.int32)
         kinds = _np(kinds, np.uint8)
-        if layer <= 0 and pos is None:
-            pos = self.book.next_positions(n_new, kinds)
-        N = int(n_new.sum())
-        nl = self.M if layer < 0 else 1
-        _dev(k, "k", self.torch_dtype, nl * N * self.H * self.d)
-        _dev(v, "v", self.torch_dtype, nl * N * self.H * self.d)
+        tied = layer <= 0 and pos is None
+        N = int(np.add.reduce(n_new))
+        n = (self.M if layer < 0 else 1) * N * self.H * self.d
+        try:
+            _dev(k, "k", self.torch_dtype, n)
+            _dev(v, "v", self.torch_dtype, n)
+        except ValueError:
+            if tied:
+                self.book.next_positions(n_new, kinds)  # its errors come first
+            raise
+        if tied:
+            pos = np.empty(max(N, 1), np.int32)
+            kvc_append_tied(self.handle, layer, k, v, n_new, kinds, pos, free_closed, stream)
+            return pos[:N]
         (kvc_append_free_closed if free_closed else kvc_append)(self.handle, layer, k, v, n_new, pos, kinds, stream)
         return pos
 
@@ -425,7 +454,8 @@ class KVCache:
         """Masked prefill of the last n_q[s] tokens of every sequence s (q: [sum n_q, H, d_head])."""
         import torch
 
-        n_tok = int(np.sum(n_q))
+        n_q = _np(n_q, np.int32)
+        n_tok = int(np.add.reduce(n_q))
         _dev(q, "q", self.torch_dtype, n_tok * self.H * self.d)
         if out is None:
             out = torch.empty(n_tok, self.H, self.d, dtype=torch.float32, device=q.device)

@@ -51,9 +51,12 @@ SIGNATURES = [
     ("kvc_required_bytes", c_int, [P, P, P, P, P]),
     ("kvc_create", c_int, [P, P]),
     ("kvc_destroy", None, [P]),
+    ("kvc_staging_bytes", c_size_t, [P]),
+    ("kvc_set_staging", c_int, [P, P, c_size_t]),
     ("kvc_get_book", P, [P]),
     ("kvc_append", c_int, [P, c_int, P, P, P, P, P, P]),
     ("kvc_append_free_closed", c_int, [P, c_int, P, P, P, P, P, P]),
+    ("kvc_append_tied", c_int, [P, c_int, P, P, P, P, P, c_int, P]),
     ("kvc_compress_spans", c_int, [P, P, P, P, c_int, P]),
     ("kvc_decode_attention", c_int, [P, c_int, P, c_float, P, P]),
     ("kvc_decode_attention_static_scratch", c_int, [P, c_int, P, c_float, P, P]),

@@ -158,15 +158,20 @@ void Book::apply_append(const int32_t* n_new, const uint8_t* kinds, const int32_
     const int64_t T0 = (int64_t)q.kind.size();
     int64_t stored_new = 0;
     bool freed_any = false;
-    for (int t = 0; t < n_new[s]; ++t) {
-      uint8_t k = kinds[off + t];
-      int64_t j = (int64_t)q.kind.size();
-      q.kind.push_back(k);
-      q.pos.push_back(pos[off + t]);
-      stored_new += kept ? kept[off + t] : 1;
-      if (k == NORMAL) {
-        q.normals += 1;
-      } else if (k == CL) {
+    const int64_t n = n_new[s];
+    q.kind.insert(q.kind.end(), kinds + off, kinds + off + n);
+    q.pos.insert(q.pos.end(), pos + off, pos + off + n);
+    if (kept)
+      for (int64_t t = 0; t < n; ++t) stored_new += kept[off + t];
+    else
+      stored_new = n;
+    int64_t sentinels = 0;
+    for (int64_t t = 0; t < n; ++t) {
+      const uint8_t k = kinds[off + t];
+      if (k == NORMAL) continue;
+      ++sentinels;
+      const int64_t j = T0 + t;
+      if (k == CL) {
         Span sp;
         sp.cl = j;
         q.spans.push_back(sp);
@@ -183,6 +188,7 @@ void Book::apply_append(const int32_t* n_new, const uint8_t* kinds, const int32_
         }
       }
     }
+    q.normals += n - sentinels;
     if (freed_any) rebuild_prefix(q);
     if (policy_ == POLICY_LOCAL) {
       const int64_t T = (int64_t)q.kind.size();

@@ -134,11 +134,24 @@ kvc_status check_config(const kvc_config* c, int64_t* C_out) {
 class PinnedRing {
  public:
   ~PinnedRing() { release(); }
-  cudaError_t init(size_t bytes) {
-    cap_ = align_up(bytes, 256);
-    return cudaHostAlloc(reinterpret_cast<void**>(&base_), cap_, cudaHostAllocDefault);
+  // own: memory of the caller's (at least ring_bytes(bytes) of it), else the ring allocates
+  cudaError_t init(size_t bytes, void* own) {
+    cap_ = ring_bytes(bytes);
+    borrowed_ = own != nullptr;
+    if (const cudaError_t e = cudaGetDevice(&device_); e != cudaSuccess) return e;
+    base_ = static_cast<unsigned char*>(own);
+    return own ? cudaSuccess : cudaHostAlloc(reinterpret_cast<void**>(&base_), cap_, cudaHostAllocDefault);
   }
+  static size_t ring_bytes(size_t bytes) { return align_up(bytes, 256); }
   void release() {
+    // freeing pinned memory waits for the device; borrowed memory is given back only after the same wait
+    if (borrowed_ && base_) {
+      int dev = -1;
+      if (cudaGetDevice(&dev) == cudaSuccess && dev != device_) cudaSetDevice(device_);
+      cudaDeviceSynchronize();
+      if (dev >= 0 && dev != device_) cudaSetDevice(dev);
+      base_ = nullptr;
+    }
     for (auto& p : pending_) cudaEventDestroy(p.ev);
     for (auto e : free_) cudaEventDestroy(e);
     pending_.clear();
@@ -192,6 +205,8 @@ class PinnedRing {
     cudaEvent_t ev;
   };
   unsigned char* base_ = nullptr;
+  bool borrowed_ = false;
+  int device_ = 0;
   size_t cap_ = 0, head_ = 0, res_ = 0;
   std::deque<Pending> pending_;
   std::vector<cudaEvent_t> free_;
@@ -214,6 +229,7 @@ struct kvc_cache {
   bool cuda_ready = false;
   int device = -1;
   int num_sms = 0;
+  void* staging = nullptr;  // the caller's memory for the ring
   PinnedRing ring;
   // token batch in progress: layers [0, layers_done) written
   int layers_done = 0;
@@ -291,6 +307,10 @@ struct kvc_cache {
     return b;
   }
 
+  size_t staging_bytes() const {
+    return 2 * ws.dyn_bytes + ws.pre_bytes + 2 * ws.st_rope + kvc::append_maps_bytes(cfg.b) + 65536;
+  }
+
   kvc_status ensure_cuda(cudaStream_t stream) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -301,7 +321,7 @@ struct kvc_cache {
     }
     e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
-    e = ring.init(2 * ws.dyn_bytes + ws.pre_bytes + 2 * ws.st_rope + kvc::append_maps_bytes(cfg.b) + 65536);
+    e = ring.init(staging_bytes(), staging);
     if (e != cudaSuccess) return cuda_fail(e, "cudaHostAlloc (staging ring)");
     // static tables
     const int b = cfg.b, half = std::max(1, cfg.rotary_dim / 2);
@@ -613,6 +633,19 @@ kvc_status kvc_create(const kvc_config* cfg, kvc_cache** out) {
 
 void kvc_destroy(kvc_cache* cache) { delete cache; }
 
+size_t kvc_staging_bytes(const kvc_cache* c) { return c ? PinnedRing::ring_bytes(c->staging_bytes()) : 0; }
+
+kvc_status kvc_set_staging(kvc_cache* c, void* pinned, size_t bytes) {
+  if (!c) return fail(KVC_ERR_INVALID_ARG, "cache is NULL");
+  if (c->cuda_ready) return fail(KVC_ERR_STATE, "the cache has its staging memory already");
+  if (pinned && (reinterpret_cast<uintptr_t>(pinned) & 15))
+    return fail(KVC_ERR_INVALID_ARG, "staging memory must be 16-byte aligned");
+  if (pinned && bytes < kvc_staging_bytes(c))
+    return fail(KVC_ERR_INVALID_ARG, "%zu bytes of staging memory, %zu needed", bytes, kvc_staging_bytes(c));
+  c->staging = pinned;
+  return ok();
+}
+
 const kvc_book* kvc_get_book(const kvc_cache* cache) { return cache ? &cache->bk : nullptr; }
 
 static kvc_status append_impl(kvc_cache* c, int layer, const void* k, const void* v, const int32_t* n_new,
@@ -707,6 +740,15 @@ static kvc_status append_impl(kvc_cache* c, int layer, const void* k, const void
   }
   c->layers_done = m0 + nl;
   return ok();
+}
+
+kvc_status kvc_append_tied(kvc_cache* c, int layer, const void* k, const void* v, const int32_t* n_new,
+                           const uint8_t* kinds, int32_t* pos_out, int free_closed, void* stream) {
+  if (!c) return fail(KVC_ERR_INVALID_ARG, "cache is NULL");
+  if (layer > 0) return fail(KVC_ERR_INVALID_ARG, "layer %d: the positions are given with layer -1 or 0", layer);
+  kvc_status st = kvc_book_next_positions(&c->bk, n_new, kinds, pos_out);
+  if (st != KVC_OK) return st;
+  return append_impl(c, layer, k, v, n_new, pos_out, kinds, stream, free_closed != 0);
 }
 
 kvc_status kvc_append(kvc_cache* c, int layer, const void* k, const void* v, const int32_t* n_new, const int32_t* pos,

@@ -1,0 +1,61 @@
+"""The host side of a call: spans listed past the binding's first buffer, appends at tied positions in one
+call, and uploads staged in the caller's pinned memory."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2310_08152_gb300 as kvc
+
+
+@pytest.mark.parametrize("n", [0, 1, 64, 65, 200])
+def test_pending_spans_of_any_number(n):
+    book = kvc.Book(2, [4 * n + 8] * 2)
+    kinds = np.array([0] + [kvc.CL, 0, kvc.CR] * n, np.uint8)
+    book.append([0, kinds.size], kinds)
+    assert book.pending_spans(1) == [(1 + 3 * i, 3 + 3 * i) for i in range(n)]
+    assert book.pending_spans(0) == []
+
+
+def _tokens(M, H, d, n, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return [torch.randn(M, n, H, d, device="cuda", generator=g).half() for _ in range(2)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("free_closed", [False, True])
+def test_append_at_tied_positions_and_own_staging(free_closed):
+    """KVCache.append without positions (one call, staging from torch's pinned pool) stores what next_positions
+    and an append with them store in a cache whose ring the library allocates."""
+    M, H, d = 2, 4, 64
+    n_new = np.array([7, 0, 5], np.int32)
+    kinds = np.array([0, kvc.CL, 0, 0, kvc.CR, 0, kvc.CL, 0, 0, kvc.CL, 0, kvc.CR], np.uint8)
+    a, b = (kvc.KVCache(M, H, d, [16] * 3) for _ in range(2))
+    kvc._check(kvc.lib().kvc_set_staging(b.handle, None, 0))
+    for x in (a.k, a.v, a.pos, a.orig, b.k, b.v, b.pos, b.orig):
+        x.zero_()
+    k, v = _tokens(M, H, d, 12, 1)
+    pos = a.append(k, v, n_new, kinds, free_closed=free_closed)
+    assert np.array_equal(pos, b.book.next_positions(n_new, kinds))
+    b.append(k, v, n_new, kinds, pos=pos, free_closed=free_closed)
+    torch.cuda.synchronize()
+    for x, y in ((a.k, b.k), (a.v, b.v), (a.pos, b.pos), (a.orig, b.orig)):
+        assert torch.equal(x, y)
+    # what was refused stays refused, with the kinds' errors before the tensors'
+    with pytest.raises(kvc.KvcError) as e:
+        a.append(k[:, :1], v, [0, 0, 1], [kvc.CR])
+    assert e.value.status == 4
+    with pytest.raises(ValueError):
+        a.append(k, v, [1, 0, 0], [0])
+    with pytest.raises(kvc.KvcError) as e:
+        kvc.kvc_append_tied(a.handle, 1, k, v, n_new, kinds, np.empty(12, np.int32), False)
+    assert e.value.status == 1
+    # staging memory: before the first append only, large enough, aligned
+    with pytest.raises(kvc.KvcError) as e:
+        kvc.kvc_set_staging(a.handle, a.staging)
+    assert e.value.status == 5
+    c = kvc.KVCache(M, H, d, [16] * 3)
+    for bad in (c.staging[:-1], torch.empty(c.staging.numel() + 16, dtype=torch.uint8)[1:]):
+        with pytest.raises(kvc.KvcError) as e:
+            kvc.kvc_set_staging(c.handle, bad)
+        assert e.value.status == 1
+    assert a.device_status() == 0 and b.device_status() == 0
