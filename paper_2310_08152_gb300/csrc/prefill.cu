@@ -397,8 +397,10 @@ __device__ __forceinline__ PfItem pf_item(const PrefillArgs& a, int64_t it) {
 // 16-byte asynchronous copies.  Each quarter of the warp, whose 128 bytes are written to shared memory together,
 // covers the chunks of one subtile in as many rows as fill its swizzle pattern, so that they fall into different
 // banks; its quarters lie side by side in the rows, as far as the row goes (96 columns: 621 us with lanes in
-// row order, 577 so).  The steps of a row of the loop wait on shuffles, so they are unrolled where the code has
-// room (128 columns: 657 us by fours, 592 by eights; 64 columns: 358 by fours, 353 by twos, 372 one by one).
+// row order, 577 so).  The gathers bound tiles of many short runs: few instructions a step and many steps in flight,
+// as far as the instruction cache has room (OPT-1.3B-shaped prompts, interiors of 32 / 8: 292 / 445 us with the
+// swizzle worked out per step, two of a group's eight steps unrolled; so 291 / 443 with two, 271 / 393 with four,
+// 286 / 419 with eight; 80, 96, 128 columns: 886, 458, 556 us with four, 867, 446, 490 with all).
 template <int D, int SW, int U0, int NS>
 __device__ __forceinline__ void gather_rows(uint32_t dst, uint32_t subb, const uint16_t* rows, int row, int p0, int kt,
                                             int lane) {
@@ -406,13 +408,16 @@ __device__ __forceinline__ void gather_rows(uint32_t dst, uint32_t subb, const u
   constexpr int RPS = RQ * 4 / NS;          // rows of a step
   const int q = lane >> 3, cw = lane % CH, u = U0 + q % NS, pr = q / NS * RQ + lane % 8 / CH;
   const uint16_t* src = rows + u * (SW / 2) + cw * 8;
-  dst += u * subb + p0 * SW;
-  const int n = kt - p0 < 32 ? kt - p0 : 32;  // a multiple of 16
-#pragma unroll (D == 64 ? 2 : 8)
-  for (int i = 0; i < n; i += RPS) {
-    const int p = i + pr, x = __shfl_sync(0xFFFFFFFFu, row, p);
-    const int phys = cw ^ ((p * SW >> 7) & (CH - 1));
-    cp_async16(dst + p * SW + phys * 16, src + (int64_t)max(x, 0) * D, x < 0 ? 0u : 16u);
+  // the swizzle of row p = pr + i (a step's rows are aligned to their number) is that of pr and that of i
+  constexpr int SH = SW == 128 ? 0 : SW == 64 ? 1 : 2;
+  dst += u * subb + (p0 + pr) * SW;
+  const int c0 = cw ^ (pr >> SH & (CH - 1));
+#pragma unroll (D == 64 ? 4 : 16)
+  for (int i = 0; i < 32; i += RPS) {
+    if (i >= 16 && kt - p0 < 32) break;  // 16 rows
+    const int x = __shfl_sync(0xFFFFFFFFu, row, pr + i);
+    const int phys = c0 ^ (i >> SH & (CH - 1));
+    cp_async16(dst + i * SW + phys * 16, src + (int64_t)max(x, 0) * D, x < 0 ? 0u : 16u);
   }
 }
 
