@@ -247,8 +247,7 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
 
 // Shared-memory matrix descriptor: start address, leading / stride byte offsets, version 1, and
 // the swizzle (layout type 2 = 128 B, 4 = 64 B, 6 = 32 B).  Its low word holds the address and the leading
-// offset, so a tile's descriptors are one word plus constants (addresses stay below 256 KB): built in full for each
-// one, about 100 cycles of the issuing thread per tcgen05.mma.
+// offset, so a tile's descriptors are one word plus constants (addresses stay below 256 KB).
 __device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) { return addr >> 4 | (lbo >> 4) << 16; }
 __device__ __forceinline__ uint64_t desc(uint32_t lo, uint32_t sbo, int sw) {
   const uint32_t hi = (sbo >> 4) | 1u << 14 | (sw == 128 ? 2u : sw == 64 ? 4u : 6u) << 29;
@@ -327,6 +326,13 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   float r;
   asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
+}
+
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+  return one != 0;
 }
 
 // Bounded wait for the phase with the given parity: false after limit_ns (< 2^32).  A few instructions,
@@ -710,66 +716,80 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
   } else if (warp == 5) {
     regs_other();
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    // The whole warp runs this role, and one lane of it issues: with the loop in one lane's branch the operands of
+    // every tcgen05.mma went from the general to the uniform registers, 8 moves and about 100 cycles each, which
+    // bounded the kernel with 13 of them a tile (compacted bf16 prompts 387 us a layer, 323 so; bf16 heads of 64
+    // 384 -> 342; heads of 128 491 -> 466; OPT-1.3B-shaped prompts 272 -> 264).  Conditions are votes, so that the
+    // compiler knows them to be the warp's.
+    {
       constexpr uint32_t idS = mma_idesc(Pack16<T>::kType, 0, kPfRows, KT);
       constexpr uint32_t idO = mma_idesc(Pack16<T>::kType, 1, kPfRows, D);
       constexpr uint32_t SBO = 8 * SW;
       const uint32_t q_d = desc_lo(smem_addr(sm + Cf::Q_OFF), 16);
       [[maybe_unused]] const uint32_t qlo_d = desc_lo(smem_addr(sm + Cf::QLO_OFF), 16);
+      auto uni_wait = [&](uint64_t* bar, uint32_t parity, uint32_t limit) -> bool {
+        return __all_sync(0xFFFFFFFFu, pf_wait(bar, parity, limit));
+      };
       // S = Q K^T of tile gj into its S tile.  One S tile: once the softmax has read S of tile
       // gj - 1.  Two: the tile last held P of tile gj - 2, whose P.V was issued before (tcgen05.mma
       // from one thread run in issue order).
       auto issue_qk = [&](uint32_t gj, bool last) -> bool {
         const int st = (int)(gj % KST), sb = (int)(gj % SBUF);
-        if (!pf_wait(&k_full[st], (gj / KST) & 1, limit_ns)) return false;
-        if (Cf::PSEP && gj >= 1 && !pf_wait(&s_free, (gj - 1) & 1, limit_ns)) return false;
+        if (!uni_wait(&k_full[st], (gj / KST) & 1, limit_ns)) return false;
+        if (Cf::PSEP && gj >= 1 && !uni_wait(&s_free, (gj - 1) & 1, limit_ns)) return false;
         fence_proxy_async_smem();  // gathered rows were written through the generic proxy
         tc_fence_after();
         const uint32_t k_d = desc_lo(smem_addr(sm + Cf::K_OFF + st * Cf::TILE), 16);
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < D / 16; ++kk) {
-          const uint32_t off = ((kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2) >> 4;
-          const uint32_t qoff = ((kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2) >> 4;
-          tc_mma(tmem + sb * KT, desc(q_d + qoff, SBO, SW), desc(k_d + off, SBO, SW), idS, kk > 0);
-        }
-        // SPLIT with RoPE: + Q_lo K^T (without RoPE the query is exact in the cache type)
-        if constexpr (Cf::SPLIT) {
-          if constexpr (ROT) {
+          for (int kk = 0; kk < D / 16; ++kk) {
+            const uint32_t off = ((kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2) >> 4;
+            const uint32_t qoff = ((kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2) >> 4;
+            tc_mma(tmem + sb * KT, desc(q_d + qoff, SBO, SW), desc(k_d + off, SBO, SW), idS, kk > 0);
+          }
+          // SPLIT with RoPE: + Q_lo K^T (without RoPE the query is exact in the cache type)
+          if constexpr (Cf::SPLIT) {
+            if constexpr (ROT) {
 #pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-              const uint32_t off = ((kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2) >> 4;
-              [[maybe_unused]] const uint32_t qoff = ((kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2) >> 4;
-              if constexpr (Cf::QLO_TMEM)
-                tc_mma_ts(tmem + sb * KT, tmem + Cf::QLO_COL + 8 * kk, desc(k_d + off, SBO, SW), idS, 1);
-              else
-                tc_mma(tmem + sb * KT, desc(qlo_d + qoff, SBO, SW), desc(k_d + off, SBO, SW), idS, 1);
+              for (int kk = 0; kk < D / 16; ++kk) {
+                const uint32_t off = ((kk * 16) / SUB * Cf::SUBB + (kk * 16) % SUB * 2) >> 4;
+                [[maybe_unused]] const uint32_t qoff = ((kk * 16) / SUB * Cf::QSUBB + (kk * 16) % SUB * 2) >> 4;
+                if constexpr (Cf::QLO_TMEM)
+                  tc_mma_ts(tmem + sb * KT, tmem + Cf::QLO_COL + 8 * kk, desc(k_d + off, SBO, SW), idS, 1);
+                else
+                  tc_mma(tmem + sb * KT, desc(qlo_d + qoff, SBO, SW), desc(k_d + off, SBO, SW), idS, 1);
+              }
             }
           }
+          tc_commit(&s_full[sb]);
+          tc_commit(&k_empty[st]);
+          if (last) tc_commit(&q_empty);
         }
-        tc_commit(&s_full[sb]);
-        tc_commit(&k_empty[st]);
-        if (last) tc_commit(&q_empty);
+        __syncwarp();
         return true;
       };
       // O += P V of tile gp (8 TMEM columns of P per 16 keys) into o_t; the first of an item: O = P V
       auto issue_pv = [&](uint32_t gp, uint32_t o_t, bool first) -> bool {
         const int st = (int)(gp % VST);
-        if (!pf_wait(&v_full[st], (gp / VST) & 1, limit_ns)) return false;
-        if (!pf_wait(&p_full, gp & 1, limit_ns)) return false;
+        if (!uni_wait(&v_full[st], (gp / VST) & 1, limit_ns)) return false;
+        if (!uni_wait(&p_full, gp & 1, limit_ns)) return false;
         fence_proxy_async_smem();
         tc_fence_after();
         const uint32_t v_d = desc_lo(smem_addr(sm + Cf::V_OFF + st * Cf::TILE), Cf::SUBB);
         const uint32_t p_t = tmem + (Cf::PSEP ? Cf::P_COL : gp % SBUF * KT);
-#pragma unroll
-        for (int kk = 0; kk < KT / 16; ++kk)
-          tc_mma_ts(o_t, p_t + 8 * kk, desc(v_d + kk * SW, SBO, SW), idO, (!first || kk > 0));
-        if constexpr (Cf::SPLIT) {  // + P_lo V
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < KT / 16; ++kk)
-            tc_mma_ts(o_t, p_t + Cf::PLO_COL + 8 * kk, desc(v_d + kk * SW, SBO, SW), idO, 1);
+            tc_mma_ts(o_t, p_t + 8 * kk, desc(v_d + kk * SW, SBO, SW), idO, (!first || kk > 0));
+          if constexpr (Cf::SPLIT) {  // + P_lo V
+#pragma unroll
+            for (int kk = 0; kk < KT / 16; ++kk)
+              tc_mma_ts(o_t, p_t + Cf::PLO_COL + 8 * kk, desc(v_d + kk * SW, SBO, SW), idO, 1);
+          }
+          tc_commit(&pv_done);
+          tc_commit(&v_empty[st]);
         }
-        tc_commit(&pv_done);
-        tc_commit(&v_empty[st]);
+        __syncwarp();
         return true;
       };
       // Q K^T of a tile goes in ahead of P.V of the tile before, also when that is the last of its item: it
@@ -784,16 +804,18 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       while (ok) {
         if (items && !(ROT && jq == 0 && gq != gp)) {
           if (jq == 0) {
-            if (!(ok = item_wait(kq))) break;
+            if (!(ok = __all_sync(0xFFFFFFFFu, item_wait(kq)))) break;
             nkq = item_slot[kq % kItemRing].nk;
-            items = nkq > 0;
-            if (items && !(ok = pf_wait(ROT ? &q_full : &q_raw, kq & 1, limit_ns))) break;
+            items = __any_sync(0xFFFFFFFFu, nkq > 0);
+            if (items && !(ok = uni_wait(ROT ? &q_full : &q_raw, kq & 1, limit_ns))) break;
             tc_fence_after();
           }
           if (items) {
-            if (!(ok = issue_qk(gq, jq == nkq - 1))) break;
+            const bool last = __any_sync(0xFFFFFFFFu, jq == nkq - 1);
+            if (!(ok = issue_qk(gq, last))) break;
             ++gq;
-            if (++jq == nkq) {
+            ++jq;
+            if (last) {
               jq = 0;
               ++kq;
             }
@@ -803,14 +825,15 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         if (gq == gp) break;
         if (!(ok = issue_pv(gp, tmem + Cf::O_COL + (Cf::OBUF == 2 ? (kp & 1) * D : 0), jp == 0))) break;
         ++gp;
-        if (++jp == item_slot[kp % kItemRing].nk) {
-          mbar_arrive(&item_empty[kp % kItemRing]);
+        if (__any_sync(0xFFFFFFFFu, ++jp == item_slot[kp % kItemRing].nk)) {
+          item_done(kp);
           jp = 0;
           ++kp;
         }
       }
       // every MMA issued above has completed once this phase does
-      tc_commit(&drain);
+      if (elect_one()) tc_commit(&drain);
+      __syncwarp();
       pf_wait(&drain, 0, limit_ns);
     }
   } else if (warp < 4) {
