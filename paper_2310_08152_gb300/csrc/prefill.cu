@@ -30,10 +30,11 @@
 // taken out paid more than its instructions' issue slots.  So waits are one short loop, the epilogue and the
 // masking exist once, and nothing but the softmax is unrolled far.  Time of a layer, against a kernel that read
 // every stored row with masks over all of them: OPT-1.3B-shaped prompts (16 x 2048 tokens, 32 heads of 64,
-// interiors of 32) 541 -> 362 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 990 us; the
-// last 512 of 32 x 4096 tokens, compacted before them, bf16 (heads of 80) 664 -> 456 us; the first with 96 and
-// 128 columns 797 -> 580 and 1042 -> 602 us; one prompt of 300 tokens 13.2 -> 12.2 us.  Copying the listed rows
-// side by side first, for TMA tiles alone, took a second kernel and 381, 992 and 454 us on the first three.
+// interiors of 32) 541 -> 248 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 747 us; the
+// last 512 of 32 x 4096 tokens, compacted before them, bf16 (heads of 80) 664 -> 312 us; the first with 96 and
+// 128 columns 797 -> 385 and 1042 -> 421 us; one prompt of 300 tokens 13.2 -> 10.8 us.  (Copying the listed rows
+// side by side first, for TMA tiles alone, took a second kernel and 381, 992 and 454 us on the first three when
+// the gathers took 372, 1026 and 450.)
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -113,8 +114,7 @@ struct PfCfg {
   // warpgroup gives registers up (setmaxnreg.dec to REG_OTHER) and the softmax warpgroup takes them
   // (setmaxnreg.inc to REG_SOFTMAX); the two shares add up to exactly what the CTA was launched with.
   static constexpr int REG_LAUNCH = 65536 / (CPS * kPfThreads);
-  // (the gather spills below that: 64 columns 370 us with 48, 358 with 56; 80 columns 1027 with 48, 984 with 64)
-  static constexpr int REG_OTHER = D == 64 ? 56 : 64;
+  static constexpr int REG_OTHER = 56;
   static constexpr int REG_SOFTMAX = (REG_LAUNCH * kPfThreads - REG_OTHER * 128) / 128 / 8 * 8;
   static_assert(CPS == 1 || REG_SOFTMAX * 128 + REG_OTHER * 128 <= REG_LAUNCH * kPfThreads,
                 "setmaxnreg shares exceed the launch allocation");
@@ -406,10 +406,9 @@ __device__ __forceinline__ PfItem pf_item(const PrefillArgs& a, int64_t it) {
 // 16-byte asynchronous copies.  Each quarter of the warp, whose 128 bytes are written to shared memory together,
 // covers the chunks of one subtile in as many rows as fill its swizzle pattern, so that they fall into different
 // banks; its quarters lie side by side in the rows, as far as the row goes (96 columns: 621 us with lanes in
-// row order, 577 so).  The gathers bound tiles of many short runs: few instructions a step and many steps in flight,
-// as far as the instruction cache has room (OPT-1.3B-shaped prompts, interiors of 32 / 8: 292 / 445 us with the
-// swizzle worked out per step, two of a group's eight steps unrolled; so 291 / 443 with two, 271 / 393 with four,
-// 286 / 419 with eight; 80, 96, 128 columns: 886, 458, 556 us with four, 867, 446, 490 with all).
+// row order, 577 so).  The gathers bound tiles of many short runs: few instructions a step and many steps in flight
+// (OPT-1.3B-shaped prompts, interiors of 32 / 8: 292 / 445 us with the swizzle worked out per step and two steps
+// unrolled, 271 / 393 so with four; 80, 96, 128 columns: 886, 458, 556 us with four, 867, 446, 490 with all).
 template <int D, int SW, int U0, int NS>
 __device__ __forceinline__ void gather_rows(uint32_t dst, uint32_t subb, const uint16_t* rows, int row, int p0, int kt,
                                             int lane) {
@@ -421,7 +420,7 @@ __device__ __forceinline__ void gather_rows(uint32_t dst, uint32_t subb, const u
   constexpr int SH = SW == 128 ? 0 : SW == 64 ? 1 : 2;
   dst += u * subb + (p0 + pr) * SW;
   const int c0 = cw ^ (pr >> SH & (CH - 1));
-#pragma unroll (D == 64 ? 4 : 16)
+#pragma unroll
   for (int i = 0; i < 32; i += RPS) {
     if (i >= 16 && kt - p0 < 32) break;  // 16 rows
     const int x = __shfl_sync(0xFFFFFFFFu, row, pr + i);
@@ -950,11 +949,11 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       __syncwarp();
       return true;
     };
-    // Epilogue of item kk (row sum l_): O / l, 16 rows at a time.  The 16-lane form of tcgen05.ld gives four
-    // neighbouring lanes 8 columns of a row, so each store fills 32-byte sectors of eight queries' rows (3000
-    // cycles an item when each warp staged 16 columns at a time in shared memory for tensor stores).  A few
-    // columns at a time: the next tile's scores are in registers meanwhile (64 columns: 348 us staged, 399 with
-    // 64 columns at a time, 333 with 32).
+    // Epilogue of item kk (row sum l_): O / l.  The 16-lane form of tcgen05.ld gives four neighbouring lanes 8 columns of
+    // a row, so each store fills 32-byte sectors of eight queries' rows (OPT-1.3B-shaped prompts 333 us so, 348 when
+    // each warp staged 16 columns at a time in shared memory for tensor stores).  All 32 rows of a few columns at a
+    // time: the next tile's scores are in registers meanwhile, and 32 columns of 64 make the softmax spill (253 us
+    // with 16 rows and 32 columns at a time, 248 with 32 and 16, 288 with 32 and 32).
     auto epilogue = [&](uint32_t kk, float l_) {
       const PfItem& w = item_slot[kk % kItemRing];
       const uint32_t o_t = tl + Cf::O_COL + (Cf::OBUF == 2 ? (kk & 1) * D : 0);
@@ -963,34 +962,35 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       inv = __fmaf_rn(inv, __fmaf_rn(-l_, inv, 1.f), inv);
       const int64_t row8 = (int64_t)8 * a.H * D;
       float* o_row = a.out + ((int64_t)(w.tok0 + warp * 32 + (lane >> 2)) * a.H + w.h) * D + 2 * (lane & 3);
-      constexpr int CO = D % 32 == 0 ? 32 : 16;  // columns at a time
+      const int left = w.qr_end - w.qr0 - (warp * 32 + (lane >> 2));  // queries from this lane's first row on
+      float inv8[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) inv8[i] = __shfl_sync(0xFFFFFFFFu, inv, 8 * i + (lane >> 2));
+      constexpr int CO = Cf::PSEP ? 16 : 32;  // columns at a time
 #pragma unroll 1
-      for (int i = 0; i < 32; i += 16) {
-        const float inv0 = __shfl_sync(0xFFFFFFFFu, inv, i + (lane >> 2));
-        const float inv1 = __shfl_sync(0xFFFFFFFFu, inv, i + 8 + (lane >> 2));
-        const int left = w.qr_end - w.qr0 - (warp * 32 + i + (lane >> 2));  // queries from this lane's row on
-#pragma unroll 1
-        for (int u = 0; u < D; u += CO) {
-          float o[CO / 2];
+      for (int u = 0; u < D; u += CO, o_row += CO) {
+        float o[2][CO / 2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
           if constexpr (CO == 32)
-            tmem_ld_16x256b_x4(o_t + (i << 16) + u, o);
+            tmem_ld_16x256b_x4(o_t + (i << 20) + u, o[i]);
           else
-            tmem_ld_16x256b_x2(o_t + (i << 16) + u, o);
-          tmem_wait_ld();
+            tmem_ld_16x256b_x2(o_t + (i << 20) + u, o[i]);
+        }
+        tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < CO / 2; ++e) asm volatile("" : "+f"(o[e]));  // no use of O moves above the wait
-          if (left > 0) {
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int e = 0; e < CO / 2; ++e) asm volatile("" : "+f"(o[i][e]));  // no use of O moves above the wait
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (left > 8 * i) {
 #pragma unroll
             for (int c = 0; c < CO / 8; ++c)
-              *reinterpret_cast<float2*>(o_row + u + 8 * c) = make_float2(o[4 * c] * inv0, o[4 * c + 1] * inv0);
-          }
-          if (left > 8) {
-#pragma unroll
-            for (int c = 0; c < CO / 8; ++c)
-              *reinterpret_cast<float2*>(o_row + row8 + u + 8 * c) = make_float2(o[4 * c + 2] * inv1, o[4 * c + 3] * inv1);
+              *reinterpret_cast<float2*>(o_row + i * row8 + 8 * c) =
+                  make_float2(o[i >> 1][4 * c + 2 * (i & 1)] * inv8[i], o[i >> 1][4 * c + 2 * (i & 1) + 1] * inv8[i]);
           }
         }
-        o_row += 2 * row8;
       }
       tc_fence_before();
       item_done(kk);
