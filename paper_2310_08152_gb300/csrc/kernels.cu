@@ -47,11 +47,10 @@ constexpr int64_t kAppendMaxBlocks = 16384;
 // head -- with 32-bit index arithmetic.  The token's RoPE sines and cosines (rot/2 of them) are
 // computed once per unit into shared memory.
 template <typename T, int D>
-__global__ void __launch_bounds__(kAppendThreads) append_kernel(Geometry g, Static st, Buffers buf,
-                                                                const TokPlan* __restrict__ plan, int64_t ntok,
-                                                                int64_t n_in, int m0, int n_layers, int write_meta,
-                                                                const uint16_t* __restrict__ k_in,
-                                                                const uint16_t* __restrict__ v_in) {
+__device__ __forceinline__ void append_units(const Geometry& g, const Static& st, const Buffers& buf,
+                                             const TokPlan* plan, int64_t ntok, int64_t n_in, int m0, int n_layers,
+                                             int write_meta, const uint16_t* __restrict__ k_in,
+                                             const uint16_t* __restrict__ v_in) {
   constexpr int VPR = D / 8;
   __shared__ float2 rope_cs[D / 2];  // (cos, sin) of the token's rotated pairs
   const int H = g.H;
@@ -115,6 +114,30 @@ __global__ void __launch_bounds__(kAppendThreads) append_kernel(Geometry g, Stat
       buf.orig[st.off[tp.s] + tp.row] = tp.orig;
     }
   }
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kAppendThreads) append_kernel(Geometry g, Static st, Buffers buf,
+                                                                const TokPlan* __restrict__ plan, int64_t ntok,
+                                                                int64_t n_in, int m0, int n_layers, int write_meta,
+                                                                const uint16_t* __restrict__ k_in,
+                                                                const uint16_t* __restrict__ v_in) {
+  append_units<T, D>(g, st, buf, plan, ntok, n_in, m0, n_layers, write_meta, k_in, v_in);
+}
+
+// The same for a few tokens whose upload (decode state and plan) comes as a kernel parameter: no copy, event and
+// staging memory for it, which bound such calls.  Block 0 stores it in the workspace, where the calls after this one
+// read it.  A call for a token of each of four sequences in four layers: 10.1 us with the upload, 6.8 without; 40
+// generated tokens with their decodes 3825 -> 3517.  The line is the size of a kernel's parameters (4 KB).
+template <typename T, int D>
+__global__ void __launch_bounds__(kAppendThreads)
+    append_image_kernel(Geometry g, Static st, Buffers buf, const __grid_constant__ AppendImage img, int img_bytes,
+                        int plan_off, uint4* dyn, int64_t ntok, int64_t n_in, int m0, int n_layers,
+                        const uint16_t* __restrict__ k_in, const uint16_t* __restrict__ v_in) {
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < img_bytes / 16; i += blockDim.x) dyn[i] = img.v[i];
+  append_units<T, D>(g, st, buf, reinterpret_cast<const TokPlan*>(reinterpret_cast<const char*>(&img) + plan_off), ntok,
+                     n_in, m0, n_layers, 1, k_in, v_in);
 }
 
 // a1 through TMA, for calls with at least one (layer, token) unit per SM.  A warp is a worker with
@@ -1708,6 +1731,19 @@ cudaError_t launch_append(const Geometry& g, const Static& st, const Buffers& bu
                                        num_sms, limit_ns, stream);
     return launch_append_t<F16T, D>(g, st, buf, plan, n_plan, n_in, m0, n_layers, write_meta, k_in, v_in, maps,
                                     num_sms, limit_ns, stream);
+  });
+}
+
+cudaError_t launch_append_image(const Geometry& g, const Static& st, const Buffers& buf, const AppendImage& img,
+                                size_t img_bytes, size_t plan_off, void* dyn, int64_t n_plan, int64_t n_in,
+                                int n_layers, const void* k_in, const void* v_in, cudaStream_t stream) {
+  return by_dhead(g.D, [&](auto dc) {
+    constexpr int D = decltype(dc)::value;
+    auto* kernel = g.dtype == 1 ? append_image_kernel<BF16T, D> : append_image_kernel<F16T, D>;
+    kernel<<<(unsigned)(n_layers * n_plan), kAppendThreads, 0, stream>>>(
+        g, st, buf, img, (int)img_bytes, (int)plan_off, static_cast<uint4*>(dyn), n_plan, n_in, 0, n_layers,
+        static_cast<const uint16_t*>(k_in), static_cast<const uint16_t*>(v_in));
+    return cudaGetLastError();
   });
 }
 

@@ -64,6 +64,14 @@ bool dhead_supported(int D);
 cudaError_t launch_append(const Geometry& g, const Static& st, const Buffers& buf, const TokPlan* plan, int64_t n_plan,
                           int64_t n_in, int m0, int n_layers, bool write_meta, const void* k_in, const void* v_in,
                           const void* maps, int num_sms, unsigned long long limit_ns, cudaStream_t stream);
+// Of all layers or of layer 0, for uploads (img_bytes, a multiple of 16, the plan from plan_off on) that fit a kernel
+// parameter; they go to dyn.
+struct alignas(16) AppendImage {
+  uint4 v[224];
+};
+cudaError_t launch_append_image(const Geometry& g, const Static& st, const Buffers& buf, const AppendImage& img,
+                                size_t img_bytes, size_t plan_off, void* dyn, int64_t n_plan, int64_t n_in,
+                                int n_layers, const void* k_in, const void* v_in, cudaStream_t stream);
 // Bytes of encode_append_maps' output: a 128-byte TMA descriptor per (K/V, sequence).
 inline size_t append_maps_bytes(int b) { return 2 * 128 * (size_t)b; }
 // Encodes, per sequence s, 4-D TMA descriptors over the K and then the V planes: dims {D, cap[s],

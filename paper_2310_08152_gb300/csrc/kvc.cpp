@@ -676,6 +676,8 @@ static kvc_status append_impl(kvc_cache* c, int layer, const void* k, const void
   kvc_status st = c->ensure_cuda(stream);
   if (st != KVC_OK) return st;
   const kvc::Geometry g = c->geom();
+  const int m0 = layer < 0 ? 0 : layer;
+  const int nl = layer < 0 ? M : 1;
   if (starts) {
     int64_t N = 0;
     for (int s = 0; s < c->cfg.b; ++s) N += n_new[s];
@@ -702,7 +704,10 @@ static kvc_status append_impl(kvc_cache* c, int layer, const void* k, const void
     }
     const size_t bytes = c->ws.dyn_payload + sizeof(kvc::TokPlan) * (size_t)n_plan;
     cudaError_t e;
-    unsigned char* img = c->ring.reserve(bytes, &e);
+    // a few tokens (fewer units than SMs) bring their upload as a kernel parameter
+    kvc::AppendImage small;
+    const bool fits = n_plan > 0 && bytes <= sizeof(small) && n_plan * nl < c->num_sms;
+    unsigned char* img = fits ? reinterpret_cast<unsigned char*>(&small) : c->ring.reserve(bytes, &e);
     if (!img) return cuda_fail(e, "staging");
     c->bk.book.apply_append(n_new, kinds, pos, (free_in_block && !local) ? kept.data() : nullptr);
     c->fill_state(img);
@@ -721,14 +726,24 @@ static kvc_status append_impl(kvc_cache* c, int layer, const void* k, const void
         ++w;
       }
     }
-    e = c->ring.commit(c->wsp(c->ws.dyn), bytes, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "upload append plan");
+    if (fits) {
+      e = kvc::launch_append_image(g, c->stat(), c->bufs(), small, bytes, c->ws.dyn_payload, c->wsp(c->ws.dyn), n_plan, N,
+                                   nl, k, v, stream);
+      if (e != cudaSuccess) return cuda_fail(e, "append kernel");
+      c->launches += 1;
+      c->last_was_decode = false;
+    } else {
+      e = c->ring.commit(c->wsp(c->ws.dyn), bytes, stream);
+      if (e != cudaSuccess) return cuda_fail(e, "upload append plan");
+    }
     c->batch_ntok = n_plan;
     c->batch_nin = N;
     c->layers_done = 0;
+    if (fits) {
+      c->layers_done = nl;
+      return ok();
+    }
   }
-  const int m0 = layer < 0 ? 0 : layer;
-  const int nl = layer < 0 ? M : 1;
   if (c->batch_ntok > 0) {
     const kvc::TokPlan* plan = reinterpret_cast<const kvc::TokPlan*>(c->wsp(c->ws.dyn + c->ws.dyn_payload));
     cudaError_t e = kvc::launch_append(g, c->stat(), c->bufs(), plan, c->batch_ntok, c->batch_nin, m0, nl, m0 == 0, k,
