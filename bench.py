@@ -439,15 +439,18 @@ def time_prompt_write_time_freeing(w, steps_total, dev):
 def prefill_work(w, block: int):
     """FLOPs of one layer's masked prefill over the prompt, summed over sequences and heads:
     (algorithmic) 4 d per visible (query, key) pair -- q.k and p.v over exactly the rows the mask
-    leaves (Sec. 3.1) -- and (executed) 4 d x 128 x 128 per key tile the kernel runs.  The visible
-    counts follow the per-row bounds of the library's host book: query iq sees rows i <= iq with
-    hid(i) >= iq, a <CL> query only itself."""
+    leaves (Sec. 3.1) -- and (executed) 4 d x 128 x keys per key tile the kernel runs: of each
+    128-query tile over the rows that no span hides before it, the interior of a span it begins in
+    and its own rows, in tiles of 128, 112 or 64 keys.  The visible counts follow the per-row bounds
+    of the library's host book: query iq sees rows i <= iq with hid(i) >= iq, a <CL> query only
+    itself."""
     import paper_2310_08152_gb300 as kvc
 
     L = w.prompt_len
     book = kvc.Book(w.b, L + 1)
     start = np.zeros(w.b, np.int64)
-    pairs = tiles = 0
+    pairs = keys = 0
+    kt = 128 if w.d > 80 else 64 if w.dtype == "bf16" else {64: 128, 80: 112}[w.d]
     while (start < L).any():
         n = L - start if block <= 0 else np.minimum(L - start, block)
         kinds = np.concatenate([w.prompt_kinds[s][start[s]:start[s] + n[s]] for s in range(w.b)]).astype(np.uint8)
@@ -462,8 +465,16 @@ def prefill_work(w, block: int):
             iq = np.arange(q0, ln)
             cnt = (iq + 1) - np.searchsorted(np.sort(hid), iq, side="left")
             pairs += int(np.where(cl[iq] == 1, 1, cnt).sum())
-            for qt in range((int(n[s]) + 127) // 128):
-                tiles += (min(q0 + 128 * (qt + 1), ln) + 127) // 128
+            never = hid == 0x3FFFFFFF
+            listed = np.concatenate([[0], np.cumsum(never)])  # rows that no span hides before each row
+            for lo in range(q0, ln, 128):
+                b0 = lo
+                while b0 > 0 and not never[b0 - 1] and hid[b0 - 1] >= lo:
+                    b0 -= 1
+                own = int(listed[b0]) + lo - b0
+                if 128 % kt == 0:
+                    own = -(-own // kt) * kt
+                keys += -(-(own + min(lo + 128, ln) - lo) // kt) * kt
         seq, cl_, cr_ = [], [], []
         for s in range(w.b):
             for a, c in book.pending_spans(s):
@@ -473,7 +484,7 @@ def prefill_work(w, block: int):
         if seq:
             book.compress(seq, cl_, cr_)
         start = start + n
-    return 4 * w.d * pairs * w.H, 4 * w.d * 128 * 128 * tiles * w.H
+    return 4 * w.d * pairs * w.H, 4 * w.d * 128 * keys * w.H
 
 
 def time_prompt_prefill(w, steps_total, dev, block: int):

@@ -398,9 +398,13 @@ class KVCache:
         self._cfg = cfg
         self.handle = kvc_create(cfg)
         # the upload ring, from torch's pool of pinned memory (allocating and freeing it with each cache takes
-        # about 300 us); kvc_destroy waits for the device before the pool gets it back
-        self.staging = torch.empty(kvc_staging_bytes(self.handle), dtype=torch.uint8, pin_memory=True)
-        kvc_set_staging(self.handle, self.staging)
+        # about 300 us); kvc_destroy waits for the device before the pool gets it back.  Above 4 MB (some 50,000
+        # rows) the library allocates it: the pool rounds up to powers of two, and pinning the rest costs as much
+        # (300 us more at 16 MB) while a cache of that size is rarely made anew.
+        self.staging = None
+        if kvc_staging_bytes(self.handle) <= 4 << 20:
+            self.staging = torch.empty(kvc_staging_bytes(self.handle), dtype=torch.uint8, pin_memory=True)
+            kvc_set_staging(self.handle, self.staging)
         self.book = Book(self.b, cap, policy, _handle=lib().kvc_get_book(self.handle))
 
     # views of the device layout (rows of d_head elements)
