@@ -30,7 +30,7 @@
 // taken out paid more than its instructions' issue slots.  So waits are one short loop, the epilogue and the
 // masking exist once, and nothing but the softmax is unrolled far.  Time of a layer, against a kernel that read
 // every stored row with masks over all of them: OPT-1.3B-shaped prompts (16 x 2048 tokens, 32 heads of 64,
-// interiors of 32) 541 -> 248 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 747 us; the
+// interiors of 32) 541 -> 248 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 735 us; the
 // last 512 of 32 x 4096 tokens, compacted before them, bf16 (heads of 80) 664 -> 312 us; the first with 96 and
 // 128 columns 797 -> 385 and 1042 -> 421 us; one prompt of 300 tokens 13.2 -> 10.8 us.  (Copying the listed rows
 // side by side first, for TMA tiles alone, took a second kernel and 381, 992 and 454 us on the first three when
@@ -292,6 +292,20 @@ __device__ __forceinline__ uint32_t bf16_split2(float2 x, uint32_t* hi) {
   return Pack16<BF16T>::two(d.x, d.y);
 }
 
+// rope_sincos (device_common.cuh) of two frequencies (hi, hi, lo, lo) at position p, with packed instructions and the
+// same roundings: sines, their negatives, cosines.  (Ragged rotary prompts 746 us a layer with rope_sincos, 735 so.)
+__device__ __forceinline__ void rope_sincos2(float p, float4 g, float2* s, float2* ns, float2* c) {
+  const float2 p2 = make_float2(p, p), gh = make_float2(g.x, g.y);
+  const float2 a = __fmul2_rn(p2, gh), na = __fmul2_rn(make_float2(-p, -p), gh);
+  const float2 e = __ffma2_rn(p2, gh, na);
+  const float2 turn = __fadd2_rn(a, make_float2(rintf(na.x), rintf(na.y)));
+  const float2 f = __fadd2_rn(turn, __ffma2_rn(p2, make_float2(g.z, g.w), e));
+  const float2 t = __fmul2_rn(make_float2(6.28318530717958647692f, 6.28318530717958647692f), f);
+  __sincosf(t.x, &s->x, &c->x);
+  __sincosf(t.y, &s->y, &c->y);
+  *ns = make_float2(-s->x, -s->y);
+}
+
 template <typename T>
 constexpr bool kSplit = false;
 template <>
@@ -463,8 +477,9 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
   __shared__ int8_t bound[128];  // of the tile being sorted
   __shared__ int32_t kslow[kClsRing];  // the tile needs the per-key rule (else every key is visible)
   __shared__ uint64_t cls_full[kClsRing], cls_empty[kClsRing];
-  __shared__ float2 rope_s[D / 2];  // a.rope_g (read from global memory in each item, with two words of a row in
-                                    // flight: ragged rotary prompts 985 us, 949 so with eight)
+  // a.rope_g, two frequencies at a time: (hi, hi, lo, lo).  (Read from global memory in each item, with two words of
+  // a row in flight: ragged rotary prompts 985 us, 949 so with eight.)
+  __shared__ float4 rope_s[D / 4];
   __shared__ uint32_t tmem_slot;
 
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~uintptr_t(1023));
@@ -479,7 +494,10 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (ROT && threadIdx.x >= 64 && threadIdx.x < 64 + a.rot / 2) rope_s[threadIdx.x - 64] = a.rope_g[threadIdx.x - 64];
+  if (ROT && threadIdx.x >= 64 && threadIdx.x < 64 + a.rot / 4) {
+    const float2 g0 = a.rope_g[2 * (threadIdx.x - 64)], g1 = a.rope_g[2 * (threadIdx.x - 64) + 1];
+    rope_s[threadIdx.x - 64] = make_float4(g0.x, g1.x, g0.y, g1.y);
+  }
   if (threadIdx.x == 32) {
     for (int i = 0; i < KST; ++i) {
       mbar_init(&k_full[i], 32);
@@ -873,7 +891,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       if constexpr (Cf::SPLIT) {
         // every row (rows past the tile's queries hold zeros), so the TMEM stores are warp-wide
         {
-          const int32_t qpos = iq < w.qr_end ? a.pos[a.off[w.s] + iq] : 0;
+          const float fpos = iq < w.qr_end ? (float)a.pos[a.off[w.s] + iq] : 0.f;
           const int hc = half / 8;  // chunks per rotated half
 #pragma unroll 1
           for (int c8 = 0; c8 < D / 16; ++c8) {
@@ -885,11 +903,10 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
 #pragma unroll
               for (int e = 0; e < 4; ++e) {
                 const float2 x1 = T::f2(w1[e]), x2 = T::f2(w2[e]);
-                float sn0, cs0, sn1, cs1;
-                rope_sincos(qpos, rope_s[8 * c8 + 2 * e], &sn0, &cs0);
-                rope_sincos(qpos, rope_s[8 * c8 + 2 * e + 1], &sn1, &cs1);
-                l1[e] = bf16_split2(make_float2(x1.x * cs0 - x2.x * sn0, x1.y * cs1 - x2.y * sn1), &h1[e]);
-                l2[e] = bf16_split2(make_float2(x2.x * cs0 + x1.x * sn0, x2.y * cs1 + x1.y * sn1), &h2[e]);
+                float2 sn, ns, cs;
+                rope_sincos2(fpos, rope_s[4 * c8 + e], &sn, &ns, &cs);
+                l1[e] = bf16_split2(__ffma2_rn(x1, cs, __fmul2_rn(x2, ns)), &h1[e]);
+                l2[e] = bf16_split2(__ffma2_rn(x2, cs, __fmul2_rn(x1, sn)), &h2[e]);
               }
               st_shared_v4(a1, h1[0], h1[1], h1[2], h1[3]);
               st_shared_v4(a2, h2[0], h2[1], h2[2], h2[3]);
@@ -903,7 +920,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
             if (c8 >= 2 * hc) qlo_store(c8, 0u, 0u, 0u, 0u);
         }
       } else if (iq < w.qr_end) {
-        const int32_t qpos = a.pos[a.off[w.s] + iq];
+        const float fpos = (float)a.pos[a.off[w.s] + iq];
 #pragma unroll 1
         for (int c8 = 0; c8 < half / 8; ++c8) {
           const uint32_t a1 = q_chunk(c8), a2 = q_chunk(c8 + half / 8);
@@ -913,11 +930,11 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float2 x1 = T::f2(w1[e]), x2 = T::f2(w2[e]);
-            float sn0, cs0, sn1, cs1;
-            rope_sincos(qpos, rope_s[8 * c8 + 2 * e], &sn0, &cs0);
-            rope_sincos(qpos, rope_s[8 * c8 + 2 * e + 1], &sn1, &cs1);
-            h1[e] = Pack16<T>::two(x1.x * cs0 - x2.x * sn0, x1.y * cs1 - x2.y * sn1);
-            h2[e] = Pack16<T>::two(x2.x * cs0 + x1.x * sn0, x2.y * cs1 + x1.y * sn1);
+            float2 sn, ns, cs;
+            rope_sincos2(fpos, rope_s[4 * c8 + e], &sn, &ns, &cs);
+            const float2 y1 = __ffma2_rn(x1, cs, __fmul2_rn(x2, ns)), y2 = __ffma2_rn(x2, cs, __fmul2_rn(x1, sn));
+            h1[e] = Pack16<T>::two(y1.x, y1.y);
+            h2[e] = Pack16<T>::two(y2.x, y2.y);
           }
           st_shared_v4(a1, h1[0], h1[1], h1[2], h1[3]);
           st_shared_v4(a2, h2[0], h2[1], h2[2], h2[3]);
