@@ -577,10 +577,8 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
         const int cs = (int)(cg % kClsRing);
         // per-key mask bounds of the tile ((hid << 1) | is_cl) sorted into the classes above; the causal
         // part (i <= iq) is left to each query
-        if (cg >= kClsRing && !pf_wait(&cls_empty[cs], ((cg / kClsRing) - 1) & 1, limit_ns)) {
-          ok = false;
+        if (cg >= kClsRing && !(ok = __all_sync(0xFFFFFFFFu, pf_wait(&cls_empty[cs], (cg / kClsRing - 1) & 1, limit_ns))))
           break;
-        }
         uint32_t* hid_w = reinterpret_cast<uint32_t*>(&khid[cs]);
         uint32_t* end_w = reinterpret_cast<uint32_t*>(&kend[cs]);
         uint32_t my_end = 0u;  // word `lane` of kend
@@ -654,14 +652,14 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     uint32_t ph = 1, issued = 0;  // parity of the stage's previous release; tiles issued
     uint32_t q_items = 0;         // items whose query rows were requested (warp 7)
     for (uint32_t k = 0; ok; ++k) {
-      if (!(ok = item_wait(k))) break;
+      if (!(ok = __all_sync(0xFFFFFFFFu, item_wait(k)))) break;
       const PfItem w = item_slot[k % kItemRing];
       item_done(k);
       if (w.nk == 0) break;
       if (is_v) {
         // the item's query rows (past its last query another sequence's, or zeros past the last token: those
         // rows' results go nowhere), once the Q.K^T of the item before are complete
-        if (k >= 1 && !(ok = pf_wait(&q_empty, (k - 1) & 1, limit_ns))) break;
+        if (k >= 1 && !(ok = __all_sync(0xFFFFFFFFu, pf_wait(&q_empty, (k - 1) & 1, limit_ns)))) break;
         if (lane == 0) {
           mbar_arrive_expect_tx(&q_raw, Cf::QTILE);
 #pragma unroll
@@ -690,10 +688,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           if (KT > 64) r2 = key_row(v0 + 64 + lane);
           if (KT > 96) r3 = key_row(v0 + 96 + lane);
         }
-        if (issued >= (uint32_t)nst && !pf_wait(&empty[st], ph, limit_ns)) {
-          ok = false;
-          break;
-        }
+        if (issued >= (uint32_t)nst && !(ok = __all_sync(0xFFFFFFFFu, pf_wait(&empty[st], ph, limit_ns)))) break;
         const uint32_t dst = ring + st * Cf::TILE;
         if (tiled) {
           if (lane == 0) {
