@@ -178,7 +178,7 @@ struct alignas(64) PrefillMaps {
 };
 
 cudaError_t encode_prefill_maps(const Geometry& g, const Buffers& buf, PrefillMaps* maps);
-// Most CTAs of the persistent prefill grid (sizes its work-range table).
+// Most CTAs of the persistent prefill grid.
 constexpr int kMaxPrefillCtas = 1024;
 // Keys of one key tile for head dimension D and the cache type, and where a tile's own rows start among
 // its keys when n_before come before them: on a key tile of their own when those divide a query tile.
