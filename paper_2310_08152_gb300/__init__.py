@@ -425,7 +425,7 @@ class KVCache:
         n_new = _np(n_new, np.int32)
         kinds = _np(kinds, np.uint8)
         tied = layer <= 0 and pos is None
-        N = int(np.add.reduce(n_new))
+        N = int(np.add.reduce(n_new, axis=None))
         n = (self.M if layer < 0 else 1) * N * self.H * self.d
         try:
             _dev(k, "k", self.torch_dtype, n)
@@ -459,7 +459,7 @@ class KVCache:
         import torch
 
         n_q = _np(n_q, np.int32)
-        n_tok = int(np.add.reduce(n_q))
+        n_tok = int(np.add.reduce(n_q, axis=None))
         _dev(q, "q", self.torch_dtype, n_tok * self.H * self.d)
         if out is None:
             out = torch.empty(n_tok, self.H, self.d, dtype=torch.float32, device=q.device)

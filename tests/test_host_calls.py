@@ -16,6 +16,21 @@ def test_pending_spans_of_any_number(n):
     assert book.pending_spans(0) == []
 
 
+@pytest.mark.parametrize("shape", [(2,), (1, 2), (2, 1)])
+def test_token_counts_of_any_shape(monkeypatch, shape):
+    """Token counts per sequence come as an array of any shape: only their order counts."""
+    c = object.__new__(kvc.KVCache)
+    c.__dict__.update(M=3, H=4, d=64, b=2, torch_dtype=torch.float16, handle=None)
+    seen = []
+    monkeypatch.setattr(kvc, "_dev", lambda t, name, dtype, n: seen.append(n))
+    monkeypatch.setattr(kvc, "kvc_append_tied", lambda handle, layer, k, v, n_new, *a: seen.append(n_new.ravel().tolist()))
+    monkeypatch.setattr(kvc, "kvc_prefill_attention", lambda handle, layer, q, n_q, *a: seen.append(np.ravel(n_q).tolist()))
+    n = np.array([3, 4]).reshape(shape)
+    assert c.append(None, None, n, [0] * 7).size == 7
+    c.prefill_attention(0, None, n, 0.125, out=torch.empty(0))
+    assert seen == [3 * 7 * 256, 3 * 7 * 256, [3, 4], 7 * 256, 7 * 256, [3, 4]]
+
+
 def _tokens(M, H, d, n, seed):
     g = torch.Generator(device="cuda").manual_seed(seed)
     return [torch.randn(M, n, H, d, device="cuda", generator=g).half() for _ in range(2)]
