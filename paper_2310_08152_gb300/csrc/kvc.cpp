@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -144,11 +145,19 @@ class PinnedRing {
   }
   static size_t ring_bytes(size_t bytes) { return align_up(bytes, 256); }
   void release() {
-    // freeing pinned memory waits for the device; borrowed memory is given back only after the same wait
+    // Borrowed memory is given back once its copies are complete, and, as freeing pinned memory does, once the
+    // device is idle: the cache's device buffers go back to their owner next, and any stream may have used
+    // them.  That wait is the freeing of a small block, which leaves a capture in progress alone where
+    // cudaDeviceSynchronize fails and ends it.  On an idle device 4 us while another small block lives, so
+    // the process keeps one per device; 130 without.
     if (borrowed_ && base_) {
       int dev = -1;
       if (cudaGetDevice(&dev) == cudaSuccess && dev != device_) cudaSetDevice(device_);
-      cudaDeviceSynchronize();
+      for (auto& p : pending_) cudaEventSynchronize(p.ev);
+      static std::atomic<bool> kept[64];
+      void* block = nullptr;
+      if (device_ >= 0 && device_ < 64 && !kept[device_].exchange(true)) (void)cudaMalloc(&block, 256);
+      if (cudaMalloc(&block, 256) != cudaSuccess || cudaFree(block) != cudaSuccess) cudaDeviceSynchronize();
       if (dev >= 0 && dev != device_) cudaSetDevice(dev);
       base_ = nullptr;
     }
@@ -631,7 +640,13 @@ kvc_status kvc_create(const kvc_config* cfg, kvc_cache** out) {
   return ok();
 }
 
-void kvc_destroy(kvc_cache* cache) { delete cache; }
+void kvc_destroy(kvc_cache* cache) {
+  // another stream may be capturing: the waits and the freeing below are no part of that
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  const bool cuda = cache && cache->cuda_ready && cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess;
+  delete cache;
+  if (cuda) cudaThreadExchangeStreamCaptureMode(&mode);
+}
 
 size_t kvc_staging_bytes(const kvc_cache* c) { return c ? PinnedRing::ring_bytes(c->staging_bytes()) : 0; }
 

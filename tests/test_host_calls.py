@@ -74,3 +74,32 @@ def test_append_at_tied_positions_and_own_staging(free_closed):
             kvc.kvc_set_staging(c.handle, bad)
         assert e.value.status == 1
     assert a.device_status() == 0 and b.device_status() == 0
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+@pytest.mark.parametrize("own", [False, True])
+def test_cache_that_ends_while_a_stream_captures(mode, own):
+    """A cache's end waits for its upload on a busy stream, before torch's pool gets the staging memory back, and
+    leaves the capture on another stream alone; so does a cache whose ring the library allocates."""
+    c = kvc.KVCache(2, 4, 64, [600] * 2)
+    if own:
+        kvc._check(kvc.lib().kvc_set_staging(c.handle, None, 0))
+    n = np.array([250, 250], np.int32)
+    k, v = _tokens(2, 4, 64, 500, 2)
+    kinds = np.zeros(500, np.uint8)
+    c.append(k, v, n, kinds)
+    x, side, uploaded = torch.ones(4, device="cuda"), torch.cuda.Stream(), torch.cuda.Event()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode=mode):
+        x += 1
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(400_000_000)  # 0.2 s
+            c.append(k, v, n, kinds)
+            uploaded.record()
+        c.close()
+        x += 1
+    assert uploaded.query()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [3.0] * 4
