@@ -187,6 +187,10 @@ void kvc_destroy(kvc_cache* cache);
 size_t kvc_staging_bytes(const kvc_cache* cache);
 kvc_status kvc_set_staging(kvc_cache* cache, void* pinned, size_t bytes);
 
+/* Sets the calling thread's stream-capture mode (0 global, 1 thread-local, 2 relaxed) and returns the one
+ * before, -1 on an error: to allocate such memory without ending a capture that is in progress. */
+int kvc_thread_capture_mode(int mode);
+
 /* The cache's span book (read-only view: positions, pending spans, lengths, layout). */
 const kvc_book* kvc_get_book(const kvc_cache* cache);
 

@@ -401,9 +401,16 @@ class KVCache:
         # about 300 us); kvc_destroy waits for the device before the pool gets it back.  Above 4 MB (some 50,000
         # rows) the library allocates it: the pool rounds up to powers of two, and pinning the rest costs as much
         # (300 us more at 16 MB) while a cache of that size is rarely made anew.
+        # A capture on another stream goes on (relaxed mode); within one the library allocates it, as the first
+        # append comes.
         self.staging = None
-        if kvc_staging_bytes(self.handle) <= 4 << 20:
-            self.staging = torch.empty(kvc_staging_bytes(self.handle), dtype=torch.uint8, pin_memory=True)
+        n = kvc_staging_bytes(self.handle)
+        if n <= 4 << 20 and not torch.cuda.is_current_stream_capturing():
+            mode = lib().kvc_thread_capture_mode(2)
+            try:
+                self.staging = torch.empty(n, dtype=torch.uint8, pin_memory=True)
+            finally:
+                lib().kvc_thread_capture_mode(mode)
             kvc_set_staging(self.handle, self.staging)
         self.book = Book(self.b, cap, policy, _handle=lib().kvc_get_book(self.handle))
 

@@ -53,6 +53,7 @@ SIGNATURES = [
     ("kvc_destroy", None, [P]),
     ("kvc_staging_bytes", c_size_t, [P]),
     ("kvc_set_staging", c_int, [P, P, c_size_t]),
+    ("kvc_thread_capture_mode", c_int, [c_int]),
     ("kvc_get_book", P, [P]),
     ("kvc_append", c_int, [P, c_int, P, P, P, P, P, P]),
     ("kvc_append_free_closed", c_int, [P, c_int, P, P, P, P, P, P]),

@@ -661,6 +661,12 @@ kvc_status kvc_set_staging(kvc_cache* c, void* pinned, size_t bytes) {
   return ok();
 }
 
+int kvc_thread_capture_mode(int mode) {
+  cudaStreamCaptureMode m = static_cast<cudaStreamCaptureMode>(mode);
+  if (mode < 0 || mode > 2 || cudaThreadExchangeStreamCaptureMode(&m) != cudaSuccess) return -1;
+  return static_cast<int>(m);
+}
+
 const kvc_book* kvc_get_book(const kvc_cache* cache) { return cache ? &cache->bk : nullptr; }
 
 static kvc_status append_impl(kvc_cache* c, int layer, const void* k, const void* v, const int32_t* n_new,

@@ -103,3 +103,35 @@ def test_cache_that_ends_while_a_stream_captures(mode, own):
     graph.replay()
     torch.cuda.synchronize()
     assert x.tolist() == [3.0] * 4
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", ["global", "thread_local", "relaxed"])
+@pytest.mark.parametrize("beside", [False, True])
+def test_cache_that_is_made_while_a_stream_captures(mode, beside):
+    """Made on the capturing stream or beside it (where torch has device memory at hand), a cache leaves the capture
+    alone and works after it."""
+    x, capturing, side = torch.ones(4, device="cuda"), torch.cuda.Stream(), torch.cuda.Stream()
+    k, v = _tokens(1, 4, 64, 300, 3)
+    kinds = np.zeros(300, np.uint8)
+    with torch.cuda.stream(side):
+        held = [kvc.KVCache(1, 4, 64, [cap]) for cap in (300, 30000)]
+        again = [torch.empty_like(t) for c in held for t in (c.k, c.v, c.pos, c.orig, c.workspace)]
+    torch.cuda.synchronize()
+    del again
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(capturing):
+        graph.capture_begin(capture_error_mode=mode)
+        x += 1
+        with torch.cuda.stream(side if beside else capturing):
+            made = [kvc.KVCache(1, 4, 64, [cap]) for cap in (300, 30000)]
+        x += 1
+        graph.capture_end()
+    graph.replay()
+    for c in made:
+        c.append(k, v, [300], kinds)
+        out = c.decode_attention(0, k[0, -1:], 0.125)
+        p = torch.softmax(torch.einsum("hd,nhd->hn", k[0, -1].double(), k[0].double()) * 0.125, -1)
+        assert (out[0].double() - torch.einsum("hn,nhd->hd", p, v[0].double())).abs().max().item() < 3e-4
+        assert c.device_status() == 0
+    assert x.tolist() == [3.0] * 4
