@@ -852,7 +852,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       // every MMA issued above has completed once this phase does
       if (elect_one()) tc_commit(&drain);
       __syncwarp();
-      pf_wait(&drain, 0, limit_ns);
+      ok = uni_wait(&drain, 0, limit_ns) && ok;
     }
   } else if (warp < 4) {
     if constexpr (Cf::CPS == 2) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(Cf::REG_SOFTMAX));
@@ -1188,7 +1188,11 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
           store_p(0);
           store_p(1);
         }
-        if (j == 0 && k >= 1) epilogue(k - 1, l_prev);
+        if (j == 0 && k >= 1) {
+          // the item before is complete only if every wait up to its last P.V was
+          if (KT == 64 && !(ok = __all_sync(0xFFFFFFFFu, got_all))) break;
+          epilogue(k - 1, l_prev);
+        }
         if (!more) break;
         if (Cf::PSEP) {
 #pragma unroll
