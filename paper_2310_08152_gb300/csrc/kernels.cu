@@ -810,7 +810,8 @@ __global__ void __launch_bounds__(32, 1) decode_kernel(Geometry g, Static st, De
       }
     }
     if (!dead) {
-      if (mbar_wait_bounded(&full[stage], (t / C::S) & 1, p.limit_ns)) {
+      // the lanes agree, since what follows takes all of them
+      if (__all_sync(kFull, mbar_wait_bounded(&full[stage], (t / C::S) & 1, p.limit_ns))) {
         t_ok = t + 1;
       } else {
         dead = true;
@@ -1027,7 +1028,7 @@ struct CtaCfg {
   static constexpr int TR = W * WR;                       // rows per tile
   static constexpr int TILE = TR * L::RB;                 // bytes per K (or V) tile
   static constexpr int THREADS = (W + 1) * 32;
-  static constexpr int PO = D + 4;                        // floats of one partial result: M, L, -, -, O[D]
+  static constexpr int PO = D + 4;                        // floats of one partial result: M, L, dead, -, O[D]
   static constexpr int OFF_Z = 2 * S * TILE;              // a row of zeros
   static constexpr int OFF_Q = OFF_Z + L::RB;             // [W][D] floats
   static constexpr int OFF_O = OFF_Q + W * D * 4;         // [2][W][PO] floats: the warps' results, by piece parity
@@ -1259,7 +1260,8 @@ __global__ void __launch_bounds__((W + 1) * 32, CtaCfg<D, W, KPT, S>::CPS)
     while (r < r1) {
       int n = min(C::TR, r1 - r);
       if (r < wrap) n = min(n, wrap - r);
-      if (!dead && !mbar_wait_bounded(&full[stage], phase, p.limit_ns)) {
+      // the lanes agree, since what follows takes all of them
+      if (!dead && !__all_sync(kFull, mbar_wait_bounded(&full[stage], phase, p.limit_ns))) {
         dead = true;
         if (lane == 0) atomicOr(p.status, STATUS_TIMEOUT);
       }
@@ -1378,6 +1380,7 @@ __global__ void __launch_bounds__((W + 1) * 32, CtaCfg<D, W, KPT, S>::CPS)
       if (lane == 0) {
         so[0] = M;
         so[1] = Ls;
+        so[2] = dead ? 1.f : 0.f;
       }
       fence_proxy_async_smem();
       __syncwarp();
@@ -1387,16 +1390,21 @@ __global__ void __launch_bounds__((W + 1) * 32, CtaCfg<D, W, KPT, S>::CPS)
       if (lane == 0) {
         so[0] = -INFINITY;
         so[1] = 0.f;
+        so[2] = 0.f;
       }
     }
     bar_sync(1, W * 32);
     const bool mine_to_merge = warp == piece % W;
     const int seg = s * H + h;
     float* orow = p.out + (int64_t)layer * p.out_stride + (int64_t)seg * D;
-    // merges n results of PO floats; lane writes its columns scaled by 1 / L, or to the cluster's rank 0
+    // merges n results of PO floats; lane writes its columns scaled by 1 / L (not where a result lacks rows, after
+    // a wait that ran out), or to the cluster's rank 0
     auto merge = [&](const float* sp, int n, bool last) {
-      float Mx = -INFINITY;
-      for (int w = 0; w < n; ++w) Mx = fmaxf(Mx, sp[w * C::PO]);
+      float Mx = -INFINITY, bad = 0.f;
+      for (int w = 0; w < n; ++w) {
+        Mx = fmaxf(Mx, sp[w * C::PO]);
+        bad = fmaxf(bad, sp[w * C::PO + 2]);
+      }
       const float Mxu = (Mx == -INFINITY) ? 0.f : Mx;
       float Lx = 0.f, O[QPL];
 #pragma unroll
@@ -1413,7 +1421,7 @@ __global__ void __launch_bounds__((W + 1) * 32, CtaCfg<D, W, KPT, S>::CPS)
         const float inv = 1.f / Lx;
 #pragma unroll
         for (int j = 0; j < QPL; ++j)
-          if (lane + 32 * j < D) orow[lane + 32 * j] = O[j] * inv;
+          if (lane + 32 * j < D && bad == 0.f) orow[lane + 32 * j] = O[j] * inv;
       } else {
         float* dst = reinterpret_cast<float*>(smem + C::OFF_C) + rank * C::PO;
 #pragma unroll
@@ -1422,6 +1430,7 @@ __global__ void __launch_bounds__((W + 1) * 32, CtaCfg<D, W, KPT, S>::CPS)
         if (lane == 0) {
           st_cluster_f32(dst, 0, Mx);
           st_cluster_f32(dst + 1, 0, Lx);
+          st_cluster_f32(dst + 2, 0, bad);
         }
       }
     };
@@ -1431,11 +1440,11 @@ __global__ void __launch_bounds__((W + 1) * 32, CtaCfg<D, W, KPT, S>::CPS)
       cluster_arrive();
       if (rank == 0) {
         cluster_wait();
-        if (mine_to_merge && !dead) merge(reinterpret_cast<const float*>(smem + C::OFF_C), CN, true);
+        if (mine_to_merge) merge(reinterpret_cast<const float*>(smem + C::OFF_C), CN, true);
       }
       return;  // one segment per cluster
     }
-    if (mine_to_merge && !dead) merge(sO + (piece & 1) * W * C::PO, W, true);
+    if (mine_to_merge) merge(sO + (piece & 1) * W * C::PO, W, true);
     ++piece;
   }
 }

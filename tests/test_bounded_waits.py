@@ -21,3 +21,17 @@ def test_prefill_reports_each_wait_that_ran_out():
     calls = [m.start() for m in re.finditer(r" epilogue\(", src)]
     assert len(calls) == 1, calls
     assert src[:calls[0]].rstrip().endswith("if (KT == 64 && !(ok = __all_sync(0xFFFFFFFFu, got_all))) break;")
+
+
+def test_decode_lanes_agree_on_a_wait_and_a_dead_part_is_not_merged():
+    src = _source("kernels.cu")
+    # every wait whose verdict guards warp-wide work is voted on; the others are one lane's, or a role's last
+    for wait in re.finditer(r"mbar_wait_bounded\(&full\[stage\]", src):
+        assert src[:wait.start()].endswith("__all_sync(kFull, "), src[wait.start() - 80:wait.end() + 60]
+    cta = src[src.index("decode_cta_kernel("):]
+    # a warp's result carries the verdict, a merge keeps the worst one, and the last merge stores none but good ones
+    assert "so[2] = dead ? 1.f : 0.f;" in cta
+    assert "bad = fmaxf(bad, sp[w * C::PO + 2]);" in cta
+    assert "st_cluster_f32(dst + 2, 0, bad);" in cta
+    stores = re.findall(r"if \(([^;{}]*)\) orow\[", cta)
+    assert stores and all("bad == 0.f" in s for s in stores), stores
