@@ -485,8 +485,15 @@ struct Lanes {
 };
 
 // Shapes of the per-warp pipeline (rows per lane per tile x stages).  Whole segments, which take this
-// kernel when they are many and short, go to the narrow 2x3 shape (seven or eight warps per SM);
-// stream-K runs a full wave of warps: 2x2 fits the most warps per SM.
+// kernel when they are many and short, go to the narrow 2x3 shape (seven or eight warps per SM); runs of
+// longer ones that a few far longer keep from the CTAs go to the wide shape, the most bytes in flight in
+// as few tiles as three warps per SM hold (8x2 at d_head 64, 6x2 at 80, 4x3 otherwise); stream-K runs a
+// full wave of warps: 2x2 fits the most warps per SM.
+template <int D>
+struct WideShape {
+  static constexpr int KPT = D == 64 ? 8 : D == 80 ? 6 : 4;
+  static constexpr int S = D == 64 || D == 80 ? 2 : 3;
+};
 #ifndef KVC_DEC_SEG2_KPT
 #define KVC_DEC_SEG2_KPT 2
 #endif
@@ -1597,32 +1604,36 @@ CtaPlan decode_cta_plan(const DecodeArgs& a, int64_t nseg, bool balanced, int64_
 }
 
 // Resident CTAs per SM of the decode kernels' instances on the current device: the CTA kernel's main and
-// small shape, the warp kernel's whole-segment and stream-K shape.  Found once per device.
+// small shape, the warp kernel's whole-segment, stream-K and wide shape.  Found once per device.
 struct DecodeOcc {
-  int main, small, seg, stream;
+  int main, small, seg, stream, wide;
 };
 template <typename T, int D>
 cudaError_t decode_occupancies(int dev, DecodeOcc* out) {
   constexpr int BK = KVC_DEC_SEG2_KPT, BS = KVC_DEC_SEG2_STAGES, TK = KVC_DEC_STREAM_KPT, TS = KVC_DEC_STREAM_STAGES;
   constexpr int MS = CtaMainStages<D>::S;
-  static std::atomic<uint32_t> found[64];  // eight bits each; 0: not yet
+  constexpr int AK = WideShape<D>::KPT, AS = WideShape<D>::S;
+  static std::atomic<uint64_t> found[64];  // eight bits each; 0: not yet
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  uint32_t v = found[dev].load(std::memory_order_acquire);
+  uint64_t v = found[dev].load(std::memory_order_acquire);
   if (v == 0) {
-    int o[4];
+    int o[5];
     using M = CtaCfg<D, 4, 2, MS>;
     using S = CtaCfg<D, 2, 2, 3>;
     using B = DecodeCfg<D, BK, BS>;
     using K = DecodeCfg<D, TK, TS>;
+    using A = DecodeCfg<D, AK, AS>;
     cudaError_t e = kernel_occupancy(decode_cta_kernel<T, D, 4, 2, MS>, M::THREADS, M::SMEM, &o[0]);
     if (e == cudaSuccess) e = kernel_occupancy(decode_cta_kernel<T, D, 2, 2, 3>, S::THREADS, S::SMEM, &o[1]);
     if (e == cudaSuccess) e = kernel_occupancy(decode_kernel<T, D, BK, BS>, B::THREADS, B::SMEM, &o[2]);
     if (e == cudaSuccess) e = kernel_occupancy(decode_kernel<T, D, TK, TS>, K::THREADS, K::SMEM, &o[3]);
+    if (e == cudaSuccess) e = kernel_occupancy(decode_kernel<T, D, AK, AS>, A::THREADS, A::SMEM, &o[4]);
     if (e != cudaSuccess) return e;
-    v = (uint32_t)o[0] | (uint32_t)o[1] << 8 | (uint32_t)o[2] << 16 | (uint32_t)o[3] << 24;
+    for (int i = 0; i < 5; ++i) v |= (uint64_t)o[i] << 8 * i;
     found[dev].store(v, std::memory_order_release);
   }
-  *out = {(int)(v & 255u), (int)(v >> 8 & 255u), (int)(v >> 16 & 255u), (int)(v >> 24)};
+  auto at = [&](int i) { return (int)(v >> 8 * i & 255u); };
+  *out = {at(0), at(1), at(2), at(3), at(4)};
   return cudaSuccess;
 }
 
@@ -1631,6 +1642,7 @@ cudaError_t launch_decode_t(const Geometry& g, const Static& st, const Buffers& 
                             cudaStream_t stream, int* grid, DecodePlan* plan) {
   constexpr int BK = KVC_DEC_SEG2_KPT, BS = KVC_DEC_SEG2_STAGES;
   constexpr int TK = KVC_DEC_STREAM_KPT, TS = KVC_DEC_STREAM_STAGES;
+  constexpr int AK = WideShape<D>::KPT, AS = WideShape<D>::S;
   // A CTA or a cluster per segment, or a few segments per CTA, unless the segments are many and short
   // or a few of them far longer than the rest (decode_cta_plan).  Those: balanced segments (longest
   // within 1.3x of the mean) one per warp while a wave of warps holds them all, else k consecutive
@@ -1645,16 +1657,24 @@ cudaError_t launch_decode_t(const Geometry& g, const Static& st, const Buffers& 
   const cudaError_t e = decode_occupancies<T, D>(a.device, &occ);
   if (e != cudaSuccess) return e;
   const CtaPlan c = decode_cta_plan<D>(a, nseg, balanced, (int64_t)occ.main * num_sms, (int64_t)occ.small * num_sms);
-  if (n_layers > 1 && !balanced && nseg > (int64_t)occ.main * num_sms) {
-    // Unbalanced segments over several layers, short ones: a wave of warps takes whole segments cut by
-    // rows when the longest segment is at most 1/16 of a warp's even share (so no warp holds more than
-    // ~6 % above the mean).
-    int64_t NW = (int64_t)occ.seg * num_sms;
+  const bool by_cta = c.use && !c.small && c.k == 1;
+  if (n_layers > 1 && !balanced && !by_cta && nseg > (int64_t)occ.main * num_sms) {
+    // Unbalanced segments over several layers, short ones or with a few far longer: a wave of warps takes
+    // whole segments cut by rows when the longest segment is at most 1/16 of a warp's even share (so no
+    // warp holds more than ~6 % above the mean).  Means from six wide tiles up take the wide shape, whose
+    // fewer warps have the larger shares too: 24 layers of 96 sequences, one of 8,000 rows among 1,000
+    // each, 2,806 us (d_head 64) and 3,528 (80), and 3,091 and 4,013 by rows split over every warp of a
+    // launch per layer.  At d_head 96 and 128, whose wide tiles are 32 rows, up to 768 rows: two of 3,600
+    // among 192 of 300 rows, bf16 d_head 128, 3,716 and 3,927, but one of 8,000 among 96 of 1,000, 5,987
+    // and 5,942.
+    const int64_t wide_tile = AK * Lanes<D>::RPI;
+    const bool wide = a.R >= 6 * wide_tile * a.n_segments && (D <= 80 || a.R <= 24 * wide_tile * a.n_segments);
+    int64_t NW = (int64_t)(wide ? occ.wide : occ.seg) * num_sms;
     if (NW > nseg) NW = nseg;
-    const bool long_segs = c.use && !c.small && c.k == 1;
-    if (!long_segs && NW >= 1 && 16 * a.max_segment <= (int64_t)n_layers * a.R / NW) {
-      *plan = {4, (int)NW, BK * Lanes<D>::RPI, BS};
-      return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, NW, -1, stream, grid);
+    if (NW >= 1 && 16 * a.max_segment <= (int64_t)n_layers * a.R / NW) {
+      *plan = {4, (int)NW, (wide ? AK : BK) * Lanes<D>::RPI, wide ? AS : BS};
+      return wide ? launch_decode_cfg<T, D, AK, AS>(g, st, buf, a, NW, -1, stream, grid)
+                  : launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, NW, -1, stream, grid);
     }
   }
   if (c.use) {

@@ -80,3 +80,45 @@ def test_open_span_hidden_row_in_every_part():
     for policy in (orc.POLICY_PAPER, orc.POLICY_KEEP_CL):
         w = wl.opt13b(b=2, L=1600, M=1)
         run_workload(w, steps=4, policy=policy)
+
+
+def _few_long(d, dtype, b, short, n_long, factor, M):
+    """Prompts of about `short` tokens and n_long of `factor` times that, no spans."""
+    rng = np.random.default_rng(b + short)
+    lens = rng.integers(int(0.7 * short), int(1.3 * short), b)
+    lens[rng.permutation(b)[:n_long]] = factor * short
+    w = wl.opt13b(b=b, L=64, M=M)
+    return dataclasses.replace(w, d=d, dtype=dtype, scale=1.0 / math.sqrt(d), prompt_kinds=[np.zeros(n, np.uint8) for n in lens],
+                               prompt_spans=[[] for _ in lens], gen_kind=lambda s, g: 0, name=f"few-long-d{d}")
+
+
+# few long sequences among many: the plan, and its rows per tile, of one call for all layers
+FEW_LONG = [
+    ("d 64, wide", lambda: _few_long(64, "f16", 90, 900, 1, 8, 24), 4, 128),
+    ("d 80 bf16, wide", lambda: _few_long(80, "bf16", 90, 700, 1, 8, 24), 4, 96),
+    ("d 96, wide", lambda: _few_long(96, "f16", 160, 300, 1, 7, 24), 4, 32),
+    ("d 128 bf16, wide", lambda: _few_long(128, "bf16", 120, 250, 1, 8, 24), 4, 32),
+    ("d 64, narrow", lambda: _few_long(64, "f16", 220, 200, 1, 8, 24), 4, 32),
+    ("d 64, too long a sequence", lambda: _few_long(64, "f16", 60, 300, 1, 12, 24), 0, 32),
+]
+
+
+@pytest.mark.parametrize("name,make,mode,tile", FEW_LONG, ids=[c[0] for c in FEW_LONG])
+def test_a_few_long_sequences_over_layers(name, make, mode, tile):
+    """Runs of whole segments per warp, cut by rows, in the wide and the narrow shape, and the layers one by one
+    where a warp would hold too much: the first, a middle and the last layer against the oracle."""
+    w = make()
+    run = harness.Runner(w, steps=1)
+    run.load_prompt()
+    out = torch.full((w.M, w.b, w.H, w.d), float("nan"), dtype=torch.float32, device="cuda")
+    inp = run.make_step_inputs(0)
+    run.append_only(inp)
+    run.cache.decode_attention_layers(inp.q, w.scale, out=out)
+    plan = run.cache.last_decode_plan
+    assert plan["mode"] == mode and plan["tile_rows"] == tile, plan
+    lens = [k.size for k in w.prompt_kinds]
+    seqs, heads = [int(np.argmax(lens)), int(np.argmin(lens)), w.b - 1], [0, 31]
+    assert torch.isfinite(out).all()
+    for m in (0, w.M // 2, w.M - 1):
+        compare(out[m].cpu().numpy()[seqs][:, heads], ow.expected_decode(w, 1, m, seqs, heads, orc.POLICY_PAPER), f"layer {m}")
+    assert run.cache.device_status() == 0
