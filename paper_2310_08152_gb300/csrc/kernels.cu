@@ -1543,6 +1543,16 @@ cudaError_t launch_decode_cta(const Geometry& g, const Static& st, const Buffers
   return cudaLaunchKernelEx(&cfg, decode_cta_kernel<T, D, W, KPT, S>, g, st, p, CN, (int)k_segs);
 }
 
+// k whole segments per warp, k as small as one wave of `occ` warps per SM allows; `busiest`: the segments on the
+// SM with the most.
+struct SegSplit {
+  int64_t k, workers, busiest;
+};
+inline SegSplit seg_split(int64_t nseg, int occ, int num_sms) {
+  const int64_t slots = (int64_t)occ * num_sms, k = (nseg + slots - 1) / slots, workers = (nseg + k - 1) / k;
+  return {k, workers, (workers + num_sms - 1) / num_sms * k};
+}
+
 // Segments of the uploaded state are balanced: the longest holds at most 1.3x the mean rows.
 inline bool decode_balanced(const DecodeArgs& a) {
   return a.n_segments > 0 && 10 * a.max_segment * a.n_segments <= 13 * a.R;
@@ -1556,14 +1566,15 @@ struct CtaMainStages {
 
 // Whether and how the CTA kernel takes a launch of nseg segments: `cluster` CTAs per segment, or k
 // segments per CTA, of the main or the small shape.  slots_m / slots_s: CTAs of the main / small shape
-// that one wave holds.
+// that one wave holds, slots_w: warps of the wide shape.
 struct CtaPlan {
   bool use, small;
   int cluster;
   int64_t k;
 };
 template <int D>
-CtaPlan decode_cta_plan(const DecodeArgs& a, int64_t nseg, bool balanced, int64_t slots_m, int64_t slots_s) {
+CtaPlan decode_cta_plan(const DecodeArgs& a, int64_t nseg, bool balanced, int64_t slots_m, int64_t slots_s,
+                        int64_t slots_w) {
   constexpr CtaPlan kNo = {false, false, 1, 1};
   const int n_layers = a.n_layers < 1 ? 1 : a.n_layers;
   const int64_t mean = a.R / (a.n_segments < 1 ? 1 : a.n_segments);  // rows of a segment that has any
@@ -1582,24 +1593,34 @@ CtaPlan decode_cta_plan(const DecodeArgs& a, int64_t nseg, bool balanced, int64_
     if (!balanced && a.max_segment > 2 * cn * share + 2048) return kNo;
     return {true, false, cn, 1};
   }
-  // More than one wave.  A tile's and a segment's fixed work have to be small beside a segment's rows:
-  // a warp per segment, or several, is as good below these means and up to 40 % better at half of them
-  // (d_head 64, 65,536 segments: 243 rows 19.2 us a layer by warps, 20.3 here; 485 rows 20.6 and 19.0;
-  // 992 rows 71.9 and 69.2.  d_head 128: 170 rows 30.8 and 30.2).
-  constexpr int64_t kMeanRows = Lanes<D>::LPR == 4 ? 160 : 384;
+  // More than one wave.  A tile's and a segment's fixed work have to be small beside a segment's rows, and the last
+  // tile of a segment full: below some mean a warp per segment, or several, is better, and twice as good at a
+  // quarter of it.
+  constexpr bool kLpr4 = Lanes<D>::LPR == 4;  // 96 and 128 columns: 64 rows a tile, else 128
   if (balanced) {
     if (nseg <= slots_s) return {true, true, 1, 1};
-    if (mean < kMeanRows) return kNo;
-    // up to eight segments per CTA where that makes one wave: 768 segments of 992 rows 30.0 us against
-    // 33.3 one by one, 2,048 75.2 against 77.1
+    // Up to eight segments per CTA where that makes one wave (768 segments of 992 rows 30.0 us against 33.3 one
+    // by one, 2,048 75.2 against 77.1), a CTA each beyond.  Where the line lies, as time here over time by warps:
+    //   a CTA each, 4,096 segments a layer, six layers in one launch: d_head 64 375 rows 1.02, 430 1.02, 460 0.98,
+    //     500 0.96; 80 375 1.03, 430 1.02, 460 0.96; 96 192 rows 1.11, 288 1.02, 320 0.97; 128 1.10, 1.01, 0.98
+    //   one wave, a launch per layer, 640 to 2,432 segments: 64 375 rows 0.77-0.99, 80 0.81-1.07; 96 192 rows
+    //     0.81-1.09, but up to a wave of wide warps, 912, 1.12 and 1.01 of those, at 350 rows 1.06 and 0.97;
+    //     128 160 rows 0.86-1.14, 192 0.78-1.05
+    // (At 128 columns the line of one wave reaches one segment per CTA further: 2,560 of 170 rows 42.8 us here,
+    // 38.7 by warps.)
     const int64_t k = (nseg + slots_m - 1) / slots_m;
+    const bool one_wave = k <= (D == 128 ? 9 : 8);
+    const int64_t line = !one_wave ? (kLpr4 ? 320 : 448) : !kLpr4 ? 384 : D == 128 ? 160 : nseg <= slots_w ? 384 : 192;
+    if (mean < line) return kNo;
     return {true, false, 1, k <= 8 ? k : 1};
   }
   if (a.max_segment > 6 * mean || a.max_segment > 2 * share + 2048) return kNo;  // as above: split the rows
   // Unbalanced: the hardware hands the CTAs out as they finish, where a split of the rows over every warp
   // pays for its partial results (6 layers of 8,192 segments: mean 210 rows 73.1 us a layer, split 109.5;
   // 80 rows 42.7 and 69.0).  Short segments two to a CTA, of the small shape at d_head 64.
-  if (mean >= kMeanRows) return {true, false, 1, 1};
+  // (64 columns, 2,048 segments a layer of 330 rows 25.7 and 29.9 with a CTA of the main shape for each; 96 of
+  // 200 25.5 and 29.3, of 243 30.0 and 32.7; 128 of 180 29.0 and 33.3, of 243 41.1 and 40.3)
+  if (mean >= (kLpr4 ? 256 : 384)) return {true, false, 1, 1};
   return {true, D == 64, 1, mean < 256 ? 2 : 1};
 }
 
@@ -1656,8 +1677,11 @@ cudaError_t launch_decode_t(const Geometry& g, const Static& st, const Buffers& 
   DecodeOcc occ;
   const cudaError_t e = decode_occupancies<T, D>(a.device, &occ);
   if (e != cudaSuccess) return e;
-  const CtaPlan c = decode_cta_plan<D>(a, nseg, balanced, (int64_t)occ.main * num_sms, (int64_t)occ.small * num_sms);
+  const CtaPlan c = decode_cta_plan<D>(a, nseg, balanced, (int64_t)occ.main * num_sms, (int64_t)occ.small * num_sms,
+                                       (int64_t)occ.wide * num_sms);
   const bool by_cta = c.use && !c.small && c.k == 1;
+  const int64_t wide_tile = AK * Lanes<D>::RPI;
+  const bool wide = a.R >= 6 * wide_tile * a.n_segments && (D <= 80 || a.R <= 24 * wide_tile * a.n_segments);
   if (n_layers > 1 && !balanced && !by_cta && nseg > (int64_t)occ.main * num_sms) {
     // Unbalanced segments over several layers, short ones or with a few far longer: a wave of warps takes
     // whole segments cut by rows when the longest segment is at most 1/16 of a warp's even share (so no
@@ -1667,8 +1691,6 @@ cudaError_t launch_decode_t(const Geometry& g, const Static& st, const Buffers& 
     // launch per layer.  At d_head 96 and 128, whose wide tiles are 32 rows, up to 768 rows: two of 3,600
     // among 192 of 300 rows, bf16 d_head 128, 3,716 and 3,927, but one of 8,000 among 96 of 1,000, 5,987
     // and 5,942.
-    const int64_t wide_tile = AK * Lanes<D>::RPI;
-    const bool wide = a.R >= 6 * wide_tile * a.n_segments && (D <= 80 || a.R <= 24 * wide_tile * a.n_segments);
     int64_t NW = (int64_t)(wide ? occ.wide : occ.seg) * num_sms;
     if (NW > nseg) NW = nseg;
     if (NW >= 1 && 16 * a.max_segment <= (int64_t)n_layers * a.R / NW) {
@@ -1683,15 +1705,24 @@ cudaError_t launch_decode_t(const Geometry& g, const Static& st, const Buffers& 
     return launch_decode_cta<T, D, 4, 2, MS>(g, st, buf, a, c.cluster, c.k, mode, stream, grid, plan);
   }
   if (balanced) {
+    if (nseg <= (int64_t)occ.wide * num_sms) {  // d_head 96: 768 segments of 160 rows 9.1 us, 11.1 narrow
+      *plan = {2, (int)nseg, AK * Lanes<D>::RPI, AS};
+      return launch_decode_cfg<T, D, AK, AS>(g, st, buf, a, nseg, 1, stream, grid);
+    }
     if (nseg <= (int64_t)occ.seg * num_sms) {
       *plan = {2, (int)nseg, BK * Lanes<D>::RPI, BS};
       return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, nseg, 1, stream, grid);
     }
-    // k whole segments per warp, k as small as one wave of warps allows
-    const int64_t slots = (int64_t)occ.seg * num_sms;
-    const int64_t k = (nseg + slots - 1) / slots, workers = (nseg + k - 1) / k;
-    *plan = {3, (int)workers, BK * Lanes<D>::RPI, BS};
-    return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, workers, k, stream, grid);
+    // k whole segments per warp, k as small as one wave of warps allows; in the wide shape from six wide
+    // tiles up, unless the narrow one leaves fewer segments to the SM with the most (d_head 128, 65,536
+    // segments of 192 rows 918 and 982 us, of 220 1,054 and 1,125)
+    const SegSplit sa = seg_split(nseg, occ.wide, num_sms), sb = seg_split(nseg, occ.seg, num_sms);
+    if (wide && sa.busiest <= sb.busiest) {
+      *plan = {3, (int)sa.workers, AK * Lanes<D>::RPI, AS};
+      return launch_decode_cfg<T, D, AK, AS>(g, st, buf, a, sa.workers, sa.k, stream, grid);
+    }
+    *plan = {3, (int)sb.workers, BK * Lanes<D>::RPI, BS};
+    return launch_decode_cfg<T, D, BK, BS>(g, st, buf, a, sb.workers, sb.k, stream, grid);
   }
   if (n_layers > 1) return cudaErrorNotSupported;  // the caller launches the layers one by one
   int64_t NW = (int64_t)occ.stream * num_sms;

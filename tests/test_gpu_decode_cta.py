@@ -122,3 +122,20 @@ def test_a_few_long_sequences_over_layers(name, make, mode, tile):
     for m in (0, w.M // 2, w.M - 1):
         compare(out[m].cpu().numpy()[seqs][:, heads], ow.expected_decode(w, 1, m, seqs, heads, orc.POLICY_PAPER), f"layer {m}")
     assert run.cache.device_status() == 0
+
+
+# balanced segments too short for a CTA each: mode (2: one warp a segment, 3: several), rows per tile
+SHORT = [
+    ("d 80, several a warp", lambda: _with(wl.opt13b_uncompressed(b=40, L=400, M=2), d=80), 3, 32),
+    ("d 96, one wide warp each", lambda: _with(wl.opt13b_uncompressed(b=22, L=250, M=1), d=96), 2, 32),
+    ("d 96, several a wide warp", lambda: _with(wl.opt13b_uncompressed(b=40, L=250, M=2), d=96, dtype="bf16"), 3, 32),
+    ("d 96, several a narrow warp", lambda: _with(wl.opt13b_uncompressed(b=40, L=170, M=2), d=96), 3, 16),
+    ("d 128, several a wide warp", lambda: _with(wl.opt13b_uncompressed(b=43, L=250, M=2), d=128), 3, 32),
+]
+
+
+@pytest.mark.parametrize("name,make,mode,tile", SHORT, ids=[c[0] for c in SHORT])
+def test_whole_segments_per_warp(name, make, mode, tile):
+    run, _ = run_workload(make(), steps=2, seqs=[0, 7, 21], heads=[0, 13, 31])
+    plan = run.cache.last_decode_plan
+    assert plan["mode"] == mode and plan["tile_rows"] == tile, plan
