@@ -1614,8 +1614,11 @@ CtaPlan decode_cta_plan(const DecodeArgs& a, int64_t nseg, bool balanced, int64_
     if (mean < line) return kNo;
     return {true, false, 1, k <= 8 ? k : 1};
   }
-  if (a.max_segment > 6 * mean || a.max_segment > 2 * share + 2048) return kNo;  // as above: split the rows
-  // Unbalanced: the hardware hands the CTAs out as they finish, where a split of the rows over every warp
+  // Unbalanced, as above: split the rows when the longest segment, which may come last, is past 1.25 shares and
+  // 1,024 rows (9 sequences of 40 heads, the longest 1.8 shares of 15,500 rows, two layers of 128 columns: 360 us
+  // split, 469 here; 25, 1.75 of 3,900, 24 layers of 96: 1,906 and 2,244; 28, 1.4 of 3,500, 128: 89.3 and 87.6).
+  if (a.max_segment > 6 * mean || 4 * a.max_segment > 5 * share + 4096) return kNo;
+  // Else the hardware hands the CTAs out as they finish, where a split of the rows over every warp
   // pays for its partial results (6 layers of 8,192 segments: mean 210 rows 73.1 us a layer, split 109.5;
   // 80 rows 42.7 and 69.0).  Short segments two to a CTA, of the small shape at d_head 64.
   // (64 columns, 2,048 segments a layer of 330 rows 25.7 and 29.9 with a CTA of the main shape for each; 96 of

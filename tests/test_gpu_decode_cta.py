@@ -100,6 +100,8 @@ FEW_LONG = [
     ("d 128 bf16, wide", lambda: _few_long(128, "bf16", 120, 250, 1, 8, 24), 4, 32),
     ("d 64, narrow", lambda: _few_long(64, "f16", 220, 200, 1, 8, 24), 4, 32),
     ("d 64, too long a sequence", lambda: _few_long(64, "f16", 60, 300, 1, 12, 24), 0, 32),
+    ("d 64, longer than a CTA's share", lambda: _few_long(64, "f16", 18, 1500, 1, 4, 1), 0, 32),
+    ("d 64, within a CTA's share of two layers", lambda: _few_long(64, "f16", 18, 1500, 1, 4, 2), 4, 128),
 ]
 
 
