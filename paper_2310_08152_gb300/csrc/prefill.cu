@@ -969,9 +969,7 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
     auto epilogue = [&](uint32_t kk, float l_) {
       const PfItem& w = item_slot[kk % kItemRing];
       const uint32_t o_t = tl + Cf::O_COL + (Cf::OBUF == 2 ? (kk & 1) * D : 0);
-      float inv;  // 1 / l_: the approximation and a Newton step
-      asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(l_));
-      inv = __fmaf_rn(inv, __fmaf_rn(-l_, inv, 1.f), inv);
+      const float inv = 1.f / l_;
       const int64_t row8 = (int64_t)8 * a.H * D;
       float* o_row = a.out + ((int64_t)(w.tok0 + warp * 32 + (lane >> 2)) * a.H + w.h) * D + 2 * (lane & 3);
       const int left = w.qr_end - w.qr0 - (warp * 32 + (lane >> 2));  // queries from this lane's first row on
