@@ -75,11 +75,39 @@ def test_ring_that_wraps_over_a_cluster():
 
 
 def test_open_span_hidden_row_in_every_part():
-    """A span opened at the step before: its <CL> row, hidden, lies in the last CTA's rows of a cluster
-    at first and moves into an earlier one as the span grows; both policies."""
+    """A span opened while generating: its <CL> row, hidden under the paper policy, among the last rows of a
+    cluster's last CTA."""
     for policy in (orc.POLICY_PAPER, orc.POLICY_KEEP_CL):
         w = wl.opt13b(b=2, L=1600, M=1)
         run_workload(w, steps=4, policy=policy)
+
+
+# (hidden from the query at row 1600 by an open <CL> or by a closed span not freed yet, which of the two sequences)
+# A cluster of 4 takes rows 0-400, 401-801, 802-1202 and 1203-1600 of 1,601.
+HIDDEN = [[("open", 400), ("open", 401)], [("open", 801), ("open", 802)], [("open", 1202), ("open", 1203)],
+          [("open", 0), ("open", 1599)], [("span", 390, 420), ("span", 0, 401)], [("span", 300, 1500), ("span", 401, 802)],
+          [("span", 1202, 1599), ("span", 1201, 1204)]]
+
+
+@pytest.mark.parametrize("policy", [orc.POLICY_PAPER, orc.POLICY_KEEP_CL])
+@pytest.mark.parametrize("hidden", HIDDEN, ids=str)
+def test_hidden_rows_at_the_ctas_of_a_cluster(hidden, policy):
+    """Hidden rows at every CTA's first and last row, across two CTAs' rows, and all rows of one or two CTAs."""
+    kinds = [np.zeros(1600, np.uint8) for _ in hidden]
+    for k, (what, *at) in zip(kinds, hidden):
+        k[at[0]] = wl.CL
+        if what == "span":
+            k[at[1]] = wl.CR
+    w = dataclasses.replace(wl.opt13b(b=2, L=64, M=1), prompt_kinds=kinds, prompt_spans=[[], []], gen_kind=lambda s, g: 0)
+    run = harness.Runner(w, 1, policy)
+    run.load_prompt()
+    inp = run.make_step_inputs(0)
+    run.append_only(inp)
+    out = run.cache.decode_attention(0, inp.q[0], w.scale)
+    plan = run.cache.last_decode_plan
+    assert plan["workers"] == 64 * 4 * 4, plan
+    compare(out.cpu().numpy(), ow.expected_decode(w, 1, 0, [0, 1], None, policy), str(hidden))
+    assert run.cache.device_status() == 0
 
 
 def _few_long(d, dtype, b, short, n_long, factor, M):
