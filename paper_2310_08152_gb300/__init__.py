@@ -397,10 +397,11 @@ class KVCache:
         cfg.workspace, cfg.workspace_bytes = self.workspace.data_ptr(), sizes["workspace"]
         self._cfg = cfg
         self.handle = kvc_create(cfg)
-        # the upload ring, from torch's pool of pinned memory (allocating and freeing it with each cache takes
-        # about 300 us); kvc_destroy waits for the device before the pool gets it back.  Above 4 MB (some 50,000
-        # rows) the library allocates it: the pool rounds up to powers of two, and pinning the rest costs as much
-        # (300 us more at 16 MB) while a cache of that size is rarely made anew.
+        # the upload ring, from torch's pool of pinned memory (1 us once the pool has it, where allocating and freeing
+        # it with each cache takes 200 to 280); kvc_destroy waits for the device before the pool gets it back.  Above
+        # 4 MB (some 50,000 rows) the library allocates it: the pool rounds up to powers of two, so the first cache
+        # of a size pays more (4.3 MB: 396 us against 289, 9 MB 746 against 547, 16.5 MB 1573 against 958), and a
+        # cache of that size is rarely made anew.
         # A capture on another stream goes on (relaxed mode); within one the library allocates it, as the first
         # append comes.
         self.staging = None

@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(kAppendThreads) append_kernel(Geometry g, Stat
 
 // The same for a few tokens whose upload (decode state and plan) comes as a kernel parameter: no copy, event and
 // staging memory for it, which bound such calls.  Block 0 stores it in the workspace, where the calls after this one
-// read it.  A call for a token of each of four sequences in four layers: 10.1 us with the upload, 6.8 without; 40
-// generated tokens with their decodes 3825 -> 3517.  The line is the size of a kernel's parameters (4 KB).
+// read it.  A call for a token of each of four sequences in four layers: 10.1 us with the upload, 6.8 without.  The
+// line is the size of a kernel's parameters (4 KB).
 template <typename T, int D>
 __global__ void __launch_bounds__(kAppendThreads)
     append_image_kernel(Geometry g, Static st, Buffers buf, const __grid_constant__ AppendImage img, int img_bytes,

@@ -150,8 +150,8 @@ struct PfItemRec {
 struct PrefillArgs {
   int layer, H, rot;
   int64_t C;
-  const PfItemRec* items;  // [n_items]
-  const PfTileRec* tiles;  // [n_items]: sequences with the most stored rows first, then head, then the query tile with the most keys first
+  const PfItemRec* items;  // [n_items]: sequences with the most stored rows first, then head, then the query tile with the most keys first
+  const PfTileRec* tiles;  // [n_items / H]: in the same order, without the heads
   int64_t n_items;         // (query tile, head) work items
   unsigned long long* item_counter;  // [2], zero at launch and after it: the next item, the CTAs that are through
   int n_ctas;              // persistent grid size

@@ -483,9 +483,8 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
   __shared__ uint32_t tmem_slot;
 
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~uintptr_t(1023));
-  // The warp's number and the TMEM base through a shuffle, which the compiler knows to be the warp's: TMEM addresses,
-  // barriers and branches are uniform then, without moves and reconvergence around each (OPT-1.3B-shaped prompts
-  // 264 us a layer, 253 so; ragged rotary prompts 850 -> 753; heads of 96 430 -> 390, of 128 466 -> 426).
+  // The warp's number and the TMEM base through a shuffle, which the compiler knows to be the warp's (OPT-1.3B-shaped
+  // prompts 264 us a layer, 253 so; ragged rotary prompts 850 -> 753; heads of 96 430 -> 390, of 128 466 -> 426).
   const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
 
   if (warp == 0) {
@@ -734,11 +733,10 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
   } else if (warp == 5) {
     regs_other();
     // ---------------- MMA issuer ----------------
-    // The whole warp runs this role, and one lane of it issues: with the loop in one lane's branch the operands of
-    // every tcgen05.mma went from the general to the uniform registers, 8 moves and about 100 cycles each, which
-    // bounded the kernel with 13 of them a tile (compacted bf16 prompts 387 us a layer, 323 so; bf16 heads of 64
-    // 384 -> 342; heads of 128 491 -> 466; OPT-1.3B-shaped prompts 272 -> 264).  Conditions are votes, so that the
-    // compiler knows them to be the warp's.
+    // The whole warp runs this role, and one lane of it issues (with the loop in one lane's branch compacted bf16
+    // prompts, 13 products a tile, took 387 us a layer, 323 so; bf16 heads of 64 384 -> 342; heads of 128
+    // 491 -> 466; OPT-1.3B-shaped prompts 272 -> 264).  Conditions are votes, so that the compiler knows them to be
+    // the warp's.
     {
       constexpr uint32_t idS = mma_idesc(Pack16<T>::kType, 0, kPfRows, KT);
       constexpr uint32_t idO = mma_idesc(Pack16<T>::kType, 1, kPfRows, D);
@@ -884,7 +882,8 @@ __global__ void __launch_bounds__(kPfThreads, PfCfg<D>::CPS)
       const int half = a.rot / 2;
       const int iq = w.qr0 + r;
       if constexpr (Cf::SPLIT) {
-        // every row (rows past the tile's queries hold zeros), so the TMEM stores are warp-wide
+        // every row, so the TMEM stores are warp-wide (past the tile's queries another sequence's, or zeros: their
+        // results go nowhere)
         {
           const float fpos = iq < w.qr_end ? (float)a.pos[a.off[w.s] + iq] : 0.f;
           const int hc = half / 8;  // chunks per rotated half
