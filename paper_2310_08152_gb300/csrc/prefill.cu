@@ -293,12 +293,14 @@ __device__ __forceinline__ uint32_t bf16_split2(float2 x, uint32_t* hi) {
 }
 
 // rope_sincos (device_common.cuh) of two frequencies (hi, hi, lo, lo) at position p, with packed instructions and the
-// same roundings: sines, their negatives, cosines.  (Ragged rotary prompts 746 us a layer with rope_sincos, 735 so.)
+// same roundings: sines, their negatives, cosines.  (Ragged rotary prompts 747 us a layer with rope_sincos, 740 so.)
+// The turns' whole part comes off with scalar subtractions: a packed sum of a packed product is fused with it by the
+// compiler, its explicit rounding notwithstanding, and loses the product's rounding error that e holds.
 __device__ __forceinline__ void rope_sincos2(float p, float4 g, float2* s, float2* ns, float2* c) {
   const float2 p2 = make_float2(p, p), gh = make_float2(g.x, g.y);
-  const float2 a = __fmul2_rn(p2, gh), na = __fmul2_rn(make_float2(-p, -p), gh);
-  const float2 e = __ffma2_rn(p2, gh, na);
-  const float2 turn = __fadd2_rn(a, make_float2(rintf(na.x), rintf(na.y)));
+  const float2 a = __fmul2_rn(p2, gh);
+  const float2 e = __ffma2_rn(p2, gh, make_float2(-a.x, -a.y));
+  const float2 turn = make_float2(__fsub_rn(a.x, rintf(a.x)), __fsub_rn(a.y, rintf(a.y)));
   const float2 f = __fadd2_rn(turn, __ffma2_rn(p2, make_float2(g.z, g.w), e));
   const float2 t = __fmul2_rn(make_float2(6.28318530717958647692f, 6.28318530717958647692f), f);
   __sincosf(t.x, &s->x, &c->x);
