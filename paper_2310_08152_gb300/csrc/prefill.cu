@@ -30,8 +30,8 @@
 // taken out paid more than its instructions' issue slots.  So waits are one short loop, the epilogue and the
 // masking exist once, and nothing but the softmax is unrolled far.  Time of a layer, against a kernel that read
 // every stored row with masks over all of them: OPT-1.3B-shaped prompts (16 x 2048 tokens, 32 heads of 64,
-// interiors of 32) 541 -> 248 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 733 us; the
-// last 512 of 32 x 4096 tokens, compacted before them, bf16 (heads of 80) 664 -> 328 us; the first with 96 and
+// interiors of 32) 541 -> 250 us; 24 ragged rotary prompts (256 to 4096 tokens, heads of 80) 1587 -> 738 us; the
+// last 512 of 32 x 4096 tokens, compacted before them, bf16 (heads of 80) 664 -> 327 us; the first with 96 and
 // 128 columns 797 -> 385 and 1042 -> 421 us; one prompt of 300 tokens 13.2 -> 10.8 us.  (Copying the listed rows
 // side by side first, for TMA tiles alone, took a second kernel and 381, 992 and 454 us on the first three when
 // the gathers took 372, 1026 and 450.)
