@@ -212,7 +212,7 @@ def test_launch_counter_counts_kernels():
 
 def _mode_workloads():
     sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 152
-    b_narrow = (5 * sms + 31) // 32  # more segments than one wave of the wide pipeline holds (3 warps/SM at d=64)
+    b_narrow = (5 * sms + 31) // 32  # more segments than one wave of CTAs holds (2 of the main, 4 of the small shape per SM)
     # more segments than one wave of the narrow pipeline holds (8 warps/SM at d=64), and a count that
     # k does not divide, so the last worker takes fewer segments
     b_multi = (10 * sms + 31) // 32 + 1
@@ -232,8 +232,10 @@ def _mode_workloads():
 
 @pytest.mark.parametrize("name,w,mode", _mode_workloads(), ids=lambda x: x if isinstance(x, str) else "")
 def test_every_scheduling_mode(name, w, mode):
-    # each way of dividing the decode work (one warp per segment, wide or narrow pipeline; several
-    # whole segments per warp; stream-K with split segments) must agree with the oracle
+    # each way of dividing the decode work must agree with the oracle: a CTA or a cluster for each of a layer's
+    # balanced segments ("wide") or of its unbalanced ones ("stream-k" and "ragged stream-k", whose longest the
+    # CTAs take; rows split over all warps are in test_gpu_decode_split.py), one warp per segment, several
+    # whole segments per warp
     run, _ = run_workload(w, steps=2, check_steps={0, 1}, seqs=None)
     plan = run.cache.last_decode_plan
     assert plan["mode"] == mode, plan
@@ -391,7 +393,7 @@ def test_fused_layers_several_segments_per_warp_with_empty_sequences(b):
 
 
 def test_fused_layers_fall_back_to_per_layer_launches_when_unbalanced():
-    """Unbalanced segments are split over a wave of warps (stream-K) one layer per launch: the
+    """Unbalanced segments fewer than a wave of CTAs go one layer per launch, each cut over a cluster: the
     multi-layer call makes M launches and matches the per-layer calls bit for bit."""
     w = dataclasses.replace(wl.opt13b(b=2, L=64, M=3), name="long-short")
     k_long, s_long = wl.block_kinds(3000, 32)
@@ -422,7 +424,7 @@ def test_fused_layers_fall_back_to_per_layer_launches_when_unbalanced():
 def test_fused_layers_whole_segments_cut_by_rows():
     """Unbalanced (ragged) segments over many layers, each short beside a warp's even share of all the
     layers' rows: one launch in which every warp takes a run of whole segments cut by rows (no split,
-    no combine).  Against the per-layer stream-K launches, which split segments and combine them, and
+    no combine).  Against the per-layer launches, which take a CTA for two segments, and
     against the oracle on the first, a middle and the last layer."""
     w = wl.ragged(b=64, lmin=64, lmax=700, M=24, steps=2)
     run = harness.Runner(w, 2)

@@ -23,7 +23,7 @@ pytestmark = pytest.mark.gpu
 
 
 def _workloads():
-    # one (sequence, head) per warp, and a stream-K split with partials combined through the scratch
+    # a CTA or a cluster per (sequence, head); parts combined through the scratch are in test_gpu_decode_split.py
     long_short = dataclasses.replace(wl.opt13b(b=2, L=64, M=2), name="long-short")
     k_long, s_long = wl.block_kinds(9000, 32)
     k_short, s_short = wl.block_kinds(70, 8)
