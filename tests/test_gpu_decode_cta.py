@@ -164,6 +164,32 @@ SHORT = [
 ]
 
 
+@pytest.mark.parametrize("d,dtype,rot,b,L,M,mode", [(96, "f16", 32, 40, 500, 2, 3), (128, "bf16", 64, 43, 470, 2, 3), (96, "bf16", 96, 22, 500, 1, 2)])
+@pytest.mark.parametrize("policy", [orc.POLICY_PAPER, orc.POLICY_KEEP_CL])
+def test_whole_segments_per_wide_warp_with_an_open_span(d, dtype, rot, b, L, M, mode, policy):
+    """Compacted prompts, rotary positions, and a span opened while generating, whose <CL> row the paper policy hides."""
+    run, _ = run_workload(_with(wl.opt13b(b=b, L=L, M=M), d=d, dtype=dtype, rotary_dim=rot), steps=3, policy=policy,
+                          seqs=[0, b // 2, b - 1], heads=[0, 31])
+    plan = run.cache.last_decode_plan
+    assert plan["mode"] == mode and plan["tile_rows"] == 32, plan
+
+
+def test_whole_segments_per_wide_warp_of_rings():
+    """Windows of 250 rows, the ring's end at another row in each step."""
+    w = _with(wl.opt13b_local(b=40, L=500, M=2), d=96)
+    run = harness.Runner(w, steps=4, capacity_slack=9)
+    run.load_prompt()
+    out = torch.empty(w.M, w.b, w.H, w.d, dtype=torch.float32, device="cuda")
+    for g in range(4):
+        run.step(run.make_step_inputs(g), out)
+        torch.cuda.synchronize()
+        assert run.cache.last_decode_plan["mode"] == 3 and run.cache.last_decode_plan["tile_rows"] == 32
+        for m in range(w.M):
+            ref = ow.expected_local_decode(w, g + 1, m, [0, 20, 39], float(np.float32(0.5)), [0, 31])
+            compare(out[m].cpu().numpy()[[0, 20, 39]][:, [0, 31]], ref, f"step {g} layer {m}")
+    assert run.cache.device_status() == 0
+
+
 @pytest.mark.parametrize("name,make,mode,tile", SHORT, ids=[c[0] for c in SHORT])
 def test_whole_segments_per_warp(name, make, mode, tile):
     run, _ = run_workload(make(), steps=2, seqs=[0, 7, 21], heads=[0, 13, 31])
