@@ -153,11 +153,16 @@ class PinnedRing {
     if (borrowed_ && base_) {
       int dev = -1;
       if (cudaGetDevice(&dev) == cudaSuccess && dev != device_) cudaSetDevice(device_);
-      for (auto& p : pending_) cudaEventSynchronize(p.ev);
+      bool failed = false;  // the event of a captured upload: the graph's to order
+      for (auto& p : pending_) failed |= cudaEventSynchronize(p.ev) != cudaSuccess;
       static std::atomic<bool> kept[64];
       void* block = nullptr;
-      if (device_ >= 0 && device_ < 64 && !kept[device_].exchange(true)) (void)cudaMalloc(&block, 256);
-      if (cudaMalloc(&block, 256) != cudaSuccess || cudaFree(block) != cudaSuccess) cudaDeviceSynchronize();
+      if (device_ >= 0 && device_ < 64 && !kept[device_].exchange(true)) failed |= cudaMalloc(&block, 256) != cudaSuccess;
+      if (cudaMalloc(&block, 256) != cudaSuccess || cudaFree(block) != cudaSuccess) {
+        failed = true;
+        cudaDeviceSynchronize();
+      }
+      if (failed) (void)cudaGetLastError();  // none of the caller's calls
       if (dev >= 0 && dev != device_) cudaSetDevice(dev);
       base_ = nullptr;
     }

@@ -135,3 +135,23 @@ def test_cache_that_is_made_while_a_stream_captures(mode, beside):
         assert (out[0].double() - torch.einsum("hn,nhd->hd", p, v[0].double())).abs().max().item() < 3e-4
         assert c.device_status() == 0
     assert x.tolist() == [3.0] * 4
+
+
+@pytest.mark.gpu
+def test_cache_that_ends_after_its_append_was_captured():
+    """The event of a captured upload cannot be waited for; no error of that is left for the calls that follow."""
+    c = kvc.KVCache(1, 4, 64, [900])
+    k, v = _tokens(1, 4, 64, 300, 5)
+    kinds = np.zeros(300, np.uint8)
+    c.append(k, v, [300], kinds)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        c.append(k, v, [300], kinds)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(c.stream_rows(c.v_plane(0), 0, 0, 600)[300:], v[0, :, 0])
+    c.close()
+    assert torch.ones(8, device="cuda").sum().item() == 8.0
+    d = kvc.KVCache(1, 4, 64, [900])
+    d.append(k, v, [300], kinds)
+    assert d.device_status() == 0
